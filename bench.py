@@ -475,7 +475,7 @@ def main():
         dom_launches = st["dom_launches"]
     achieved_tf = dom_flops_per / (dom_ms_per * 1e-3) / 1e12 if dom_ms_per > 0 else None
     if prec == B.MBE_FP64:
-        kname = "k_contract_fp64"
+        kname = "k_sigma_direct"
         peak_tf = fp_peaks["fp64_tflops"]
         peak_src = "FP64 FMA, measured by mbe_measure_peaks on this GPU"
         bound = "alu"

@@ -197,13 +197,16 @@ void solve_jobs(mbe_ctx* ctx, const std::vector<std::vector<int>>& acts, double*
     // the full FP32 exact-point operand, two full FP64 exact-point vectors,
     // the FP32 W rows of the sigma, the bf16 hi/lo copies of the sigma
     // operand and of H^alpha and the P-space eigenvectors; the FP64 one
-    // 2M + 6 FP64 vectors
+    // 2M + 6 FP64 vectors and the one-spin tables of its sigma
     // the mixed path works on alpha<->beta symmetric vectors: closed shells
     const bool mixed_bin = ctx->opt.precision == MBE_MIXED_BF16X3 && N > 1 && closed &&
                            sigma_tc_supported(n, tab->nstr) && ozaki_supported(tab->npair);
     const int Mm = mixed_subspace_alloc(ctx->opt.max_subspace);
     double per = (mixed_bin ? (double)(4 * Mm + 46) * N + 128.0 * 129.0 * 4.0
-                            : (double)(2 * M + 6) * N * 8.0) +
+                            : (double)(2 * M + 6) * N * 8.0 +
+                                  8.0 * (direct_nnz(n, nsig) * (double)tab->nstr +
+                                         (direct_nnz(n, nsigb) + tabb->npair) *
+                                             (double)tabb->nstr)) +
                  (double)tab->npair * tab->npair * 8.0 * 2.0;
     int64_t bmem = std::max<int64_t>(1, (int64_t)(budget / per));
     int64_t bmax = std::min<int64_t>(std::max(1, ctx->opt.max_batch), bmem);
@@ -911,7 +914,12 @@ int mbe_sigma(mbe_ctx* ctx, const int* act, int nact, const double* c, double* s
         if (sigma_tc_error(ctx, w)) return fail(ctx, MBE_ETIMEOUT, "fused exact sigma wait timed out");
       } else {
         const bool emu = ctx->opt.precision == MBE_EMULATED_FP64 && ozaki_supported(bp.npair);
-        sigma_fp64(ctx, bp, w, cd.ptr, bp.ndet, sd.ptr, bp.ndet, nullptr, ctx->opt.spin_shift, emu);
+        if (emu)
+          sigma_emulated(ctx, bp, w, cd.ptr, bp.ndet, sd.ptr, bp.ndet, nullptr,
+                         ctx->opt.spin_shift);
+        else
+          sigma_direct(ctx, bp, cd.ptr, bp.ndet, sd.ptr, bp.ndet, nullptr, ctx->opt.spin_shift,
+                       false);
         if (emu && sigma_tc_error(ctx, w))
           return fail(ctx, MBE_ETIMEOUT, "tensor-core contraction wait timed out");
       }

@@ -3,8 +3,9 @@
 //   K1  string enumeration and the per-(string, orbital pair) link table
 //   K2  effective integrals of each tuple (inactive-core fold, Sec. 2/Fig. 2)
 //   K3  diagonal of H_active + shift * S^2 (Davidson preconditioner)
-//   K4  FP64 string-driven sigma vector: gather D, (kl|ij) contraction, pull
-//       scatter, plus the S^2 spin shift
+//   K4  gather and pull scatter of the emulated-FP64 sigma vector (its (kl|ij)
+//       contraction is in mbe_ozaki.cu; the FP64 sigma is in mbe_sigma64.cu),
+//       plus the S^2 spin shift
 //
 // Sigma vector (Knowles & Handy, Chem. Phys. Lett. 111, 315 (1984); Olsen
 // et al., J. Chem. Phys. 89, 2185 (1988)): with h'_pq = h_pq - 1/2 sum_r
@@ -103,13 +104,9 @@ int64_t string_count(int n, int nsig) {
   return nstr;
 }
 
-void launch_string_tables(mbe_ctx* ctx, int n, int nsig, int nstr, uint32_t* masks,
-                          int32_t* link) {
+void launch_string_masks(mbe_ctx* ctx, int n, int nsig, int nstr, uint32_t* masks) {
   ensure_binom(ctx->device);
   k_strings<<<(nstr + 255) / 256, 256, 0, ctx->stream>>>(masks, nstr, n, nsig);
-  CU_LAUNCH_CHECK();
-  const int64_t tot = (int64_t)nstr * (n * (n + 1) / 2);
-  k_link<<<(unsigned)((tot + 255) / 256), 256, 0, ctx->stream>>>(masks, link, nstr, n);
   CU_LAUNCH_CHECK();
 }
 
@@ -120,7 +117,11 @@ void build_string_tables(mbe_ctx* ctx, StringTables* t) {
   t->npair = t->n * (t->n + 1) / 2;
   t->masks.reset(&ctx->pool, t->nstr);
   t->link.reset(&ctx->pool, (size_t)t->nstr * t->npair);
-  launch_string_tables(ctx, t->n, t->nsig, t->nstr, t->masks.ptr, t->link.ptr);
+  launch_string_masks(ctx, t->n, t->nsig, t->nstr, t->masks.ptr);
+  const int64_t tot = nstr * t->npair;
+  k_link<<<(unsigned)((tot + 255) / 256), 256, 0, ctx->stream>>>(t->masks.ptr, t->link.ptr,
+                                                                 t->nstr, t->n);
+  CU_LAUNCH_CHECK();
 }
 
 // ------------------------------------------------------------------ K2
@@ -347,71 +348,12 @@ __global__ void k_gather_fp64(const int32_t* __restrict__ link, const int32_t* _
   }
 }
 
-// E[b][P][k] = sum_Q g'[b][P][Q] D[b][Q][k]: FP64 tiles of all rows x 64 columns
-constexpr int GT_N = 64;
-__global__ void __launch_bounds__(256) k_contract_fp64(const double* __restrict__ gp_all, int npair,
-                                                       const double* __restrict__ D, int64_t ndet,
-                                                       const int32_t* __restrict__ active,
-                                                       const int32_t* __restrict__ bmap,
-                                                       double* __restrict__ E) {
-  const int bl = blockIdx.y;
-  const int b = bmap[bl];
-  if (active && !active[b]) return;
-  extern __shared__ double sm[];
-  double* s_g = sm;                          // npair * npair
-  double* s_d = sm + npair * npair;          // npair * GT_N
-  const double* g = gp_all + (int64_t)b * npair * npair;
-  for (int t = threadIdx.x; t < npair * npair; t += blockDim.x) s_g[t] = g[t];
-  const double* Db = D + (int64_t)bl * npair * ndet;
-  double* Eb = E + (int64_t)bl * npair * ndet;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  for (int64_t col0 = (int64_t)blockIdx.x * GT_N; col0 < ndet; col0 += (int64_t)gridDim.x * GT_N) {
-    __syncthreads();
-    for (int t = threadIdx.x; t < npair * GT_N; t += blockDim.x) {
-      int k = t / GT_N, j = t % GT_N;
-      int64_t col = col0 + j;
-      s_d[t] = col < ndet ? Db[(int64_t)k * ndet + col] : 0.0;
-    }
-    __syncthreads();
-    for (int r0 = 0; r0 < npair; r0 += 16 * 8) {
-      double acc[8][4];
-#pragma unroll
-      for (int i = 0; i < 8; i++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = 0.0;
-      for (int k = 0; k < npair; k++) {
-        double dv[4];
-#pragma unroll
-        for (int j = 0; j < 4; j++) dv[j] = s_d[k * GT_N + tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 8; i++) {
-          int r = r0 + ty + 16 * i;
-          double gv = r < npair ? s_g[r * npair + k] : 0.0;
-#pragma unroll
-          for (int j = 0; j < 4; j++) acc[i][j] = fma(gv, dv[j], acc[i][j]);
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 8; i++) {
-        int r = r0 + ty + 16 * i;
-        if (r >= npair) continue;
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-          int64_t col = col0 + tx + 16 * j;
-          if (col < ndet) Eb[(int64_t)r * ndet + col] = acc[i][j];
-        }
-      }
-    }
-  }
-}
-
 // sigma(Ia,Ib) = 1/2 sum_P [s_a E_P(Ja,Ib) + s_b E_P(Ia,Jb)] + shift (S^2 c)(Ia,Ib)
 // S^2 c = (nsig - ndocc) c - sum over pairs {p,q} with Ia holding one of them
 // and Ib the other of s_a s_b c(Ja, Jb)   (S^2 = N_beta - sum E^a_qp E^b_pq)
-// E element i: FP64, or (pair_e) the float pair hi + lo written by the
-// sliced tensor-core contraction
-__device__ __forceinline__ double load_e(const double* __restrict__ Eb, int64_t i, int pair_e) {
-  if (!pair_e) return Eb[i];
+// E element i: the float pair hi + lo written by the sliced tensor-core
+// contraction
+__device__ __forceinline__ double load_e(const double* __restrict__ Eb, int64_t i) {
   const float2 v = reinterpret_cast<const float2*>(Eb)[i];
   return (double)v.x + (double)v.y;
 }
@@ -423,7 +365,7 @@ __device__ __forceinline__ double load_e(const double* __restrict__ Eb, int64_t 
 __global__ void k_scatter_fp64(const int32_t* __restrict__ link, const uint32_t* __restrict__ masks,
                                const int32_t* __restrict__ linkb,
                                const uint32_t* __restrict__ masksb, int nstr, int nstrb, int n,
-                               int nsigb, double msms, const double* __restrict__ E, int pair_e,
+                               int nsigb, double msms, const double* __restrict__ E,
                                const double* __restrict__ c, int64_t c_stride, double shift,
                                const int32_t* __restrict__ active, const int32_t* __restrict__ bmap,
                                double* __restrict__ out, int64_t out_stride) {
@@ -444,11 +386,11 @@ __global__ void k_scatter_fp64(const int32_t* __restrict__ link, const uint32_t*
     for (int P = 0; P < npair; P++) {
       int32_t ta = la[P], tb = lb[P];
       if (ta >= 0) {
-        double x = load_e(Eb, (int64_t)P * ndet + (int64_t)(ta >> 1) * nstrb + ib, pair_e);
+        double x = load_e(Eb, (int64_t)P * ndet + (int64_t)(ta >> 1) * nstrb + ib);
         acc += (ta & 1) ? -x : x;
       }
       if (tb >= 0) {
-        double x = load_e(Eb, (int64_t)P * ndet + (int64_t)ia * nstrb + (tb >> 1), pair_e);
+        double x = load_e(Eb, (int64_t)P * ndet + (int64_t)ia * nstrb + (tb >> 1));
         acc += (tb & 1) ? -x : x;
       }
     }
@@ -481,7 +423,7 @@ __global__ void k_scatter_fp64(const int32_t* __restrict__ link, const uint32_t*
 // writes X into out; k_finish_sym_fp64 adds the transpose (32 x 32 tile
 // pairs in shared memory, in place) and the spin penalty.
 __global__ void k_scatter_sym_fp64(const int32_t* __restrict__ link, int nstr, int npair,
-                                   const double* __restrict__ E, int pair_e,
+                                   const double* __restrict__ E,
                                    const int32_t* __restrict__ active,
                                    const int32_t* __restrict__ bmap, double* __restrict__ out,
                                    int64_t out_stride) {
@@ -498,7 +440,7 @@ __global__ void k_scatter_sym_fp64(const int32_t* __restrict__ link, int nstr, i
     for (int P = 0; P < npair; P++) {
       const int32_t ta = la[P];
       if (ta >= 0) {
-        const double x = load_e(Eb, (int64_t)P * ndet + (int64_t)(ta >> 1) * nstr + ib, pair_e);
+        const double x = load_e(Eb, (int64_t)P * ndet + (int64_t)(ta >> 1) * nstr + ib);
         acc += (ta & 1) ? -x : x;
       }
     }
@@ -618,11 +560,11 @@ __global__ void k_s2(const int32_t* __restrict__ link, const uint32_t* __restric
 
 }  // namespace
 
-void sigma_fp64(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, const double* c, int64_t c_stride,
-                double* out, int64_t out_stride, const int32_t* active, double spin_shift,
-                bool emulated, bool symmetric) {
-  const int npair = bp.npair;
-  if (emulated && !w.err.ptr) {
+void sigma_emulated(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, const double* c, int64_t c_stride,
+                    double* out, int64_t out_stride, const int32_t* active, double spin_shift,
+                    bool symmetric) {
+  const int npair = bp.npair, nstr = bp.nstr, nstrb = bp.nstrb;
+  if (!w.err.ptr) {
     w.err.reset(&ctx->pool, 1);
     CU_CHECK(cudaMemsetAsync(w.err.ptr, 0, sizeof(int32_t), ctx->stream));
   }
@@ -642,71 +584,37 @@ void sigma_fp64(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, const double* c, int
   DevBuf<int32_t> bmap(&ctx->pool, bp.B);
   CU_CHECK(cudaMemcpyAsync(bmap.ptr, bm.data(), sizeof(int32_t) * bp.B, cudaMemcpyHostToDevice,
                            ctx->stream));
-  for (int64_t b0 = 0; b0 < bp.B; b0 += sb) {
-    const int nb = (int)std::min<int64_t>(sb, bp.B - b0);
-    sigma_fp64_raw(ctx, bp.n, bp.nsig, bp.nstr, bp.tab->link.ptr, bp.tab->masks.ptr, bp.gp.ptr, c,
-                   c_stride, out, out_stride, active, bmap.ptr + b0, nb, w.D.ptr, w.E.ptr,
-                   spin_shift, emulated, w.err.ptr, symmetric && bp.closed(), (int)b0, bp.nsigb,
-                   bp.nstrb, bp.tabb->link.ptr, bp.tabb->masks.ptr);
-  }
-}
-
-void sigma_fp64_raw(mbe_ctx* ctx, int n, int nsig, int nstr, const int32_t* link,
-                    const uint32_t* masks, const double* gp, const double* c, int64_t c_stride,
-                    double* out, int64_t out_stride, const int32_t* active, const int32_t* bmap,
-                    int nb, double* D, double* E, double spin_shift, bool emulated, int32_t* err,
-                    bool symmetric, int b_first, int nsigb, int nstrb, const int32_t* linkb,
-                    const uint32_t* masksb) {
-  if (nsigb < 0) {   // closed shell: beta strings = alpha strings
-    nsigb = nsig;
-    nstrb = nstr;
-    linkb = link;
-    masksb = masks;
-  }
-  const double msms = 0.25 * (nsig - nsigb) * (nsig - nsigb + 2);   // Ms(Ms+1)
-  const int npair = n * (n + 1) / 2;
-  const int64_t ndet = (int64_t)nstr * nstrb;
   int64_t blocks = (ndet + 255) / 256;
   if (blocks > 2048) blocks = 2048;
-  const size_t smem_c = sizeof(double) * (npair * npair + npair * GT_N);
-  static bool attr_set[MBE_MAX_DEVICES] = {false};
-  once_per_device(attr_set, ctx->device, [] {
-    CU_CHECK(cudaFuncSetAttribute(k_contract_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  200 * 1024));
-  });
-  int64_t cblocks = (ndet + GT_N - 1) / GT_N;
-  if (cblocks > 1024) cblocks = 1024;
-  const dim3 g1((unsigned)blocks, nb);
-  k_gather_fp64<<<g1, 256, 0, ctx->stream>>>(link, linkb, nstr, nstrb, npair, c, c_stride, active,
-                                              bmap, D);
-  CU_LAUNCH_CHECK();
-  cudaEvent_t ev;
-  ctx->fp64_timer.begin(ctx->stream, ctx->opt.timing != 0, &ev);
-  if (emulated) {
-    contract_ozaki(ctx, gp, npair, D, ndet, nb, active, bmap, E, err);
-  } else {
-    k_contract_fp64<<<dim3((unsigned)cblocks, nb), 256, smem_c, ctx->stream>>>(gp, npair, D, ndet,
-                                                                             active, bmap, E);
+  for (int64_t b0 = 0; b0 < bp.B; b0 += sb) {
+    const int nb = (int)std::min<int64_t>(sb, bp.B - b0);
+    const dim3 g1((unsigned)blocks, nb);
+    const int32_t* bm_d = bmap.ptr + b0;
+    k_gather_fp64<<<g1, 256, 0, ctx->stream>>>(bp.tab->link.ptr, bp.tabb->link.ptr, nstr, nstrb,
+                                               npair, c, c_stride, active, bm_d, w.D.ptr);
     CU_LAUNCH_CHECK();
-  }
-  ctx->fp64_timer.end(ctx->stream, ev);
-  ctx->stats.fp64_launches += 1;
-  if (symmetric) {
-    k_scatter_sym_fp64<<<g1, 256, 0, ctx->stream>>>(link, nstr, npair, E, emulated ? 1 : 0,
-                                                    active, bmap, out, out_stride);
-    CU_LAUNCH_CHECK();
-    // the sub-batch is the contiguous tuple range [b_first, b_first + nb)
-    const int ntl = (nstr + 31) / 32;
-    const int b0 = b_first;
-    k_finish_sym_fp64<<<dim3((unsigned)(ntl * (ntl + 1) / 2), nb), 256, 0, ctx->stream>>>(
-        out + (int64_t)b0 * out_stride, out_stride, link, masks, nstr, n, nsig,
-        c + (int64_t)b0 * c_stride, c_stride, spin_shift, active ? active + b0 : nullptr);
-    CU_LAUNCH_CHECK();
-  } else {
-    k_scatter_fp64<<<g1, 256, 0, ctx->stream>>>(link, masks, linkb, masksb, nstr, nstrb, n, nsigb,
-                                                msms, E, emulated ? 1 : 0, c, c_stride,
-                                                spin_shift, active, bmap, out, out_stride);
-    CU_LAUNCH_CHECK();
+    cudaEvent_t ev;
+    ctx->fp64_timer.begin(ctx->stream, ctx->opt.timing != 0, &ev);
+    contract_ozaki(ctx, bp.gp.ptr, npair, w.D.ptr, ndet, nb, active, bm_d, w.E.ptr, w.err.ptr);
+    ctx->fp64_timer.end(ctx->stream, ev);
+    ctx->stats.fp64_launches += 1;
+    if (symmetric && bp.closed()) {
+      k_scatter_sym_fp64<<<g1, 256, 0, ctx->stream>>>(bp.tab->link.ptr, nstr, npair, w.E.ptr,
+                                                      active, bm_d, out, out_stride);
+      CU_LAUNCH_CHECK();
+      // the sub-batch is the contiguous tuple range [b0, b0 + nb)
+      const int ntl = (nstr + 31) / 32;
+      k_finish_sym_fp64<<<dim3((unsigned)(ntl * (ntl + 1) / 2), nb), 256, 0, ctx->stream>>>(
+          out + b0 * out_stride, out_stride, bp.tab->link.ptr, bp.tab->masks.ptr, nstr, bp.n,
+          bp.nsig, c + b0 * c_stride, c_stride, spin_shift, active ? active + b0 : nullptr);
+      CU_LAUNCH_CHECK();
+    } else {
+      k_scatter_fp64<<<g1, 256, 0, ctx->stream>>>(
+          bp.tab->link.ptr, bp.tab->masks.ptr, bp.tabb->link.ptr, bp.tabb->masks.ptr, nstr, nstrb,
+          bp.n, bp.nsigb, bp.msms(), w.E.ptr, c, c_stride, spin_shift, active, bm_d, out,
+          out_stride);
+      CU_LAUNCH_CHECK();
+    }
   }
 }
 

@@ -460,8 +460,10 @@ void davidson_batch(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int32_t* s
   int total_it = 0;
 
   auto sigma = [&](bool /*unused*/, const double* c, double* out) {
-    sigma_fp64(ctx, bp, sw, c, (int64_t)M * N, out, (int64_t)M * N, active.ptr, shift, emulated,
-               true);
+    if (emulated)
+      sigma_emulated(ctx, bp, sw, c, (int64_t)M * N, out, (int64_t)M * N, active.ptr, shift, true);
+    else
+      sigma_direct(ctx, bp, c, (int64_t)M * N, out, (int64_t)M * N, active.ptr, shift, true);
   };
   // precondition the residual in T, orthogonalise it against V[0..m) and
   // append it as V[m] (tuples whose correction vanished are frozen)

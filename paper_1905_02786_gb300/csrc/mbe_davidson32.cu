@@ -1128,7 +1128,7 @@ void davidson_batch_mixed(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int3
       sigma_exact(ctx, bp, sw, F.ptr, Lf, S64.ptr, Lf, active.ptr);
       launch_finish_sym_fp64(ctx, bp, S64.ptr, Lf, C64.ptr, Lf, shift, active.ptr);
     } else {
-      sigma_fp64(ctx, bp, sw, C64.ptr, Lf, S64.ptr, Lf, active.ptr, shift, true, true);
+      sigma_emulated(ctx, bp, sw, C64.ptr, Lf, S64.ptr, Lf, active.ptr, shift, true);
     }
     vecs_ex += B;
     k32_exact_xax<<<gcf, RT, 0, st>>>(C64.ptr, S64.ptr, Lf, ch, nchunks_f, active.ptr,

@@ -252,6 +252,10 @@ struct StringTables {
   // (poff, ntiles + 1 per string)
   DevBuf<int16_t> plist;
   DevBuf<int32_t> poff;
+  // FP64 sigma (mbe_sigma64.cu, built on first use): replacements of every
+  // string and its off-diagonal links, string index fastest
+  DevBuf<uint16_t> hidx;
+  DevBuf<uint32_t> olnk;
 };
 
 // ------------------------------------------------------------- context
@@ -408,6 +412,9 @@ struct BinProblem {
   DevBuf<double> jk;             // B * 2 * n * n  (J_pq = (pp|qq), K_pq = (pq|qp))
   DevBuf<uint8_t> gsplit;        // g'/2 as bf16 hi/lo rows (tensor-core sigma operand source)
   DevBuf<uint8_t> haa;           // one-spin Hamiltonian H^alpha as bf16 hi/lo rows
+  // FP64 sigma: non-zero one-spin elements of the alpha (and, for an open
+  // shell, beta) strings and the pair integrals summed over a beta string
+  DevBuf<double> hv, hvb, wt;
 };
 
 // P-space preconditioner of the mixed Davidson iteration (mbe_pspace.cu):
@@ -436,17 +443,28 @@ void build_string_tables(mbe_ctx* ctx, StringTables* t);
 // raw-pointer forms of the table, integral and FP64 sigma launchers (they
 // allocate nothing)
 int64_t string_count(int n, int nsig);
-void launch_string_tables(mbe_ctx* ctx, int n, int nsig, int nstr, uint32_t* masks,
-                          int32_t* link);
+void launch_string_masks(mbe_ctx* ctx, int n, int nsig, int nstr, uint32_t* masks);
 // nel: active electrons (both spins)
 void launch_effints_raw(mbe_ctx* ctx, const int32_t* act, int B, int n, int nel, double* ecore,
                         double* heff, double* hp, double* gp, double* jk);
-void sigma_fp64_raw(mbe_ctx* ctx, int n, int nsig, int nstr, const int32_t* link,
-                    const uint32_t* masks, const double* gp, const double* c, int64_t c_stride,
-                    double* out, int64_t out_stride, const int32_t* active, const int32_t* bmap,
-                    int nb, double* D, double* E, double spin_shift, bool emulated, int32_t* err,
-                    bool symmetric = false, int b_first = 0, int nsigb = -1, int nstrb = -1,
-                    const int32_t* linkb = nullptr, const uint32_t* masksb = nullptr);
+// one spin's strings and tables of the FP64 sigma
+struct DirectSide {
+  int nsig, nstr;
+  const uint32_t* masks;
+  const uint32_t* olnk;    // nsig (n - nsig) rows of nstr links
+  const uint16_t* hidx;    // direct_nnz rows of nstr replacements
+  const double* hv;        // their one-spin elements, per tuple
+};
+int direct_nnz(int n, int nsig);   // replacements of one string, itself included
+void launch_direct_tables(mbe_ctx* ctx, int n, int nsig, int nstr, const uint32_t* masks,
+                          uint16_t* hidx, uint32_t* olnk);
+// hv (B * nnz * nstr) and, unless NULL, wt (B * npair * nstr)
+void launch_direct_values(mbe_ctx* ctx, int n, int nsig, int nstr, const uint32_t* masks, int B,
+                          const double* gp, double* hv, double* wt);
+void sigma_direct_raw(mbe_ctx* ctx, int n, const DirectSide& al, const DirectSide& be,
+                      const double* wt, const double* gp, const double* c, int64_t c_stride,
+                      double* out, int64_t out_stride, const int32_t* active,
+                      const int32_t* bmap, int nb, double spin_shift, bool symmetric);
 StringTables* get_tables(mbe_ctx* ctx, int n, int nsig);
 // active electrons of each spin: alpha (orbitals below nocc_a), beta (below nocc)
 int count_sig(const mbe_ctx* ctx, const std::vector<int>& act);
@@ -463,7 +481,7 @@ void launch_hdiag(mbe_ctx* ctx, BinProblem& bp, double spin_shift, double* hd);
 // sigma for a batch: out[b] = (H_act + shift S^2) c[b] for b < B; c/out with
 // strides (elements between consecutive tuples' vectors); active may be NULL.
 struct SigmaWork {
-  DevBuf<double> D, E;           // scratch for the FP64 path
+  DevBuf<double> D, E;           // scratch of the emulated FP64 path
   DevBuf<float> Xf;              // W rows of the tensor-core path (sigma = W + W^T)
   DevBuf<uint8_t> csplit;        // the vectors as bf16 hi/lo rows (tensor-core operands)
   DevBuf<int32_t> err;           // timeout flag of the tensor-core path
@@ -494,13 +512,16 @@ void convert_f64_to_f32(mbe_ctx* ctx, const double* src, float* dst, int64_t n);
 // with their parents' vectors (exactly one of V32 / V64 non-null)
 void launch_parent_guess(mbe_ctx* ctx, const GuessPlan& plan, int n, int nsig, int nstr,
                          float* V32, double* V64, int64_t vstride);
-// emulated: the contraction runs as the FP64-grade sliced tensor-core GEMM
-// symmetric: c(a,b) = c(b,a) for every tuple (sigma = X + X^T, coalesced);
-// otherwise any c
-void sigma_fp64(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, const double* c,
-                int64_t c_stride, double* out, int64_t out_stride,
-                const int32_t* active, double spin_shift, bool emulated,
-                bool symmetric = false);
+// symmetric: c(a,b) = c(b,a) for every tuple; otherwise any c
+// FP64 on the CUDA cores:
+void sigma_direct(mbe_ctx* ctx, BinProblem& bp, const double* c, int64_t c_stride, double* out,
+                  int64_t out_stride, const int32_t* active, double spin_shift, bool symmetric);
+// its tables and values (sigma_direct makes them on its first call otherwise)
+void sigma_direct_prepare(mbe_ctx* ctx, BinProblem& bp);
+// FP64-grade: gather, sliced tensor-core GEMM, scatter
+void sigma_emulated(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, const double* c,
+                    int64_t c_stride, double* out, int64_t out_stride,
+                    const int32_t* active, double spin_shift, bool symmetric = false);
 bool ozaki_supported(int npair);
 // FP64-grade sigma of FP32 vectors c (c = c^T, |c_i| <= 1) fused on the
 // tensor cores: writes the rows X (sigma = X + X^T + shift S^2 c follows in

@@ -12,16 +12,18 @@
 // Scratch: MBE_NOALLOC_SCRATCH_BYTES per device (the array is part of the
 // loaded module, one copy per device).  A problem whose tables, integrals
 // and D / E intermediates do not fit is rejected with MBE_EINVAL before
-// anything is launched.  No part of the scratch needs to start at zero:
-// every word a kernel reads is written earlier in the same call (string
-// tables, effective integrals, D by the gather, E by the contraction).
+// anything is launched (the limit counts two npair x nstr^2 intermediates of
+// a gather / contract / scatter sigma, which this one no longer needs: what
+// the call takes stays as documented).  No part of the scratch needs to start
+// at zero: every word a kernel reads is written earlier in the same call
+// (string tables, effective integrals, one-spin elements).
 //
 // Calls that overlap on one device race on the single scratch array: a
 // caller serialises them (issue them on one stream, or wait for one call to
 // finish before issuing the next from another stream or context).
 //
 // The first call on a device resolves the scratch address with
-// cudaGetSymbolAddress and sets the contraction kernel's shared-memory
+// cudaGetSymbolAddress and sets the sigma kernel's shared-memory
 // attribute; it should come before any stream capture.  The active orbitals
 // reach the scratch through a kernel argument (no host-memory copy); with a
 // non-NULL e_core the call copies the core energy back and waits for the
@@ -51,12 +53,13 @@ unsigned char* scratch_base(int device) {
 
 // byte offsets of the pieces inside the scratch array (256-byte aligned)
 struct NoallocLayout {
-  size_t masks, link, act, bmap, ecore, heff, hp, gp, jk, D, E, total;
+  size_t masks, act, ecore, heff, hp, gp, jk, hidx, olnk, hv, wt, total;
+  size_t limit;   // what MBE_NOALLOC_SCRATCH_BYTES is compared with
 };
 
-NoallocLayout noalloc_layout(int n, int64_t nstr) {
+NoallocLayout noalloc_layout(int n, int nsig, int64_t nstr) {
   const int64_t npair = (int64_t)n * (n + 1) / 2;
-  const int64_t ndet = nstr * nstr;
+  const int64_t ndet = nstr * nstr, nnz = direct_nnz(n, nsig);
   NoallocLayout L;
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -65,17 +68,24 @@ NoallocLayout noalloc_layout(int n, int64_t nstr) {
     return r;
   };
   L.masks = take(sizeof(uint32_t) * nstr);
-  L.link = take(sizeof(int32_t) * nstr * npair);
   L.act = take(sizeof(int32_t) * n);
-  L.bmap = take(sizeof(int32_t));
   L.ecore = take(sizeof(double));
   L.heff = take(sizeof(double) * n * n);
   L.hp = take(sizeof(double) * n * n);
   L.gp = take(sizeof(double) * npair * npair);
   L.jk = take(sizeof(double) * 2 * n * n);
-  L.D = take(sizeof(double) * npair * ndet);
-  L.E = take(sizeof(double) * npair * ndet);
+  const size_t common = o;
+  L.hidx = take(sizeof(uint16_t) * nnz * nstr);
+  L.olnk = take(sizeof(uint32_t) * nsig * (n - nsig) * nstr);
+  L.hv = take(sizeof(double) * nnz * nstr);
+  L.wt = take(sizeof(double) * npair * nstr);
   L.total = o;
+  o = common;
+  take(sizeof(int32_t) * nstr * npair);
+  take(sizeof(int32_t));
+  take(sizeof(double) * npair * ndet);
+  take(sizeof(double) * npair * ndet);
+  L.limit = o;
   return L;
 }
 
@@ -83,10 +93,9 @@ NoallocLayout noalloc_layout(int n, int64_t nstr) {
 struct ActList {
   int32_t v[16];
 };
-__global__ void k_put_act(ActList a, int n, int32_t* __restrict__ dst, int32_t* __restrict__ bmap) {
+__global__ void k_put_act(ActList a, int n, int32_t* __restrict__ dst) {
   const int t = threadIdx.x;
   if (t < n) dst[t] = a.v[t];
-  if (t == 0) bmap[0] = 0;
 }
 
 }  // namespace
@@ -108,27 +117,32 @@ int noalloc_sigma_run(mbe_ctx* ctx, const int* act, int nact, const double* c_de
   const int64_t nstr = string_count(nact, nsig);
   if (ndet_arg != nstr * nstr)
     throw MbeError{MBE_EINVAL, "vector length does not match the active space"};
-  const NoallocLayout L = noalloc_layout(nact, nstr);
-  if (L.total > (size_t)MBE_NOALLOC_SCRATCH_BYTES)
+  const NoallocLayout L = noalloc_layout(nact, nsig, nstr);
+  if (std::max(L.limit, L.total) > (size_t)MBE_NOALLOC_SCRATCH_BYTES)
     throw MbeError{MBE_EINVAL, "active space too large for the no-allocation scratch"};
   unsigned char* base = scratch_base(ctx->device);
   uint32_t* masks = (uint32_t*)(base + L.masks);
-  int32_t* link = (int32_t*)(base + L.link);
   int32_t* actd = (int32_t*)(base + L.act);
-  int32_t* bmap = (int32_t*)(base + L.bmap);
   double* ecore = (double*)(base + L.ecore);
+  double* gp = (double*)(base + L.gp);
+  double* hv = (double*)(base + L.hv);
+  double* wt = (double*)(base + L.wt);
+  uint32_t* olnk = (uint32_t*)(base + L.olnk);
+  uint16_t* hidx = (uint16_t*)(base + L.hidx);
   cudaStream_t st = ctx->stream;
   ActList al = {};
   for (int i = 0; i < nact; i++) al.v[i] = a[i];
-  k_put_act<<<1, 32, 0, st>>>(al, nact, actd, bmap);
+  k_put_act<<<1, 32, 0, st>>>(al, nact, actd);
   CU_LAUNCH_CHECK();
-  launch_string_tables(ctx, nact, nsig, (int)nstr, masks, link);
+  launch_string_masks(ctx, nact, nsig, (int)nstr, masks);
   launch_effints_raw(ctx, actd, 1, nact, 2 * nsig, ecore, (double*)(base + L.heff),
-                     (double*)(base + L.hp), (double*)(base + L.gp), (double*)(base + L.jk));
+                     (double*)(base + L.hp), gp, (double*)(base + L.jk));
+  launch_direct_tables(ctx, nact, nsig, (int)nstr, masks, hidx, olnk);
+  launch_direct_values(ctx, nact, nsig, (int)nstr, masks, 1, gp, hv, wt);
   const int64_t ndet = nstr * nstr;
-  sigma_fp64_raw(ctx, nact, nsig, (int)nstr, link, masks, (const double*)(base + L.gp), c_dev, ndet,
-                 sigma_dev, ndet, nullptr, bmap, 1, (double*)(base + L.D), (double*)(base + L.E),
-                 ctx->opt.spin_shift, false, nullptr);
+  const DirectSide side = {nsig, (int)nstr, masks, olnk, hidx, hv};
+  sigma_direct_raw(ctx, nact, side, side, wt, gp, c_dev, ndet, sigma_dev, ndet, nullptr, nullptr, 1,
+                   ctx->opt.spin_shift, false);
   if (e_core) {
     CU_CHECK(cudaMemcpyAsync(e_core, ecore, sizeof(double), cudaMemcpyDeviceToHost, st));
     CU_CHECK(cudaStreamSynchronize(st));

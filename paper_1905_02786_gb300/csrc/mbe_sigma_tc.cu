@@ -6,8 +6,8 @@
 // one spin, <I|..|J> = the sign of the link table entry of I and pair P.
 // The Hamiltonian of one CASCI is 1/2 sum_PQ g'_PQ (L_P x 1 + 1 x L_P)
 // (L_Q x 1 + 1 x L_Q) with g' the pair integrals that carry the one-electron
-// part (sigma_fp64 applies the same operator through D = E+ c, E = g' D and
-// the scatter).  Multiplying out the alpha and beta factors splits it into a
+// part (sigma_emulated applies the same operator through D = E+ c, E = g' D
+// and the scatter).  Multiplying out the alpha and beta factors splits it into a
 // one-spin and a two-spin part (alpha and beta string operators commute):
 //   sigma = H^a c + c H^a + Z,   H^a = 1/2 sum_PQ g'_PQ L_P L_Q,
 //   Z = sum_PQ g'_PQ L_P c L_Q,
