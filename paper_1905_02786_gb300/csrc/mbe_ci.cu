@@ -265,7 +265,7 @@ __device__ __forceinline__ double string_self(uint32_t m, const double* heff, co
 __global__ void k_hdiag(const uint32_t* __restrict__ masks, const uint32_t* __restrict__ masksb,
                         int nstr, int nstrb, int n, int nsigb, double msms,
                         const double* __restrict__ heff_all, const double* __restrict__ jk_all,
-                        double shift, double* hd_all) {
+                        double shift, double* hd_all, int64_t ld, int packed) {
   const int b = blockIdx.y;
   extern __shared__ double sm[];
   double* s_heff = sm;
@@ -281,6 +281,7 @@ __global__ void k_hdiag(const uint32_t* __restrict__ masks, const uint32_t* __re
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < ndet;
        i += (int64_t)gridDim.x * blockDim.x) {
     int ia = (int)(i / nstrb), ib = (int)(i % nstrb);
+    if (packed && ia > ib) continue;
     uint32_t ma = masks[ia], mb = masksb[ib];
     double ea = string_self(ma, s_heff, s_J, s_K, n);
     double eb = string_self(mb, s_heff, s_J, s_K, n);
@@ -294,13 +295,15 @@ __global__ void k_hdiag(const uint32_t* __restrict__ masks, const uint32_t* __re
       }
     }
     int ndocc = __popc(ma & mb);
-    hd_all[(int64_t)b * ndet + i] = (ea + eb) + cross + shift * ((double)(nsigb - ndocc) + msms);
+    hd_all[(int64_t)b * ld + (packed ? sym_index(ia, ib, nstr) : i)] =
+        (ea + eb) + cross + shift * ((double)(nsigb - ndocc) + msms);
   }
 }
 
 }  // namespace
 
-void launch_hdiag(mbe_ctx* ctx, BinProblem& bp, double spin_shift, double* hd) {
+void launch_hdiag(mbe_ctx* ctx, BinProblem& bp, double spin_shift, double* hd, int64_t ld,
+                  bool packed) {
   const int n = bp.n;
   size_t smem = 3 * sizeof(double) * n * n;
   int64_t blocks = (bp.ndet + 255) / 256;
@@ -308,7 +311,7 @@ void launch_hdiag(mbe_ctx* ctx, BinProblem& bp, double spin_shift, double* hd) {
   dim3 grid((unsigned)blocks, bp.B);
   k_hdiag<<<grid, 256, smem, ctx->stream>>>(bp.tab->masks.ptr, bp.tabb->masks.ptr, bp.nstr,
                                             bp.nstrb, n, bp.nsigb, bp.msms(), bp.heff.ptr,
-                                            bp.jk.ptr, spin_shift, hd);
+                                            bp.jk.ptr, spin_shift, hd, ld, packed ? 1 : 0);
   CU_LAUNCH_CHECK();
 }
 

@@ -1,362 +1,117 @@
 // Batched Davidson iteration (Davidson, J. Comput. Phys. 17, 87 (1975)) for
-// the lowest singlet of every CASCI of one bin in the FP64 and emulated-FP64
-// modes (the mixed mode's Davidson is in mbe_davidson32.cu), FP64 throughout:
-//   K5  batched projections V^T w (two-phase, fixed-order reductions)
-//   K6  Rayleigh-Ritz: cyclic Jacobi on the m x m projected matrix, one warp
-//       per tuple
-//   K7  residual r = AV y - theta V y, diagonal preconditioner
-//       t = r / (theta - H_II) with |denominator| >= 1e-8, two-pass
-//       Gram-Schmidt, normalisation
-// The operator is H_active + spin_shift * S^2 restricted to the alpha<->beta
-// symmetric vectors; the start vector is the lowest diagonal determinant,
-// symmetrised.  All tuples of a batch share the subspace size m; a tuple
-// that has converged is frozen (every kernel skips it).
-#include "mbe_internal.cuh"
-#include "mbe_ritz.cuh"
+// the lowest state of every CASCI of one bin in the FP64 and emulated-FP64
+// modes (the mixed mode's Davidson is in mbe_davidson32.cu), FP64 throughout.
+// The operator is H_active + spin_shift * S^2; a closed shell is restricted to
+// the alpha<->beta symmetric vectors, kept packed (half the bytes and half
+// the FP64 operations of the full ones).  The start vector is the lowest
+// diagonal determinant, symmetrised; the preconditioner t = r / (theta -
+// H_II) with |denominator| >= 1e-8; two-pass Gram-Schmidt.  All tuples of a
+// batch share the subspace size m; a tuple that has converged is frozen
+// (every kernel skips it).
+//
+// An iteration is six kernels: append (V[m] = T / |T|, expanded to the full
+// vector the sigma reads), sigma, subspace row with the Ritz step, residual
+// with the preconditioner and the convergence test, two Gram-Schmidt passes
+// (mbe_dvec.cuh), issued as one CUDA graph.  Small batches are bound by that
+// chain: with a launch for each reduction it was 22 kernels and 330 us per
+// iteration on 17 CASCIs of 6e/7o and 8e/7o.
+#include "mbe_dvec.cuh"
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <limits>
+
+using namespace dvec;
 
 namespace {
 
-constexpr int DOT_CHUNK = 4096;
-
-// partial[b][i][chunk] = sum over the chunk of X[b][i][k] * y[b][k], i < m
-__global__ void k_multidot_partial(const double* __restrict__ X, int64_t x_bstride,
-                                   int64_t x_vstride, const double* __restrict__ Y,
-                                   int64_t y_bstride, int m, int64_t N, int nchunks,
-                                   const int32_t* __restrict__ active, double* __restrict__ partial) {
+// V[m] = T / |T| of the tuples still iterating, and (closed shell) the full
+// vector C from it, one CTA per 32 x 32 tile pair, both halves written
+// coalesced.  inv == NULL: C from V[m] as it stands (every tuple).
+__global__ void k_append_sym(const double* __restrict__ T, double* __restrict__ V, int64_t vstride,
+                             int64_t L, const double* __restrict__ inv, int nstr,
+                             const int32_t* __restrict__ active, double* __restrict__ C) {
   const int b = blockIdx.y;
   if (active && !active[b]) return;
-  const int chunk = blockIdx.x;
-  const int64_t k0 = (int64_t)chunk * DOT_CHUNK;
-  const int64_t k1 = min(N, k0 + DOT_CHUNK);
-  __shared__ double red[32][33];
-  const double* yb = Y + (int64_t)b * y_bstride;
-  for (int i0 = 0; i0 < m; i0 += 32) {
-    double acc[32];
-    const int ni = min(32, m - i0);
-#pragma unroll
-    for (int i = 0; i < 32; i++) acc[i] = 0.0;
-    for (int64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
-      double yv = yb[k];
-#pragma unroll
-      for (int i = 0; i < 32; i++)
-        if (i < ni) acc[i] = fma(X[(int64_t)b * x_bstride + (int64_t)(i0 + i) * x_vstride + k], yv, acc[i]);
+  const int nt = (nstr + 31) / 32;
+  int t = blockIdx.x, I = 0;
+  while (t >= nt - I) {
+    t -= nt - I;
+    I++;
+  }
+  const int J = I + t;
+  __shared__ double sC[32][33];
+  double* Vb = V + (int64_t)b * vstride;
+  const double* src = inv ? T + (int64_t)b * L : Vb;
+  const double f = inv ? inv[b] : 1.0;
+  double* Cb = C + (int64_t)b * nstr * nstr;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, ny = blockDim.x >> 5;
+  for (int i = ty; i < 32; i += ny) {
+    const int r = I * 32 + i, k = J * 32 + tx;
+    double v = 0.0;
+    if (r < nstr && k < nstr && (I < J || r <= k)) {
+      const int64_t p = sym_index(r, k, nstr);
+      v = src[p] * f;
+      if (inv) Vb[p] = v;
+      Cb[(int64_t)r * nstr + k] = v;
     }
-    // reduce over the block: warp shuffle then shared memory (fixed order)
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < 32; i++) {
-      double v = acc[i];
-      for (int off = 16; off; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-      if (lane == 0) red[warp][i] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < ni) {
-      double s = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); w++) s += red[w][threadIdx.x];
-      partial[((int64_t)b * m + i0 + threadIdx.x) * nchunks + chunk] = s;
-    }
-    __syncthreads();
-  }
-}
-
-__global__ void k_multidot_final(const double* __restrict__ partial, int m, int nchunks,
-                                 const int32_t* __restrict__ active, double* __restrict__ out,
-                                 int64_t out_bstride, int64_t out_istride) {
-  const int b = blockIdx.x;
-  if (active && !active[b]) return;
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    const double* p = partial + ((int64_t)b * m + i) * nchunks;
-    double s = 0.0;
-    for (int c = 0; c < nchunks; c++) s += p[c];
-    out[(int64_t)b * out_bstride + (int64_t)i * out_istride] = s;
-  }
-}
-
-// G[b][j][i] = G[b][i][j] = dots[b][i] for i < m (row/column j = m-1)
-__global__ void k_store_grow(const double* __restrict__ dots, int m, int M,
-                             const int32_t* __restrict__ active, double* __restrict__ G) {
-  const int b = blockIdx.x;
-  if (!active[b]) return;
-  const int j = m - 1;
-  for (int i = threadIdx.x; i < m; i += blockDim.x) {
-    double v = dots[(int64_t)b * M + i];
-    G[(int64_t)b * M * M + (int64_t)j * M + i] = v;
-    G[(int64_t)b * M * M + (int64_t)i * M + j] = v;
-  }
-}
-
-// lowest eigenpair of the m x m subspace matrix G[b] (one warp per tuple)
-__global__ void k_jacobi(const double* __restrict__ G, int m, int M,
-                        const int32_t* __restrict__ active, double* __restrict__ theta,
-                        double* __restrict__ y) {
-  const int b = blockIdx.x;
-  if (!active[b]) return;
-  __shared__ RitzShared S;
-  ritz_lowest(G + (int64_t)b * M * M, m, M, S, theta + b, y + (int64_t)b * M);
-}
-
-// x = V y, T = AV y - theta x, partial ||T||^2; X receives x.
-__global__ void k_residual(const double* __restrict__ V, const double* __restrict__ AV, int m,
-                           int M, int64_t N, const double* __restrict__ y,
-                           const double* __restrict__ theta, const int32_t* __restrict__ active,
-                           double* __restrict__ X, double* __restrict__ T, int nchunks,
-                           double* __restrict__ partial) {
-  const int b = blockIdx.y;
-  if (!active[b]) return;
-  __shared__ double sy[32];
-  __shared__ double red[32];
-  if (threadIdx.x < m) sy[threadIdx.x] = y[(int64_t)b * M + threadIdx.x];
-  __syncthreads();
-  const double th = theta[b];
-  const int64_t k0 = (int64_t)blockIdx.x * DOT_CHUNK, k1 = min(N, k0 + DOT_CHUNK);
-  const double* Vb = V + (int64_t)b * M * N;
-  const double* AVb = AV + (int64_t)b * M * N;
-  double acc = 0.0;
-  for (int64_t k = k0 + threadIdx.x; k < k1; k += blockDim.x) {
-    double x = 0.0, ax = 0.0;
-    for (int i = 0; i < m; i++) {
-      x = fma(sy[i], Vb[(int64_t)i * N + k], x);
-      ax = fma(sy[i], AVb[(int64_t)i * N + k], ax);
-    }
-    double r = ax - th * x;
-    X[(int64_t)b * N + k] = x;
-    T[(int64_t)b * N + k] = r;
-    acc = fma(r, r, acc);
-  }
-  for (int off = 16; off; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); w++) s += red[w];
-    partial[(int64_t)b * nchunks + blockIdx.x] = s;
-  }
-}
-
-// convergence bookkeeping after the residual norms are known
-__global__ void k_converge(const double* __restrict__ partial, int nchunks, int B, int it,
-                           const double* __restrict__ tol_r, double tol_e, int rel,
-                           const double* __restrict__ theta,
-                           double* __restrict__ theta_old, double* __restrict__ rnorm,
-                           int32_t* __restrict__ active, int32_t* __restrict__ iters,
-                           int32_t* __restrict__ nactive) {
-  __shared__ int cnt;
-  if (threadIdx.x == 0) cnt = 0;
-  __syncthreads();
-  for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    if (!active[b]) continue;
-    double s = 0.0;
-    for (int c = 0; c < nchunks; c++) s += partial[(int64_t)b * nchunks + c];
-    double rn = sqrt(s);
-    rnorm[b] = rn;
-    iters[b] += 1;
-    // rel: the residual tolerance scales with max(1, |theta|) (the floor of a
-    // reduced-precision sigma is relative to the size of H)
-    const double tr = rel ? tol_r[b] * fmax(1.0, fabs(theta[b])) : tol_r[b];
-    bool conv = it > 0 && fabs(theta[b] - theta_old[b]) < tol_e && rn < tr;
-    theta_old[b] = theta[b];
-    if (conv) active[b] = 0;
-    else atomicAdd(&cnt, 1);
+    sC[i][tx] = v;
   }
   __syncthreads();
-  if (threadIdx.x == 0) *nactive = cnt;
-}
-
-// Restart keeping two vectors: the current Ritz vector x = V y and the
-// previous one, orthonormalised against x in coefficient space
-// (q = y_prev - (y.y_prev) y, twice, normalised; V is orthonormal, so this
-// avoids the cancellation of subtracting two nearly parallel long vectors).
-// The new 2x2 projected matrix is [y q]^T G [y q].  One warp per tuple.
-__global__ void k_restart_coef(const double* __restrict__ y, double* __restrict__ yp, int m, int M,
-                               const int32_t* __restrict__ active, double* __restrict__ G) {
-  const int b = blockIdx.x;
-  if (!active[b]) return;
-  __shared__ double sy[32], sq[32], sG[32][33];
-  const int r = threadIdx.x;
-  sy[r] = r < m ? y[(int64_t)b * M + r] : 0.0;
-  sq[r] = r < m ? yp[(int64_t)b * M + r] : 0.0;
-  for (int i = 0; i < m; i++)
-    if (r < m) sG[i][r] = G[(int64_t)b * M * M + (int64_t)i * M + r];
-  __syncwarp();
-  auto wsum = [](double v) {
-    for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
-  };
-  for (int pass = 0; pass < 2; pass++) {
-    double d = wsum(sy[r] * sq[r]);
-    sq[r] -= d * sy[r];
-    __syncwarp();
-  }
-  double nq = sqrt(wsum(sq[r] * sq[r]));
-  if (!(nq > 1e-14)) {
-    // x did not move: take the unit vector on which x has least weight
-    double a = r < m ? fabs(sy[r]) : 1e300;
-    int idx = r;
-    for (int off = 16; off; off >>= 1) {
-      double oa = __shfl_xor_sync(0xffffffffu, a, off);
-      int oi = __shfl_xor_sync(0xffffffffu, idx, off);
-      if (oa < a || (oa == a && oi < idx)) { a = oa; idx = oi; }
-    }
-    sq[r] = (r == idx) ? 1.0 : 0.0;
-    __syncwarp();
-    double d = wsum(sy[r] * sq[r]);
-    sq[r] -= d * sy[r];
-    __syncwarp();
-    nq = sqrt(wsum(sq[r] * sq[r]));
-  }
-  sq[r] /= nq;
-  __syncwarp();
-  double gy = 0.0, gq = 0.0;   // (G y)_r, (G q)_r
-  if (r < m)
-    for (int j = 0; j < m; j++) {
-      gy = fma(sG[r][j], sy[j], gy);
-      gq = fma(sG[r][j], sq[j], gq);
-    }
-  double g00 = wsum(sy[r] * gy), g01 = wsum(sy[r] * gq), g11 = wsum(sq[r] * gq);
-  double g10 = wsum(sq[r] * gy);
-  if (r < m) yp[(int64_t)b * M + r] = sq[r];
-  if (r == 0) {
-    double* Gb = G + (int64_t)b * M * M;
-    double off = 0.5 * (g01 + g10);
-    Gb[0] = g00;
-    Gb[1] = off;
-    Gb[M] = off;
-    Gb[M + 1] = g11;
+  for (int i = ty; i < 32; i += ny) {
+    const int r = J * 32 + i, k = I * 32 + tx;
+    if (r < nstr && k < nstr && (I < J || r > k)) Cb[(int64_t)r * nstr + k] = sC[tx][i];
   }
 }
 
-// In place: V_0 = V y, V_1 = V q, AV_0 = AV y, AV_1 = AV q (q in yp)
-__global__ void k_restart_vec(double* __restrict__ V, double* __restrict__ AV, int m, int M,
-                              int64_t N, const double* __restrict__ y, const double* __restrict__ q,
+// open shell: V[m] = T / |T|
+__global__ void k_append_full(const double* __restrict__ T, double* __restrict__ V, int64_t vstride,
+                              int64_t L, const double* __restrict__ inv,
                               const int32_t* __restrict__ active) {
   const int b = blockIdx.y;
   if (!active[b]) return;
-  __shared__ double sy[32], sq[32];
-  if (threadIdx.x < m) {
-    sy[threadIdx.x] = y[(int64_t)b * M + threadIdx.x];
-    sq[threadIdx.x] = q[(int64_t)b * M + threadIdx.x];
-  }
-  __syncthreads();
-  double* Vb = V + (int64_t)b * M * N;
-  double* AVb = AV + (int64_t)b * M * N;
+  const double f = inv[b];
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < L;
+       k += (int64_t)gridDim.x * blockDim.x)
+    V[(int64_t)b * vstride + k] = T[(int64_t)b * L + k] * f;
+}
+
+// packed V (stride vstride) from full symmetric vectors C; mask may be NULL
+__global__ void k_pack(const double* __restrict__ C, int nstr, const int32_t* __restrict__ mask,
+                       double* __restrict__ V, int64_t vstride) {
+  const int b = blockIdx.y;
+  if (mask && !mask[b]) return;
+  const int64_t N = (int64_t)nstr * nstr;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N;
        k += (int64_t)gridDim.x * blockDim.x) {
-    double x = 0.0, xp = 0.0, ax = 0.0, axp = 0.0;
-    for (int i = 0; i < m; i++) {
-      double v = Vb[(int64_t)i * N + k], av = AVb[(int64_t)i * N + k];
-      x = fma(sy[i], v, x);
-      xp = fma(sq[i], v, xp);
-      ax = fma(sy[i], av, ax);
-      axp = fma(sq[i], av, axp);
-    }
-    Vb[k] = x;
-    Vb[N + k] = xp;
-    AVb[k] = ax;
-    AVb[N + k] = axp;
+    const int ia = (int)(k / nstr), ib = (int)(k - (int64_t)ia * nstr);
+    if (ia <= ib) V[(int64_t)b * vstride + sym_index(ia, ib, nstr)] = C[(int64_t)b * N + k];
   }
 }
 
-// y_prev <- y (zero padded), or e_0 right after a restart
-__global__ void k_save_yprev(const double* __restrict__ y, int m, int M, int restarted,
-                             const int32_t* __restrict__ active, double* __restrict__ yp) {
-  const int b = blockIdx.x;
-  if (!active[b]) return;
-  for (int i = threadIdx.x; i < M; i += blockDim.x)
-    yp[(int64_t)b * M + i] = restarted ? (i == 0 ? 1.0 : 0.0) : (i < m ? y[(int64_t)b * M + i] : 0.0);
-}
-
-// t = r / (theta - H_II), then (closed shell, nstrb < 0) t <- (t + t^T)/2
-// so that every subspace vector stays exactly in the alpha<->beta symmetric
-// (even-S) sector; each thread owns the pair (Ia,Ib), (Ib,Ia) with Ia <= Ib.
-// A high-spin space (nstrb >= 0 beta strings) has no such symmetry.
-__global__ void k_precondition(double* __restrict__ T, const double* __restrict__ hd, int nstr,
-                               int nstrb, const double* __restrict__ theta,
-                               const int32_t* __restrict__ active) {
+// full X (stride N) from open-shell vectors of stride L
+__global__ void k_unpad(const double* __restrict__ V, int64_t L, int64_t N, double* __restrict__ X) {
   const int b = blockIdx.y;
-  if (!active[b]) return;
-  const double th = theta[b];
-  const int64_t N = (int64_t)nstr * (nstrb < 0 ? nstr : nstrb);
-  double* Tb = T + (int64_t)b * N;
-  const double* hb = hd + (int64_t)b * N;
-  if (nstrb >= 0) {
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N;
-         k += (int64_t)gridDim.x * blockDim.x) {
-      double d = th - hb[k];
-      if (fabs(d) < 1e-8) d = d < 0.0 ? -1e-8 : 1e-8;
-      Tb[k] = Tb[k] / d;
-    }
-    return;
-  }
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    const int ia = (int)(k / nstr), ib = (int)(k % nstr);
-    if (ia > ib) continue;
-    const int64_t kt = (int64_t)ib * nstr + ia;
-    double d1 = th - hb[k], d2 = th - hb[kt];
-    if (fabs(d1) < 1e-8) d1 = d1 < 0.0 ? -1e-8 : 1e-8;
-    if (fabs(d2) < 1e-8) d2 = d2 < 0.0 ? -1e-8 : 1e-8;
-    const double t = 0.5 * (Tb[k] / d1 + Tb[kt] / d2);
-    Tb[k] = t;
-    Tb[kt] = t;
-  }
-}
-
-// T -= sum_i coef[i] V[i]
-__global__ void k_orth_axpy(double* __restrict__ T, const double* __restrict__ V, int m, int M,
-                            int64_t N, const double* __restrict__ coef,
-                            const int32_t* __restrict__ active) {
-  const int b = blockIdx.y;
-  if (!active[b]) return;
-  __shared__ double sc[32];
-  if (threadIdx.x < m) sc[threadIdx.x] = coef[(int64_t)b * M + threadIdx.x];
-  __syncthreads();
-  const double* Vb = V + (int64_t)b * M * N;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N;
-       k += (int64_t)gridDim.x * blockDim.x) {
-    double t = T[(int64_t)b * N + k];
-    for (int i = 0; i < m; i++) t = fma(-sc[i], Vb[(int64_t)i * N + k], t);
-    T[(int64_t)b * N + k] = t;
-  }
-}
-
-// V[m] = T / ||T||; a tuple whose correction vanished is marked converged
-__global__ void k_append(const double* __restrict__ T, double* __restrict__ V, int m, int M,
-                         int64_t N, const double* __restrict__ nrm2, int32_t* __restrict__ active) {
-  const int b = blockIdx.y;
-  if (!active[b]) return;
-  double n2 = nrm2[(int64_t)b * M];
-  if (!(n2 > 1e-28)) {
-    __syncthreads();
-    if (blockIdx.x == 0 && threadIdx.x == 0) active[b] = 2;   // frozen after this pass
-    return;
-  }
-  double inv = 1.0 / sqrt(n2);
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < N;
        k += (int64_t)gridDim.x * blockDim.x)
-    V[(int64_t)b * M * N + (int64_t)m * N + k] = T[(int64_t)b * N + k] * inv;
-}
-
-__global__ void k_fix_frozen(int32_t* active, int B) {
-  for (int b = threadIdx.x; b < B; b += blockDim.x)
-    if (active[b] == 2) active[b] = 0;
+    X[(int64_t)b * N + k] = V[(int64_t)b * L + k];
 }
 
 // start vector: lowest diagonal determinant (Ia, Ib), symmetrised for a
-// closed shell (nstrb < 0); for a high-spin space (nstrb beta strings) the
-// determinant itself
-__global__ void k_guess(const double* __restrict__ hd, int nstr, int nstrb, int M,
-                        double* __restrict__ V) {
+// closed shell (packed vectors); for an open shell (nstrb beta strings) the
+// determinant itself.  V_0 is zero on entry.
+__global__ void k_guess(const double* __restrict__ hd, int nstr, int nstrb, int closed, int64_t L,
+                        int64_t vstride, double* __restrict__ V) {
   const int b = blockIdx.x;
-  const int64_t N = (int64_t)nstr * (nstrb < 0 ? nstr : nstrb);
+  const int64_t N = (int64_t)nstr * nstrb;
   __shared__ double sv[256];
   __shared__ int64_t si[256];
   double best = 1e300;
   int64_t bi = 0;
   for (int64_t k = threadIdx.x; k < N; k += blockDim.x) {
-    double v = hd[(int64_t)b * N + k];
+    const int ia = (int)(k / nstrb), ib = (int)(k - (int64_t)ia * nstrb);
+    if (closed && ia > ib) continue;   // the mirror element has the same value, a larger k
+    const double v = hd[(int64_t)b * L + (closed ? sym_index(ia, ib, nstr) : k)];
     if (v < best) { best = v; bi = k; }
   }
   sv[threadIdx.x] = best;
@@ -364,8 +119,8 @@ __global__ void k_guess(const double* __restrict__ hd, int nstr, int nstrb, int 
   __syncthreads();
   for (int s = blockDim.x / 2; s; s >>= 1) {
     if (threadIdx.x < s) {
-      double o = sv[threadIdx.x + s];
-      int64_t oi = si[threadIdx.x + s];
+      const double o = sv[threadIdx.x + s];
+      const int64_t oi = si[threadIdx.x + s];
       if (o < sv[threadIdx.x] || (o == sv[threadIdx.x] && oi < si[threadIdx.x])) {
         sv[threadIdx.x] = o;
         si[threadIdx.x] = oi;
@@ -373,47 +128,17 @@ __global__ void k_guess(const double* __restrict__ hd, int nstr, int nstrb, int 
     }
     __syncthreads();
   }
-  double* Vb = V + (int64_t)b * M * N;
-  for (int64_t k = threadIdx.x; k < N; k += blockDim.x) Vb[k] = 0.0;
-  __syncthreads();
   if (threadIdx.x == 0) {
-    int64_t i0 = si[0];
-    int ia = (int)(i0 / nstr), ib = (int)(i0 % nstr);
-    if (nstrb >= 0 || ia == ib) Vb[i0] = 1.0;
-    else {
-      Vb[(int64_t)ia * nstr + ib] = sqrt(0.5);
-      Vb[(int64_t)ib * nstr + ia] = sqrt(0.5);
-    }
+    const int64_t i0 = si[0];
+    const int ia = (int)(i0 / nstrb), ib = (int)(i0 % nstrb);
+    double* Vb = V + (int64_t)b * vstride;
+    // (|a b> + |b a>) / sqrt(2): its packed element carries both halves
+    if (closed) Vb[sym_index(ia, ib, nstr)] = ia == ib ? 1.0 : sqrt(0.5);
+    else Vb[i0] = 1.0;
   }
-}
-
-__global__ void k_fill(double* __restrict__ v, int n, double x) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] = x;
-}
-
-__global__ void k_set_i32(int32_t* __restrict__ v, int n, int32_t x) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) v[i] = x;
 }
 
 }  // namespace
-
-struct Multidot {
-  DevBuf<double> partial;
-  int nchunks = 0;
-  // out[b*out_bstride + i*out_istride] = X[b][i] . Y[b], i < m
-  void run(mbe_ctx* ctx, const double* X, int64_t xb, int64_t xv, const double* Y, int64_t yb,
-           int m, int64_t N, int B, const int32_t* active, double* out, int64_t ob, int64_t oi) {
-    nchunks = (int)((N + DOT_CHUNK - 1) / DOT_CHUNK);
-    size_t need = (size_t)B * m * nchunks;
-    if (partial.n < need) partial.reset(&ctx->pool, need);
-    dim3 g(nchunks, B);
-    k_multidot_partial<<<g, 256, 0, ctx->stream>>>(X, xb, xv, Y, yb, m, N, nchunks, active,
-                                                   partial.ptr);
-    CU_LAUNCH_CHECK();
-    k_multidot_final<<<B, 32, 0, ctx->stream>>>(partial.ptr, m, nchunks, active, out, ob, oi);
-    CU_LAUNCH_CHECK();
-  }
-};
 
 // Davidson for one batch of tuples: one stage with FP64 (or emulated-FP64)
 // sigma vectors to conv_tol_r / conv_tol_e.
@@ -422,68 +147,147 @@ void davidson_batch(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int32_t* s
   const int B = bp.B;
   const int M = std::max(4, std::min(32, ctx->opt.max_subspace));
   const int64_t N = bp.ndet;
+  const bool closed = bp.closed();
+  const int64_t L = closed ? sym_len(bp.nstr) : (N + 3) & ~(int64_t)3;
+  const int64_t nd = closed ? sym_nd(bp.nstr) : L;
+  const int64_t vs = (int64_t)M * L;   // stride of a tuple's subspace
   const double shift = ctx->opt.spin_shift;
   DevPool* P = &ctx->pool;
-  DevBuf<double> V(P, (size_t)B * M * N), AV(P, (size_t)B * M * N), hd(P, (size_t)B * N),
-      T(P, (size_t)B * N), Xown(P, x_out_dev ? 0 : (size_t)B * N), G(P, (size_t)B * M * M),
-      y(P, (size_t)B * M), yp(P, (size_t)B * M), theta(P, B), theta_old(P, B), rnorm(P, B),
-      tolr(P, B), coef(P, (size_t)B * M), xx(P, (size_t)B * M),
-      rpart(P, (size_t)B * ((N + DOT_CHUNK - 1) / DOT_CHUNK));
-  DevBuf<int32_t> active(P, B), iters(P, B), nact(P, 1);
-  double* X = x_out_dev ? x_out_dev : Xown.ptr;
-  SigmaWork sw;
-  Multidot md;
   cudaStream_t st = ctx->stream;
   // sigma vectors: FP64 CUDA cores (MBE_FP64) or the FP64-grade sliced
   // tensor-core contraction (MBE_EMULATED_FP64, and the mixed mode's
   // fallback for spaces the fused tensor-core kernel does not cover)
   const bool emulated = ctx->opt.precision != MBE_FP64 && ozaki_supported(bp.npair);
+  int nsm = 0;
+  CU_CHECK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device));
+  const int ch = chunk_of(L, B, nsm, 4);
+  const int nchunks = (int)((L + ch - 1) / ch), nchunks_f = (int)((N + ch - 1) / ch);
+  DevBuf<double> V(P, (size_t)B * vs), AV(P, (size_t)B * vs), hd(P, (size_t)B * L),
+      T(P, (size_t)B * L), X(P, (size_t)B * L), C(P, (size_t)B * N),
+      SF(P, emulated && closed ? (size_t)B * N : 0), G(P, (size_t)B * M * M), y(P, (size_t)B * M),
+      yp(P, (size_t)B * M), theta(P, B), theta_old(P, B), rnorm(P, B), tolr(P, B),
+      coef(P, (size_t)B * M), inv(P, B), xs2(P, B), xx(P, B),
+      partial(P, (size_t)B * (M + 2) * nchunks),
+      rpart(P, (size_t)B * std::max(nchunks, nchunks_f));
+  DevBuf<float> Z(P, (size_t)B * 1024);
+  DevBuf<int32_t> active(P, B), iters(P, B), nact(P, 1), cnt(P, B);
+  SigmaWork sw;
+  set_attributes<double>(ctx->device);
 
-  launch_hdiag(ctx, bp, shift, hd.ptr);
-  const int nstrb_arg = bp.closed() ? -1 : bp.nstrb;
-  k_guess<<<B, 256, 0, st>>>(hd.ptr, bp.nstr, nstrb_arg, M, V.ptr);
-  CU_LAUNCH_CHECK();
-  if (plan) launch_parent_guess(ctx, *plan, bp.n, bp.nsig, bp.nstr, nullptr, V.ptr, (int64_t)M * N);
-  k_set_i32<<<1, 256, 0, st>>>(active.ptr, B, 1);
-  CU_LAUNCH_CHECK();
+  // zero padding: no kernel writes it, the streaming kernels read it
+  CU_CHECK(cudaMemsetAsync(V.ptr, 0, sizeof(double) * B * vs, st));
+  CU_CHECK(cudaMemsetAsync(AV.ptr, 0, sizeof(double) * B * vs, st));
+  CU_CHECK(cudaMemsetAsync(hd.ptr, 0, sizeof(double) * B * L, st));
   CU_CHECK(cudaMemsetAsync(iters.ptr, 0, sizeof(int32_t) * B, st));
+  CU_CHECK(cudaMemsetAsync(cnt.ptr, 0, sizeof(int32_t) * B, st));
   CU_CHECK(cudaMemsetAsync(G.ptr, 0, sizeof(double) * B * M * M, st));
-  k_fill<<<1, 256, 0, st>>>(tolr.ptr, B, ctx->opt.conv_tol_r);
+  launch_hdiag(ctx, bp, shift, hd.ptr, L, closed);
+  k_guess<<<B, 256, 0, st>>>(hd.ptr, bp.nstr, bp.nstrb, closed ? 1 : 0, L, vs, V.ptr);
   CU_LAUNCH_CHECK();
-
-  int64_t eblocks = std::min<int64_t>((N + 255) / 256, 1024);
-  dim3 ge((unsigned)eblocks, B);
-  const int nchunks = (int)((N + DOT_CHUNK - 1) / DOT_CHUNK);
-  dim3 gc(nchunks, B);
-  const int max_iter = std::max(1, ctx->opt.max_iter);
-  int64_t vecs_tc = 0, vecs_64 = 0;
-  int total_it = 0;
-
-  auto sigma = [&](bool /*unused*/, const double* c, double* out) {
-    if (emulated)
-      sigma_emulated(ctx, bp, sw, c, (int64_t)M * N, out, (int64_t)M * N, active.ptr, shift, true);
-    else
-      sigma_direct(ctx, bp, c, (int64_t)M * N, out, (int64_t)M * N, active.ptr, shift, true);
-  };
-  // precondition the residual in T, orthogonalise it against V[0..m) and
-  // append it as V[m] (tuples whose correction vanished are frozen)
-  auto extend = [&](int m) {
-    k_precondition<<<ge, 256, 0, st>>>(T.ptr, hd.ptr, bp.nstr, nstrb_arg, theta.ptr, active.ptr);
+  const dim3 gN((unsigned)std::min<int64_t>((N + 255) / 256, 1024), B);
+  const dim3 gL((unsigned)std::min<int64_t>((L + 255) / 256, 1024), B);
+  if (plan) {
+    // the parent guess writes full vectors, packed into V_0 here
+    launch_parent_guess(ctx, *plan, bp.n, bp.nsig, bp.nstr, nullptr, C.ptr, N);
+    std::vector<int32_t> pm(B, 0);
+    for (int b : plan->b) pm[b] = 1;
+    DevBuf<int32_t> pmask(P, B);
+    CU_CHECK(cudaMemcpyAsync(pmask.ptr, pm.data(), sizeof(int32_t) * B, cudaMemcpyHostToDevice, st));
+    k_pack<<<gN, 256, 0, st>>>(C.ptr, bp.nstr, pmask.ptr, V.ptr, vs);
     CU_LAUNCH_CHECK();
-    for (int pass = 0; pass < 2; pass++) {
-      md.run(ctx, V.ptr, (int64_t)M * N, N, T.ptr, N, m, N, B, active.ptr, coef.ptr, M, 1);
-      k_orth_axpy<<<ge, 256, 0, st>>>(T.ptr, V.ptr, m, M, N, coef.ptr, active.ptr);
+    CU_CHECK(cudaStreamSynchronize(st));   // pm is read by the copy above
+  }
+  k_fill_i<<<1, 256, 0, st>>>(active.ptr, B, 1);
+  CU_LAUNCH_CHECK();
+  k_fill_d<<<1, 256, 0, st>>>(tolr.ptr, B, ctx->opt.conv_tol_r);
+  CU_LAUNCH_CHECK();
+  if (!emulated) sigma_direct_prepare(ctx, bp);
+
+  const int nt = (bp.nstr + 31) / 32;
+  const dim3 gt((unsigned)(nt * (nt + 1) / 2), B), gc(nchunks, B);
+  const int max_iter = std::max(1, ctx->opt.max_iter);
+  int64_t vecs = 0;
+  Converge cv = {tolr.ptr, ctx->opt.conv_tol_e, 0,          1,        theta_old.ptr,
+                 rnorm.ptr, active.ptr,         iters.ptr, nact.ptr};
+
+  // V[m-1] (from T unless it is the start vector) and its sigma vector, the
+  // subspace row and Ritz step, the residual and its correction in T
+  auto head = [&](int m, bool append, bool warm, bool first) {
+    double* Vm = V.ptr + (int64_t)(m - 1) * L;
+    double* AVm = AV.ptr + (int64_t)(m - 1) * L;
+    if (closed) {
+      k_append_sym<<<gt, 256, 0, st>>>(T.ptr, Vm, vs, L, append ? inv.ptr : nullptr, bp.nstr,
+                                       append ? active.ptr : nullptr, C.ptr);
+      CU_LAUNCH_CHECK();
+    } else if (append) {
+      k_append_full<<<gL, 256, 0, st>>>(T.ptr, Vm, vs, L, inv.ptr, active.ptr);
       CU_LAUNCH_CHECK();
     }
-    md.run(ctx, T.ptr, N, 0, T.ptr, N, 1, N, B, active.ptr, coef.ptr, M, 1);
-    k_append<<<ge, 256, 0, st>>>(T.ptr, V.ptr, m, M, N, coef.ptr, active.ptr);
+    if (!emulated) {
+      sigma_direct(ctx, bp, closed ? C.ptr : Vm, closed ? N : vs, AVm, vs, active.ptr, shift, closed);
+    } else if (closed) {
+      sigma_emulated(ctx, bp, sw, C.ptr, N, SF.ptr, N, active.ptr, shift, true);
+      k_pack<<<gN, 256, 0, st>>>(SF.ptr, bp.nstr, active.ptr, AVm, vs);
+      CU_LAUNCH_CHECK();
+    } else {
+      sigma_emulated(ctx, bp, sw, Vm, vs, AVm, vs, active.ptr, shift, false);
+    }
+    k_subspace<double><<<gc, RT, subspace_smem<double>(m), st>>>(
+        V.ptr, AV.ptr, L, nd, m, M, ch, nchunks, active.ptr, partial.ptr, cnt.ptr, 0, nullptr,
+        nullptr, G.ptr, Z.ptr, warm ? 1 : 0, theta.ptr, y.ptr, nact.ptr);
     CU_LAUNCH_CHECK();
-    k_fix_frozen<<<1, 256, 0, st>>>(active.ptr, B);
+    cv.first = first ? 1 : 0;
+    // (a restart follows a full subspace and needs the previous y)
+    k_residual<double><<<gc, RT, (size_t)m * RT * sizeof(double), st>>>(
+        V.ptr, AV.ptr, nullptr, 0, m, M, L, nd, y.ptr, theta.ptr, nullptr, hd.ptr, X.ptr, T.ptr, ch,
+        nchunks, rpart.ptr, partial.ptr, 0, nullptr, nullptr, nullptr, 1e-8, cnt.ptr, cv, coef.ptr,
+        m == M ? nullptr : yp.ptr);
     CU_LAUNCH_CHECK();
   };
-  auto count_active = [&]() {
-    int32_t n = 0;
-    CU_CHECK(cudaMemcpyAsync(&n, nact.ptr, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  // orthogonalise the correction T against V[0..m); after a full subspace
+  // restart with {x, x_prev} first
+  auto tail = [&](int m, bool restart) {
+    if (restart) {
+      k_restart_coef<<<B, 32, 0, st>>>(y.ptr, yp.ptr, m, M, active.ptr, G.ptr);
+      CU_LAUNCH_CHECK();
+      k_restart_vec<double><<<gL, 256, 0, st>>>(V.ptr, AV.ptr, m, M, L, y.ptr, yp.ptr, active.ptr);
+      CU_LAUNCH_CHECK();
+      k_restart_yprev<<<B, 32, 0, st>>>(yp.ptr, M, active.ptr);
+      CU_LAUNCH_CHECK();
+      m = 2;
+      // V changed: the first pass's dots are taken again
+      k_dots<double><<<gc, RT, (size_t)m * RT * sizeof(double), st>>>(
+          V.ptr, vs, L, T.ptr, L, m, M, L, nd, ch, nchunks, active.ptr, partial.ptr, cnt.ptr,
+          coef.ptr);
+      CU_LAUNCH_CHECK();
+    }
+    for (int pass = 0; pass < 2; pass++) {
+      k_orth<double><<<gc, RT, pass ? 0 : (size_t)m * RT * sizeof(double), st>>>(
+          T.ptr, V.ptr, m, M, L, nd, coef.ptr, active.ptr, pass, ch, nchunks, partial.ptr, nullptr,
+          nullptr, cnt.ptr, inv.ptr, 1e-28);
+      CU_LAUNCH_CHECK();
+    }
+  };
+  // Each iteration's tail is issued together with the next one's head, as one
+  // CUDA graph (opt.graphs; the emulated sigma stages host data and runs
+  // plain, as does the legacy default stream, which cannot be captured); one
+  // synchronisation per iteration, for the number of tuples still iterating.
+  const bool use_graphs =
+      ctx->opt.graphs != 0 && !emulated && st != nullptr && st != cudaStreamLegacy;
+  GraphRunner gr(st);
+  int m = 1, m_tail = 0, nact_h = B;
+  bool restart = false;
+  for (int it = 0; it < max_iter; it++) {
+    const int mt = m_tail, mc = m;
+    const bool rs = restart, pend = it > 0;
+    auto body = [&] {
+      if (pend) tail(mt, rs);
+      head(mc, pend, pend && !rs, it == 0);
+    };
+    if (use_graphs && it >= 1) gr.run(rs ? 1 : 0, body);
+    else body();
+    vecs += nact_h;
+    CU_CHECK(cudaMemcpyAsync(&nact_h, nact.ptr, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     CU_CHECK(cudaStreamSynchronize(st));
     if (ctx->opt.verbose) {
       std::vector<double> rn(B), th(B);
@@ -492,60 +296,13 @@ void davidson_batch(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int32_t* s
       double mx = 0.0;
       for (double r : rn) mx = std::max(mx, r);
       fprintf(stderr, "[mbe davidson] n=%d nsig=%d B=%d it=%d active=%d max|r|=%.3e theta0=%.12f\n",
-              bp.n, bp.nsig, B, total_it, n, mx, th[0]);
+              bp.n, bp.nsig, B, it, nact_h, mx, th[0]);
     }
-    return n;
-  };
-
-  // One stage of Davidson iterations from the current (V, AV, G): the
-  // subspace holds m_start vectors and the newest one's sigma is pending.
-  // exact0: V_0 carries an exact (FP64) A V_0; its couplings G_0j are then
-  // taken as (A V_0).V_j, which involves no reduced-precision sigma, and the
-  // stage ends before a restart would replace V_0.
-  auto stage = [&](bool use_tc, double tol_e, int rel, int m_start, int cap, int nact0,
-                   bool exact0) {
-    int m = m_start;
-    int nact_h = nact0;
-    for (int it = 0; it < cap && total_it < max_iter; it++, total_it++) {
-      sigma(use_tc, V.ptr + (int64_t)(m - 1) * N, AV.ptr + (int64_t)(m - 1) * N);
-      (use_tc ? vecs_tc : vecs_64) += nact_h;
-      md.run(ctx, V.ptr, (int64_t)M * N, N, AV.ptr + (int64_t)(m - 1) * N, (int64_t)M * N, m, N,
-             B, active.ptr, coef.ptr, M, 1);
-      if (exact0) {
-        md.run(ctx, AV.ptr, (int64_t)M * N, 0, V.ptr + (int64_t)(m - 1) * N, (int64_t)M * N, 1, N,
-               B, active.ptr, coef.ptr, M, 1);
-      }
-      k_store_grow<<<B, 32, 0, st>>>(coef.ptr, m, M, active.ptr, G.ptr);
-      CU_LAUNCH_CHECK();
-      k_jacobi<<<B, 32, 0, st>>>(G.ptr, m, M, active.ptr, theta.ptr, y.ptr);
-      CU_LAUNCH_CHECK();
-      k_residual<<<gc, 256, 0, st>>>(V.ptr, AV.ptr, m, M, N, y.ptr, theta.ptr, active.ptr, X,
-                                     T.ptr, nchunks, rpart.ptr);
-      CU_LAUNCH_CHECK();
-      k_converge<<<1, 256, 0, st>>>(rpart.ptr, nchunks, B, m_start > 1 ? it + 1 : it, tolr.ptr,
-                                    tol_e, rel, theta.ptr, theta_old.ptr, rnorm.ptr, active.ptr,
-                                    iters.ptr, nact.ptr);
-      CU_LAUNCH_CHECK();
-      nact_h = count_active();
-      if (nact_h == 0) return;
-      if (exact0 && m == M) return;   // the next exact point restarts
-      int restarted = 0;
-      if (m == M) {   // restart with {x, x_prev}
-        k_restart_coef<<<B, 32, 0, st>>>(y.ptr, yp.ptr, m, M, active.ptr, G.ptr);
-        CU_LAUNCH_CHECK();
-        k_restart_vec<<<ge, 256, 0, st>>>(V.ptr, AV.ptr, m, M, N, y.ptr, yp.ptr, active.ptr);
-        CU_LAUNCH_CHECK();
-        m = 2;
-        restarted = 1;
-      }
-      k_save_yprev<<<B, 32, 0, st>>>(y.ptr, m, M, restarted, active.ptr, yp.ptr);
-      CU_LAUNCH_CHECK();
-      extend(m);
-      m++;
-    }
-  };
-
-  stage(false, ctx->opt.conv_tol_e, 0, 1, max_iter, B, false);
+    if (nact_h == 0) break;
+    restart = m == M;
+    m_tail = m;
+    m = (restart ? 2 : m) + 1;
+  }
   if (emulated && sigma_tc_error(ctx, sw))
     throw MbeError{MBE_ETIMEOUT, "tensor-core contraction wait timed out"};
 
@@ -554,12 +311,24 @@ void davidson_batch(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int32_t* s
   std::vector<double> rn_h(B);
   CU_CHECK(cudaMemcpyAsync(it_h.data(), iters.ptr, sizeof(int32_t) * B, cudaMemcpyDeviceToHost, st));
   CU_CHECK(cudaMemcpyAsync(rn_h.data(), rnorm.ptr, sizeof(double) * B, cudaMemcpyDeviceToHost, st));
-  s2_apply(ctx, bp, X, N, T.ptr, N, nullptr);
-  md.run(ctx, X, N, 0, T.ptr, N, 1, N, B, nullptr, coef.ptr, 1, 1);
-  md.run(ctx, X, N, 0, X, N, 1, N, B, nullptr, xx.ptr, 1, 1);
+  double* XF = x_out_dev ? x_out_dev : C.ptr;   // the converged vectors, full
+  if (closed) {
+    k_append_sym<<<gt, 256, 0, st>>>(nullptr, X.ptr, L, L, nullptr, bp.nstr, nullptr, XF);
+    CU_LAUNCH_CHECK();
+  } else {
+    k_unpad<<<gN, 256, 0, st>>>(X.ptr, L, N, XF);
+    CU_LAUNCH_CHECK();
+  }
+  double* S2X = V.ptr;   // the subspace is not needed any more (M >= 4 vectors of N / 2)
+  s2_apply(ctx, bp, XF, N, S2X, N, nullptr);
+  const dim3 gcf(nchunks_f, B);
+  k_dot64<<<gcf, RT, 0, st>>>(XF, S2X, N, ch, nchunks_f, nullptr, rpart.ptr, cnt.ptr, xs2.ptr);
+  CU_LAUNCH_CHECK();
+  k_dot64<<<gcf, RT, 0, st>>>(XF, XF, N, ch, nchunks_f, nullptr, rpart.ptr, cnt.ptr, xx.ptr);
+  CU_LAUNCH_CHECK();
   std::vector<double> th(B), s2(B), ec(B), nx(B);
   CU_CHECK(cudaMemcpyAsync(th.data(), theta.ptr, sizeof(double) * B, cudaMemcpyDeviceToHost, st));
-  CU_CHECK(cudaMemcpyAsync(s2.data(), coef.ptr, sizeof(double) * B, cudaMemcpyDeviceToHost, st));
+  CU_CHECK(cudaMemcpyAsync(s2.data(), xs2.ptr, sizeof(double) * B, cudaMemcpyDeviceToHost, st));
   CU_CHECK(cudaMemcpyAsync(nx.data(), xx.ptr, sizeof(double) * B, cudaMemcpyDeviceToHost, st));
   CU_CHECK(cudaMemcpyAsync(ec.data(), bp.ecore.ptr, sizeof(double) * B, cudaMemcpyDeviceToHost, st));
   CU_CHECK(cudaStreamSynchronize(st));
@@ -575,8 +344,10 @@ void davidson_batch(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int32_t* s
     ctx->stats.noconv += ok ? 0 : 1;
   }
   const double per = 2.0 * (double)N * bp.npair * bp.npair;
+  ctx->stats.graph_launches += gr.launched;
+  ctx->stats.graph_builds += gr.instantiated;
   ctx->stats.casci += B;
-  ctx->stats.sigma_vectors += vecs_tc + vecs_64;
-  ctx->stats.sigma_flops += (double)(vecs_tc + vecs_64) * per;
-  ctx->stats.fp64_flops += (double)(vecs_tc + vecs_64) * per;   // exact sigma vectors
+  ctx->stats.sigma_vectors += vecs;
+  ctx->stats.sigma_flops += (double)vecs * per;
+  ctx->stats.fp64_flops += (double)vecs * per;   // exact sigma vectors
 }

@@ -431,12 +431,15 @@ int pspace_size(const BinProblem& bp, int requested);
 // hd, T, V, Uo, X: one vector per tuple every ld elements
 void pspace_setup(mbe_ctx* ctx, BinProblem& bp, const float* hd, int64_t ld, double shift,
                   int npp, PspaceWork& w);
-// the P-space block of t (and with olsen of u = M^-1 x in Uo, X the Ritz
-// vector), correcting the partial dot products that the residual kernel left
+// the P-space block of the correction T (with olsen: and of u = M^-1 x in Uo,
+// X the Ritz vector) and what follows from the partial dots the residual
+// kernel left: coef = V.t - eps V.u (with dots) and Olsen's eps.  yp != NULL:
+// y_prev <- y
 void pspace_apply(mbe_ctx* ctx, const BinProblem& bp, const PspaceWork& w, float* T,
                   const float* hd, int64_t ld, const double* theta, const float* V, int m, int M,
-                  int nchunks, double* partial, bool fix_dots, const int32_t* active,
-                  bool olsen, float* Uo, const float* X, double* upart, double* xpart);
+                  int nchunks, const double* dpart, bool dots, const int32_t* active, bool olsen,
+                  float* Uo, const float* X, const double* upart, const double* xpart,
+                  const double* y, double* yp, double* coef, float* eps);
 
 // ------------------------------------------------------------ launchers
 void build_string_tables(mbe_ctx* ctx, StringTables* t);
@@ -476,7 +479,9 @@ int noalloc_sigma_run(mbe_ctx* ctx, const int* act, int nact, const double* c_de
 // energy gradient of the processed expansion (mbe_energy_backward)
 int backward_run(mbe_ctx* ctx, double scale, double* dh_host, double* deri_host);
 void launch_effints(mbe_ctx* ctx, BinProblem& bp);
-void launch_hdiag(mbe_ctx* ctx, BinProblem& bp, double spin_shift, double* hd);
+// packed: the diagonal in the packed symmetric layout; ld between tuples
+void launch_hdiag(mbe_ctx* ctx, BinProblem& bp, double spin_shift, double* hd, int64_t ld,
+                  bool packed);
 
 // sigma for a batch: out[b] = (H_act + shift S^2) c[b] for b < B; c/out with
 // strides (elements between consecutive tuples' vectors); active may be NULL.
@@ -492,10 +497,11 @@ struct SigmaWork {
 };
 bool sigma_tc_supported(int n, int nstr);
 // FP32 vectors in and out (c = c^T assumed: sigma = X + X^T)
-// packed: c and the result in the packed symmetric layout (sym_index)
-void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, const float* c, int64_t c_stride,
+// packed: c and the result in the packed symmetric layout (sym_index); then
+// with T (one vector every sym_len) and inv, c is first set to inv T
+void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, float* c, int64_t c_stride,
               float* out, int64_t out_stride, const int32_t* active, double spin_shift,
-              bool packed = false);
+              bool packed = false, const float* T = nullptr, const double* inv = nullptr);
 int32_t sigma_tc_error(mbe_ctx* ctx, SigmaWork& w);
 // subspace vectors allocated per tuple by the mixed Davidson: max_subspace
 // (clamped to 4..32) for its first stage and its refinement rounds, up to 12
@@ -512,13 +518,14 @@ void convert_f64_to_f32(mbe_ctx* ctx, const double* src, float* dst, int64_t n);
 // with their parents' vectors (exactly one of V32 / V64 non-null)
 void launch_parent_guess(mbe_ctx* ctx, const GuessPlan& plan, int n, int nsig, int nstr,
                          float* V32, double* V64, int64_t vstride);
-// symmetric: c(a,b) = c(b,a) for every tuple; otherwise any c
-// FP64 on the CUDA cores:
+// FP64 on the CUDA cores (symmetric: c(a,b) = c(b,a) for every tuple and the
+// result in the packed layout; otherwise any c and the full result):
 void sigma_direct(mbe_ctx* ctx, BinProblem& bp, const double* c, int64_t c_stride, double* out,
                   int64_t out_stride, const int32_t* active, double spin_shift, bool symmetric);
 // its tables and values (sigma_direct makes them on its first call otherwise)
 void sigma_direct_prepare(mbe_ctx* ctx, BinProblem& bp);
-// FP64-grade: gather, sliced tensor-core GEMM, scatter
+// FP64-grade: gather, sliced tensor-core GEMM, scatter (symmetric: c(a,b) =
+// c(b,a), full vectors)
 void sigma_emulated(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, const double* c,
                     int64_t c_stride, double* out, int64_t out_stride,
                     const int32_t* active, double spin_shift, bool symmetric = false);

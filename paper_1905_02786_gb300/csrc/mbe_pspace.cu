@@ -20,9 +20,10 @@
 // per iteration:
 //   k_psp_apply   t_P = U (theta - Lambda)^{-1} U^T r_P (r_P recovered from
 //                 the diagonal correction as t_I (theta - A_II)), written
-//                 back into the packed vector, and the first Gram-Schmidt pass's
-//                 dot products corrected for the changed elements; the same
-//                 for M^-1 x, x the Ritz vector.
+//                 back into the packed vector; the same for M^-1 x, x the
+//                 Ritz vector; and the first Gram-Schmidt pass's
+//                 coefficients from the residual kernel's partial dots and
+//                 the changed elements.
 // With an exact block M^-1 r = -x on P whenever x lies in P and does not
 // couple out of it (the lowest-diagonal start vector of a small space does),
 // which the orthogonalisation removes, so the Davidson iteration takes
@@ -39,7 +40,7 @@ constexpr int PSP_MAX = 128;
 constexpr int PSP_PITCH = PSP_MAX + 1;   // row pitch of the shared matrices
 constexpr int SEL_THREADS = 1024;
 constexpr int EIG_THREADS = 1024;
-constexpr int APPLY_THREADS = 256;
+constexpr int APPLY_THREADS = 4 * PSP_MAX;
 constexpr int EIG_SWEEPS = 10;
 
 // FP32 bit pattern mapped to an unsigned key with the same order
@@ -383,123 +384,148 @@ __global__ void __launch_bounds__(EIG_THREADS)
   }
 }
 
-// t_P = U (theta - Lambda)^{-1} U^T r_P for the tuples still iterating; with
-// fix_dots the first Gram-Schmidt pass's partial dot products (chunk 0 of
-// `partial`) take the change of t.  With olsen the same block solve turns
-// u = x / (theta - A_II) (Uo, from the residual kernel) into M^-1 x on P,
-// and the partial sums x.t, x.u (xpart) and, with fix_dots, V.u (upart)
-// take their changes.
+// What an iteration does between the residual and the Gram-Schmidt passes,
+// one CTA per tuple still iterating:
+//   t_P = U (theta - Lambda)^{-1} U^T r_P (npp = 0: no P-space);
+//   with olsen the same block solve turns u = x / (theta - A_II) (Uo, from the
+//   residual kernel) into M^-1 x on P;
+//   the dots x.t, x.u (xpart) and, with dots, V.t (dpart) and V.u (upart) are
+//   summed over their chunks, with the changes of t and u on P;
+//   Olsen's eps = x.t / x.u and the first Gram-Schmidt pass's coefficients
+//   coef = V.t - eps V.u.
+// U comes from L2 twice (by columns for U^T r, by rows for U w), a quarter of
+// a column or a warp per row; the whole is a latency chain of a few thousand
+// cycles (one warp-wide pass over U in shared memory and four more kernels
+// for the sums took 40 us and four launches).
 __global__ void __launch_bounds__(APPLY_THREADS)
     k_psp_apply(float* __restrict__ T, const float* __restrict__ hd_all, int nstr, int64_t ld,
                 const double* __restrict__ theta, int npp, const int32_t* __restrict__ psel,
                 const float* __restrict__ U_all, const float* __restrict__ lam_all,
                 const float* __restrict__ V, int m, int M, int nchunks,
-                double* __restrict__ partial, int fix_dots, const int32_t* __restrict__ active,
+                const double* __restrict__ dpart, int dots, const int32_t* __restrict__ active,
                 int olsen, float* __restrict__ Uo, const float* __restrict__ X,
-                double* __restrict__ upart, double* __restrict__ xpart) {
+                const double* __restrict__ upart, const double* __restrict__ xpart,
+                const double* __restrict__ y, double* __restrict__ yp, double* __restrict__ coef,
+                float* __restrict__ eps) {
   const int b = blockIdx.x;
   if (!active[b]) return;
-  extern __shared__ __align__(16) unsigned char smem[];
-  float* sU = (float*)smem;   // npp x npp, pitch PSP_PITCH
   __shared__ float s_r[PSP_MAX], s_x[PSP_MAX], s_w[PSP_MAX], s_wx[PSP_MAX];
   __shared__ float s_del[PSP_MAX], s_delu[PSP_MAX], s_xv[PSP_MAX];
+  __shared__ float s_pr[4][PSP_MAX], s_px[4][PSP_MAX];
   __shared__ int s_i[PSP_MAX];
-  const int tid = threadIdx.x;
-  float* Tb = T + (int64_t)b * ld;
-  float* Ob = olsen ? Uo + (int64_t)b * ld : nullptr;
-  const float* Xb = olsen ? X + (int64_t)b * ld : nullptr;
-  const float* hb = hd_all + (int64_t)b * ld;
-  const float th = (float)theta[b];
-  const float* Ub = U_all + (int64_t)b * PSP_MAX * PSP_MAX;
-  for (int t = tid; t < npp * npp; t += blockDim.x) {
-    const int u = t / npp, k = t - u * npp;
-    sU[u * PSP_PITCH + k] = Ub[u * PSP_MAX + k];
-  }
-  const float sq2 = 1.41421356237309505f, r2 = 0.70710678118654752f;
-  for (int u = tid; u < npp; u += blockDim.x) {
-    const int i0 = psel[(int64_t)b * PSP_MAX + u];
-    const int a = i0 / nstr, c = i0 - a * nstr;
-    const int i = (int)sym_index(a, c, nstr);          // packed position
-    // the diagonal correction's denominator, exactly as the residual kernel
-    float d = th - hb[i];
-    if (fabsf(d) < 1e-4f) d = d < 0.f ? -1e-4f : 1e-4f;
-    const float r = Tb[i] * d;
-    s_r[u] = a == c ? r : sq2 * r;
-    if (olsen) {
-      const float x = Xb[i];
+  __shared__ double s_c[32], s_c2[32], s_xs[2];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int NW = APPLY_THREADS / 32;
+  if (yp)
+    for (int i = tid; i < M; i += APPLY_THREADS)
+      yp[(int64_t)b * M + i] = i < m ? y[(int64_t)b * M + i] : 0.0;
+  if (npp) {
+    float* Tb = T + (int64_t)b * ld;
+    float* Ob = olsen ? Uo + (int64_t)b * ld : nullptr;
+    const float* Xb = olsen ? X + (int64_t)b * ld : nullptr;
+    const float* hb = hd_all + (int64_t)b * ld;
+    const float* Ub = U_all + (int64_t)b * PSP_MAX * PSP_MAX;
+    const float th = (float)theta[b];
+    const float sq2 = 1.41421356237309505f, r2 = 0.70710678118654752f;
+    if (tid < npp) {
+      const int u = tid;
+      const int i0 = psel[(int64_t)b * PSP_MAX + u];
+      const int a = i0 / nstr, c = i0 - a * nstr;
+      const int i = (int)sym_index(a, c, nstr);          // packed position
+      // the diagonal correction's denominator, exactly as the residual kernel
+      float d = th - hb[i];
+      if (fabsf(d) < 1e-4f) d = d < 0.f ? -1e-4f : 1e-4f;
+      const float r = Tb[i] * d;
+      s_r[u] = a == c ? r : sq2 * r;
+      const float x = olsen ? Xb[i] : 0.f;
       s_xv[u] = x;
       s_x[u] = a == c ? x : sq2 * x;
+      s_i[u] = i;
     }
-    s_i[u] = i;
+    __syncthreads();
+    {
+      // U^T r: thread -> column k and a quarter of the rows u
+      const int k = tid & (PSP_MAX - 1), part = tid / PSP_MAX;
+      float w = 0.f, wx = 0.f;
+      if (k < npp) {
+        const int u1 = npp * (part + 1) / 4;
+#pragma unroll 8
+        for (int u = npp * part / 4; u < u1; u++) {
+          const float uk = Ub[u * PSP_MAX + k];
+          w = fmaf(uk, s_r[u], w);
+          wx = fmaf(uk, s_x[u], wx);
+        }
+      }
+      s_pr[part][k] = w;
+      s_px[part][k] = wx;
+    }
+    __syncthreads();
+    if (tid < npp) {
+      float dl = th - lam_all[(int64_t)b * PSP_MAX + tid];
+      if (fabsf(dl) < 1e-4f) dl = dl < 0.f ? -1e-4f : 1e-4f;
+      s_w[tid] = ((s_pr[0][tid] + s_pr[1][tid]) + (s_pr[2][tid] + s_pr[3][tid])) / dl;
+      s_wx[tid] = ((s_px[0][tid] + s_px[1][tid]) + (s_px[2][tid] + s_px[3][tid])) / dl;
+    }
+    __syncthreads();
+    for (int u = warp; u < npp; u += NW) {
+      float v = 0.f, vx = 0.f;
+#pragma unroll
+      for (int q = 0; q < PSP_MAX / 32; q++) {
+        const int k = lane + 32 * q;
+        if (k < npp) {
+          const float uk = Ub[u * PSP_MAX + k];
+          v = fmaf(uk, s_w[k], v);
+          vx = fmaf(uk, s_wx[k], vx);
+        }
+      }
+      for (int o = 16; o; o >>= 1) {
+        v += __shfl_xor_sync(0xffffffffu, v, o);
+        vx += __shfl_xor_sync(0xffffffffu, vx, o);
+      }
+      if (lane == 0) {
+        const int i = s_i[u];
+        const bool diag = i < sym_nd(nstr);
+        const float f = diag ? 1.f : 2.f;   // both elements of a pair change alike
+        const float tn = diag ? v : v * r2;
+        s_del[u] = (tn - Tb[i]) * f;
+        Tb[i] = tn;
+        if (olsen) {
+          const float un = diag ? vx : vx * r2;
+          s_delu[u] = (un - Ob[i]) * f;
+          Ob[i] = un;
+        }
+      }
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  for (int k = tid; k < npp; k += blockDim.x) {
-    float w = 0.f, wx = 0.f;
-    for (int u = 0; u < npp; u++) {
-      const float uk = sU[u * PSP_PITCH + k];
-      w = fmaf(uk, s_r[u], w);
-      if (olsen) wx = fmaf(uk, s_x[u], wx);
-    }
-    float dl = th - lam_all[(int64_t)b * PSP_MAX + k];
-    if (fabsf(dl) < 1e-4f) dl = dl < 0.f ? -1e-4f : 1e-4f;
-    s_w[k] = w / dl;
-    s_wx[k] = wx / dl;
-  }
-  __syncthreads();
-  for (int u = tid; u < npp; u += blockDim.x) {
-    float y = 0.f, yx = 0.f;
-    for (int k = 0; k < npp; k++) {
-      const float uk = sU[u * PSP_PITCH + k];
-      y = fmaf(uk, s_w[k], y);
-      if (olsen) yx = fmaf(uk, s_wx[k], yx);
-    }
-    const int i = s_i[u];
-    const bool diag = i < sym_nd(nstr);
-    const float f = diag ? 1.f : 2.f;   // both elements of a pair change alike
-    const float tn = diag ? y : y * r2;
-    s_del[u] = (tn - Tb[i]) * f;
-    Tb[i] = tn;
-    if (olsen) {
-      const float un = diag ? yx : yx * r2;
-      s_delu[u] = (un - Ob[i]) * f;
-      Ob[i] = un;
-    }
-  }
-  __syncthreads();
-  const int lane = tid & 31, warp = tid >> 5;
-  if (olsen && warp == 0) {
-    double at = 0.0, au = 0.0;
-    for (int u = lane; u < npp; u += 32) {
-      at += (double)s_xv[u] * (double)s_del[u];
-      au += (double)s_xv[u] * (double)s_delu[u];
-    }
-    for (int o = 16; o; o >>= 1) {
-      at += __shfl_down_sync(0xffffffffu, at, o);
-      au += __shfl_down_sync(0xffffffffu, au, o);
-    }
-    if (lane == 0) {
-      xpart[((int64_t)b * 2) * nchunks] += at;
-      xpart[((int64_t)b * 2 + 1) * nchunks] += au;
-    }
-  }
-  if (!fix_dots) return;
+  if (!olsen && !dots) return;
+  // the sums: a warp per value
   const float* Vb = V + (int64_t)b * M * ld;
-  for (int j = warp; j < m; j += APPLY_THREADS / 32) {
-    double acc = 0.0, accu = 0.0;
+  const int nv = dots ? m : 0;
+  const int ntask = olsen ? 2 * nv + 2 : nv;
+  for (int t = warp; t < ntask; t += NW) {
+    const bool xs = t >= 2 * nv && olsen, second = xs ? t == 2 * nv + 1 : t >= nv;
+    const int i = xs ? 0 : second ? t - nv : t;
+    const double* p = xs ? xpart + ((int64_t)b * 2 + (second ? 1 : 0)) * nchunks
+                         : (second ? upart : dpart) + ((int64_t)b * M + i) * nchunks;
+    double s = 0.0;
+    for (int c = lane; c < nchunks; c += 32) s += p[c];
     for (int u = lane; u < npp; u += 32) {
-      const double v = (double)Vb[(int64_t)j * ld + s_i[u]];
-      acc += v * (double)s_del[u];
-      if (olsen) accu += v * (double)s_delu[u];
+      const float v = xs ? s_xv[u] : Vb[(int64_t)i * ld + s_i[u]];
+      s += (double)v * (double)(second ? s_delu[u] : s_del[u]);
     }
-    for (int o = 16; o; o >>= 1) {
-      acc += __shfl_down_sync(0xffffffffu, acc, o);
-      accu += __shfl_down_sync(0xffffffffu, accu, o);
-    }
-    if (lane == 0) {
-      partial[((int64_t)b * m + j) * nchunks] += acc;
-      if (olsen) upart[((int64_t)b * m + j) * nchunks] += accu;
-    }
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) (xs ? s_xs : second ? s_c2 : s_c)[xs ? (second ? 1 : 0) : i] = s;
   }
+  __syncthreads();
+  double e = 0.0;
+  if (olsen) {
+    const double xu = s_xs[1];
+    e = s_xs[0] / xu;
+    if (!(xu != 0.0) || !isfinite(e)) e = 0.0;
+    if (tid == 0) eps[b] = (float)e;
+  }
+  if (tid < nv) coef[(int64_t)b * M + tid] = olsen ? s_c[tid] - e * s_c2[tid] : s_c[tid];
 }
 
 }  // namespace
@@ -529,8 +555,6 @@ void pspace_setup(mbe_ctx* ctx, BinProblem& bp, const float* hd, int64_t ld, dou
   once_per_device(attr_set, ctx->device, [] {
     CU_CHECK(cudaFuncSetAttribute(k_psp_eigh, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   227 * 1024 - 4096));
-    CU_CHECK(cudaFuncSetAttribute(k_psp_apply, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  PSP_MAX * PSP_PITCH * 4));
   });
   k_psp_eigh<<<B, EIG_THREADS, smem, st>>>(bp.tab->masks.ptr, bp.nstr, bp.n, bp.nsig,
                                            bp.heff.ptr, bp.hp.ptr, bp.gp.ptr, hd, ld,
@@ -540,12 +564,11 @@ void pspace_setup(mbe_ctx* ctx, BinProblem& bp, const float* hd, int64_t ld, dou
 
 void pspace_apply(mbe_ctx* ctx, const BinProblem& bp, const PspaceWork& w, float* T,
                   const float* hd, int64_t ld, const double* theta, const float* V, int m, int M,
-                  int nchunks, double* partial, bool fix_dots, const int32_t* active,
-                  bool olsen, float* Uo, const float* X, double* upart, double* xpart) {
-  if (!w.npp) return;
-  const uint32_t smem = (uint32_t)w.npp * PSP_PITCH * 4;
-  k_psp_apply<<<bp.B, APPLY_THREADS, smem, ctx->stream>>>(
-      T, hd, bp.nstr, ld, theta, w.npp, w.sel.ptr, w.U.ptr, w.lam.ptr, V, m, M, nchunks, partial,
-      fix_dots ? 1 : 0, active, olsen ? 1 : 0, Uo, X, upart, xpart);
+                  int nchunks, const double* dpart, bool dots, const int32_t* active, bool olsen,
+                  float* Uo, const float* X, const double* upart, const double* xpart,
+                  const double* y, double* yp, double* coef, float* eps) {
+  k_psp_apply<<<bp.B, APPLY_THREADS, 0, ctx->stream>>>(
+      T, hd, bp.nstr, ld, theta, w.npp, w.sel.ptr, w.U.ptr, w.lam.ptr, V, m, M, nchunks, dpart,
+      dots ? 1 : 0, active, olsen ? 1 : 0, Uo, X, upart, xpart, y, yp, coef, eps);
   CU_LAUNCH_CHECK();
 }

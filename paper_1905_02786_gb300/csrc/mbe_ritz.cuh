@@ -1,30 +1,39 @@
 // Lowest eigenpair of the Davidson subspace matrix (the Rayleigh-Ritz step),
-// one warp per tuple.
+// one CTA of 256 threads per tuple.
 //
 // GB300 issues FP64 at a small fraction of its FP32 rate, so the O(m^3)
 // diagonalisation runs in FP32 and only O(m^2) work per step is FP64:
 //   1. cyclic Jacobi in FP32 with the round-robin (tournament) ordering: the
 //      m/2 rotations of one step touch disjoint index pairs and are applied
-//      together (columns, then rows), so every lane works on every step;
+//      together, rows and columns at once;
 //   2. the lowest FP32 eigenvector z_k is refined in FP64 by Newton steps in
 //      the approximate eigenbasis: with s = G y - theta y (FP64),
 //        y <- y - sum_{j != k} z_j (z_j . s) / (lambda_j - theta),
 //      each step multiplying the error by ~ (FP32 residual of Z) / gap, and
 //      theta = y.G.y is the FP64 Rayleigh quotient of the normalised y.
 // m <= 32; G is read symmetrised, (G + G^T) / 2.
+//
+// The step is a chain of short dependent phases, so its latency is what
+// counts.  A thread owns column (lane) and four rows of A and Z; it forms the
+// rotation of its own column's pair itself, takes those of its rows from the
+// other lanes by shuffles and writes into the other buffer: one barrier per
+// Jacobi step.  When the subspace has grown by one vector since the last call
+// the sweeps start from Z_prev^T G Z_prev, an arrow matrix whose border is
+// small near convergence (2-3 sweeps instead of 6).  FP64 sums run in one
+// warp (each of the others would take the same 16 cycles of the SM's FP64
+// unit per instruction).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+constexpr int RITZ_THREADS = 256;
+
 struct RitzShared {
-  float A[32][33];
-  float Z[32][33];
   double G[32][33];
-  float cs[16][2];
-  int pq[16][2];
-  float lam[32];
-  float s32[32];
-  float coef[32];
+  double y[32], gy[32];
+  float A[2][32][33];
+  float Z[2][32][33];
+  float lam[32], s32[32], coef[32], theta;
 };
 
 __device__ __forceinline__ double ritz_warp_sum(double v) {
@@ -36,118 +45,169 @@ __device__ __forceinline__ float ritz_warp_sumf(float v) {
   return v;
 }
 
-// Called by all 32 lanes of one warp.  Gb: row-major, leading dimension M.
+// Called by all RITZ_THREADS threads of a block.  Gb: row-major, leading
+// dimension M.  Zk: the eigenvectors kept between calls (32 x 32), read when
+// `warm` (they then belong to the leading m - 1 rows of G) and written.
 static __device__ void ritz_lowest(const double* __restrict__ Gb, int m, int M, RitzShared& S,
-                            double* theta_out, double* y_out) {
-  const int r = threadIdx.x & 31;
-  for (int i = 0; i < m; i++)
-    if (r < m) {
-      const double g = 0.5 * (Gb[(int64_t)i * M + r] + Gb[(int64_t)r * M + i]);
-      S.G[i][r] = g;
-      S.A[i][r] = (float)g;
-      S.Z[i][r] = (i == r) ? 1.f : 0.f;
+                                   float* __restrict__ Zk, bool warm, double* theta_out,
+                                   double* y_out) {
+  const int tid = threadIdx.x, r = tid & 31, w = tid >> 5;
+  for (int i = w; i < 32; i += 8) {
+    double g = 0.0;
+    if (i < m && r < m) g = 0.5 * (Gb[(int64_t)i * M + r] + Gb[(int64_t)r * M + i]);
+    S.G[i][r] = g;
+    S.A[0][i][r] = (float)g;
+    S.Z[0][i][r] = warm && i < m - 1 && r < m - 1 ? Zk[i * 32 + r] : (i == r) ? 1.f : 0.f;
+  }
+  __syncthreads();
+  if (warm) {
+    // A <- Z^T A Z through Z[1]
+    for (int i = w; i < m; i += 8) {
+      float v = 0.f;
+      for (int j = 0; j < m; j++) v = fmaf(S.A[0][i][j], S.Z[0][j][r], v);
+      S.Z[1][i][r] = v;
     }
-  __syncwarp();
+    __syncthreads();
+    for (int i = w; i < m; i += 8) {
+      float v = 0.f;
+      for (int j = 0; j < m; j++) v = fmaf(S.Z[0][j][i], S.Z[1][j][r], v);
+      S.A[0][i][r] = v;
+    }
+    __syncthreads();
+  }
   // ---- 1. FP32 tournament Jacobi
   const int n2 = m + (m & 1);
+  int cur = 0;
   for (int sweep = 0; sweep < 12 && m > 1; sweep++) {
+    // every warp sums the whole matrix: the decision is the same in all
     float off = 0.f, dia = 0.f;
-    if (r < m)
-      for (int j = 0; j < m; j++) {
-        const float a = S.A[r][j];
-        if (j != r) off += a * a;
-        else dia += a * a;
-      }
+    for (int j = 0; j < m; j++) {
+      const float a = r < m ? S.A[cur][j][r] : 0.f;
+      if (j != r) off += a * a;
+      else dia += a * a;
+    }
     off = ritz_warp_sumf(off);
     dia = ritz_warp_sumf(dia);
     if (off <= 1e-12f * dia) break;
     for (int step = 0; step < n2 - 1; step++) {
-      if (r < n2 / 2) {
-        auto pos = [&](int j) { return j == 0 ? 0 : 1 + (j - 1 + step) % (n2 - 1); };
-        int p = pos(r), q = pos(n2 - 1 - r);
-        if (p > q) { const int t = p; p = q; q = t; }
-        float c = 1.f, s = 0.f;
+      const float(*A)[33] = S.A[cur];
+      const float(*Z)[33] = S.Z[cur];
+      // the partner of index r in this step and the rotation of their pair:
+      // new column r = cr * column r + sr * column pr
+      int pr = r;
+      float cr = 1.f, sr = 0.f;
+      if (r < m) {
+        int k = 0;
+        if (r != 0) {
+          k = r - step;
+          if (k < 1) k += n2 - 1;
+        }
+        const int kp = n2 - 1 - k;
+        int q = 0;
+        if (kp != 0) {
+          q = kp + step;
+          if (q > n2 - 1) q -= n2 - 1;
+        }
         if (q < m) {
-          const float apq = S.A[p][q];
+          pr = q;
+          const int lo = min(r, q), hi = max(r, q);
+          const float apq = A[lo][hi];
           if (fabsf(apq) > 1e-30f) {
-            const float th = (S.A[q][q] - S.A[p][p]) / (2.f * apq);
-            const float t = (th >= 0.f ? 1.f : -1.f) / (fabsf(th) + sqrtf(th * th + 1.f));
-            c = rsqrtf(t * t + 1.f);
-            s = t * c;
+            // an approximate angle does (c and s stay normalised to an ulp)
+            const float th = __fdividef(A[hi][hi] - A[lo][lo], 2.f * apq);
+            const float h = fmaf(th, th, 1.f);
+            // |th| above 2^63 (h infinite): t = 1 / (2 th) underflows to 0
+            const float t = h < 3e38f
+                                ? copysignf(__fdividef(1.f, fabsf(th) + h * rsqrtf(h)), th) : 0.f;
+            cr = rsqrtf(fmaf(t, t, 1.f));
+            sr = r == lo ? -t * cr : t * cr;
           }
         }
-        S.pq[r][0] = p;
-        S.pq[r][1] = q < m ? q : -1;
-        S.cs[r][0] = c;
-        S.cs[r][1] = s;
       }
-      __syncwarp();
-      // columns: A <- A J, Z <- Z J (lane = row)
-      if (r < m)
-        for (int i = 0; i < n2 / 2; i++) {
-          const int p = S.pq[i][0], q = S.pq[i][1];
-          if (q < 0) continue;
-          const float c = S.cs[i][0], s = S.cs[i][1];
-          const float a = S.A[r][p], b = S.A[r][q];
-          S.A[r][p] = c * a - s * b;
-          S.A[r][q] = s * a + c * b;
-          const float za = S.Z[r][p], zb = S.Z[r][q];
-          S.Z[r][p] = c * za - s * zb;
-          S.Z[r][q] = s * za + c * zb;
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const int i = w + 8 * k;
+        const int pi = __shfl_sync(0xffffffffu, pr, i);
+        const float ci = __shfl_sync(0xffffffffu, cr, i), si = __shfl_sync(0xffffffffu, sr, i);
+        if (i < m && r < m) {
+          const float x = fmaf(cr, A[i][r], sr * A[i][pr]);
+          const float y = fmaf(cr, A[pi][r], sr * A[pi][pr]);
+          S.A[cur ^ 1][i][r] = fmaf(ci, x, si * y);
+          S.Z[cur ^ 1][i][r] = fmaf(cr, Z[i][r], sr * Z[i][pr]);
         }
-      __syncwarp();
-      // rows: A <- J^T A (lane = column)
-      if (r < m)
-        for (int i = 0; i < n2 / 2; i++) {
-          const int p = S.pq[i][0], q = S.pq[i][1];
-          if (q < 0) continue;
-          const float c = S.cs[i][0], s = S.cs[i][1];
-          const float a = S.A[p][r], b = S.A[q][r];
-          S.A[p][r] = c * a - s * b;
-          S.A[q][r] = s * a + c * b;
-        }
-      __syncwarp();
+      }
+      __syncthreads();
+      cur ^= 1;
     }
   }
-  if (r < m) S.lam[r] = S.A[r][r];
-  __syncwarp();
-  int k = 0;
-  for (int i = 1; i < m; i++)
-    if (S.lam[i] < S.lam[k]) k = i;
-  // ---- 2. FP64 Newton refinement of the lowest pair
-  double y = r < m ? (double)S.Z[r][k] : 0.0;
-  double nn = ritz_warp_sum(y * y);
-  y /= sqrt(nn);
+  const float(*Z)[33] = S.Z[cur];
+  for (int i = w; i < m; i += 8)
+    if (r < m) Zk[i * 32 + r] = Z[i][r];
+  // the lowest eigenvalue (the first of equal ones), known to every lane
+  int k = r;
+  {
+    float v = r < m ? S.A[cur][r][r] : 3.4e38f;
+    for (int o = 16; o; o >>= 1) {
+      const float ov = __shfl_xor_sync(0xffffffffu, v, o);
+      const int ok = __shfl_xor_sync(0xffffffffu, k, o);
+      if (ov < v || (ov == v && ok < k)) {
+        v = ov;
+        k = ok;
+      }
+    }
+  }
+  // ---- 2. FP64 Newton refinement of the lowest pair (y unnormalised; warp 0
+  // keeps it, lane = component); row products are spread over 8 threads
+  double y = r < m ? (double)Z[r][k] : 0.0;
   double theta = 0.0;
+  const int row = tid >> 3, part = tid & 7;
   for (int it = 0; it < 4; it++) {
-    double gy = 0.0;
-    for (int j = 0; j < m; j++) {
-      const double yj = __shfl_sync(0xffffffffu, y, j);
-      if (r < m) gy = fma(S.G[r][j], yj, gy);
+    if (w == 0) S.y[r] = y;
+    __syncthreads();
+    if (4 * w < m) {   // the warps that hold rows below m
+      double gy = 0.0;
+      for (int j = part; j < m; j += 8) gy = fma(S.G[row][j], S.y[j], gy);
+      for (int o = 4; o; o >>= 1) gy += __shfl_xor_sync(0xffffffffu, gy, o);
+      if (part == 0) S.gy[row] = gy;
     }
-    theta = ritz_warp_sum(y * gy);
+    __syncthreads();
+    if (w == 0) {
+      const double g = r < m ? S.gy[r] : 0.0;
+      double a = y * g, n = y * y;
+      for (int o = 16; o; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        n += __shfl_xor_sync(0xffffffffu, n, o);
+      }
+      theta = a / n;
+      S.s32[r] = (float)(g - theta * y);
+      if (r == 0) S.theta = (float)theta;
+      if (it == 3) y /= sqrt(n);
+    }
     if (it == 3) break;
-    S.s32[r] = (float)(gy - theta * y);
-    __syncwarp();
-    float cf = 0.f;
-    if (r < m && r != k) {
-      const float den = S.lam[r] - (float)theta;
-      if (fabsf(den) > 1e-6f * fmaxf(1.f, fabsf((float)theta))) {
-        float d = 0.f;
-        for (int j = 0; j < m; j++) d = fmaf(S.Z[j][r], S.s32[j], d);
-        cf = d / den;
+    __syncthreads();
+    if (4 * w < m) {
+      float d = 0.f;
+      for (int j = part; j < m; j += 8) d = fmaf(Z[j][row], S.s32[j], d);
+      for (int o = 4; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+      if (part == 0) {
+        float cf = 0.f;
+        if (row < m && row != k) {
+          const float th = S.theta, den = S.A[cur][row][row] - th;
+          if (fabsf(den) > 1e-6f * fmaxf(1.f, fabsf(th))) cf = d / den;
+        }
+        S.coef[row] = cf;
       }
     }
-    S.coef[r] = cf;
-    __syncwarp();
-    float w = 0.f;
-    if (r < m)
-      for (int j = 0; j < m; j++) w = fmaf(S.Z[r][j], S.coef[j], w);
-    y -= (double)w;
-    nn = ritz_warp_sum(y * y);
-    y /= sqrt(nn);
-    __syncwarp();
+    __syncthreads();
+    if (4 * w < m) {
+      float c = 0.f;
+      for (int j = part; j < m; j += 8) c = fmaf(Z[row][j], S.coef[j], c);
+      for (int o = 4; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+      if (part == 0) S.lam[row] = c;
+    }
+    __syncthreads();
+    if (w == 0 && r < m) y -= (double)S.lam[r];
   }
-  if (r == 0) *theta_out = theta;
-  if (r < m) y_out[r] = y;
+  if (tid == 0) *theta_out = theta;
+  if (w == 0 && r < m) y_out[r] = y;
 }

@@ -387,8 +387,7 @@ k_sigma_direct(const DirArgs A, const DirPlan L) {
   for (int k = tid; k < nb; k += nt) {
     double s = sPart[k];
     for (int part = 1; part < S; part++) s += sPart[part * nb + k];
-    ob[(int64_t)a * nstrb + b0 + k] = s;
-    if (A.sym && k > 0) ob[(int64_t)(b0 + k) * nstrb + a] = s;
+    ob[A.sym ? sym_index(a, b0 + k, nstrb) : (int64_t)a * nstrb + k] = s;
   }
 }
 

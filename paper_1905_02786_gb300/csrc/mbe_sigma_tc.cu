@@ -106,8 +106,11 @@ __global__ void k_split_c(const float* __restrict__ c, int64_t c_stride, int nst
 // the same from a packed symmetric vector (sym_index layout): one CTA per
 // 32 x 32 tile pair (I, J), I <= J, reads tile (I, J) from the packed rows
 // (coalesced) and writes the rows of both tiles, the transposed one through
-// shared memory; the values are those k_split_c gives for the full vector
-__global__ void k_split_c_sym(const float* __restrict__ c, int64_t c_stride, int nstr, int ldc,
+// shared memory; the values are those k_split_c gives for the full vector.
+// With T the vector is inv T (a new subspace vector, normalised here) and is
+// also written to c.
+__global__ void k_split_c_sym(float* __restrict__ c, int64_t c_stride, const float* __restrict__ T,
+                              int64_t t_stride, const double* __restrict__ inv, int nstr, int ldc,
                               const int32_t* __restrict__ active, bf16* __restrict__ cs,
                               int64_t cs_stride) {
   const int b = blockIdx.y;
@@ -120,13 +123,24 @@ __global__ void k_split_c_sym(const float* __restrict__ c, int64_t c_stride, int
   }
   const int J = I + t;
   __shared__ float sC[32][33];
-  const float* cb = c + (int64_t)b * c_stride;
+  float* cb = c + (int64_t)b * c_stride;
+  const float* src = T ? T + (int64_t)b * t_stride : cb;
+  const float f = T ? (float)inv[b] : 1.f;
   bf16* hi = cs + (int64_t)b * cs_stride;
   bf16* lo = hi + (int64_t)nstr * ldc;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, ny = blockDim.x >> 5;
   for (int i = ty; i < 32; i += ny) {
     const int r = I * 32 + i, k = J * 32 + tx;
-    sC[i][tx] = (r < nstr && k < nstr) ? cb[sym_index(r, k, nstr)] : 0.f;
+    float v = 0.f;
+    if (r < nstr && k < nstr) {
+      const int64_t p = sym_index(r, k, nstr);
+      v = src[p];
+      if (T) {
+        v *= f;
+        if (r <= k) cb[p] = v;
+      }
+    }
+    sC[i][tx] = v;
   }
   __syncthreads();
   // rows of tile I, columns of tile J (zeros from nstr up to ldc)
@@ -1036,9 +1050,9 @@ bool sigma_tc_supported(int n, int nstr) {
   return true;
 }
 
-void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, const float* c, int64_t c_stride,
+void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, float* c, int64_t c_stride,
               float* out, int64_t out_stride, const int32_t* active, double spin_shift,
-              bool packed) {
+              bool packed, const float* T, const double* inv) {
   const int npair = bp.npair, nstr = bp.nstr, B = bp.B;
   const int nsm = sm_count(ctx->device);
   AbPlan p;
@@ -1105,8 +1119,8 @@ void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, const float* c, int64_
   bf16* cs = (bf16*)w.csplit.ptr;
   if (packed) {
     const int ntp = (nstr + 31) / 32;
-    k_split_c_sym<<<dim3((unsigned)(ntp * (ntp + 1) / 2), B), 256, 0, st>>>(c, c_stride, nstr,
-                                                                           p.ldc, active, cs, hs);
+    k_split_c_sym<<<dim3((unsigned)(ntp * (ntp + 1) / 2), B), 256, 0, st>>>(
+        c, c_stride, T, sym_len(nstr), inv, nstr, p.ldc, active, cs, hs);
     CU_LAUNCH_CHECK();
   } else {
     const int64_t work = (int64_t)nstr * (p.ldc / 8);
