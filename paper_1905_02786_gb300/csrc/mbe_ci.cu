@@ -18,6 +18,7 @@
 // E+_P acting on one spin string has at most one non-zero matrix element
 // per string, which the link table stores.
 #include "mbe_internal.cuh"
+#include <algorithm>
 
 namespace {
 
@@ -131,90 +132,93 @@ __device__ __forceinline__ int64_t gpair(int p, int q) {
   return p >= q ? (int64_t)p * (p + 1) / 2 + q : (int64_t)q * (q + 1) / 2 + p;
 }
 
-// One CTA per tuple.  act: n sorted global orbital ids.
-__global__ void k_effints(const double* __restrict__ h, const double* __restrict__ eri,
-                          int norb, int nocc, int npair_g, const int32_t* __restrict__ act_all,
-                          int n, int nel, double* ecore_out, double* heff_out, double* hp_out,
-                          double* gp_out, double* jk_out) {
+// gridDim.y CTAs per tuple, each forming the small parts (a few thousand
+// gathers) and writing a slice of g' (B = 1 with one CTA and the pairs decoded
+// by an FP64 square root per element took 21 us).  act: n sorted global
+// orbital ids, or NULL: the ones in `al` (one tuple).
+__global__ void __launch_bounds__(256)
+k_effints(const double* __restrict__ h, const double* __restrict__ eri, int norb, int nocc,
+          int npair_g, const int32_t* __restrict__ act_all, ActList al, int n, int nel,
+          double* ecore_out, double* heff_out, double* hp_out, double* gp_out, double* jk_out) {
   const int b = blockIdx.x;
-  const int32_t* act = act_all + (int64_t)b * n;
   extern __shared__ double sm[];
   double* s_heff = sm;            // n*n
   double* s_hp = sm + n * n;      // n*n
   __shared__ int s_core[MBE_MAX_NORB];
   __shared__ int s_ncore;
   __shared__ int s_act[MBE_MAX_ACT];
-  if (threadIdx.x == 0) {
-    int nc = 0, j = 0;
-    for (int i = 0; i < nocc; i++) {
-      while (j < n && act[j] < i) j++;
-      if (!(j < n && act[j] == i)) s_core[nc++] = i;
+  __shared__ uint8_t s_p[128], s_q[128];   // orbitals of a packed active pair
+  __shared__ int s_g[128];                 // its global pair index
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const bool lead = blockIdx.y == 0;
+  if (tid < n) s_act[tid] = act_all ? act_all[(int64_t)b * n + tid] : al.v[tid];
+  const int npair = n * (n + 1) / 2;
+  for (int p = tid; p < n; p += nt)
+    for (int q = 0; q <= p; q++) {
+      s_p[p * (p + 1) / 2 + q] = (uint8_t)p;
+      s_q[p * (p + 1) / 2 + q] = (uint8_t)q;
     }
-    s_ncore = nc;
+  __syncthreads();
+  if (tid < 32) {
+    // inactive core: occupied orbitals outside the active space, ascending
+    int nc = 0;
+    for (int i0 = 0; i0 < nocc; i0 += 32) {
+      const int i = i0 + tid;
+      bool in = i < nocc;
+      for (int j = 0; in && j < n; j++) in = s_act[j] != i;
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      if (in) s_core[nc + __popc(m & ((1u << tid) - 1u))] = i;
+      nc += __popc(m);
+    }
+    if (tid == 0) s_ncore = nc;
   }
-  if (threadIdx.x < n) s_act[threadIdx.x] = act[threadIdx.x];
+  for (int P = tid; P < npair; P += nt) s_g[P] = (int)gpair(s_act[s_p[P]], s_act[s_q[P]]);
   __syncthreads();
   const int nc = s_ncore;
   const int64_t NP = npair_g;
   // inactive-core energy (Fig. 2: occupied orbitals outside the active space
   // stay doubly occupied): sum 2 h_ii + sum_ij [2 (ii|jj) - (ij|ji)]
-  if (threadIdx.x == 0) {
+  if (lead && tid < 32) {
     double e = 0.0;
-    for (int x = 0; x < nc; x++) {
-      int i = s_core[x];
-      e += 2.0 * h[(int64_t)i * norb + i];
+    for (int t = tid; t < nc * nc; t += 32) {
+      const int i = s_core[t / nc], j = s_core[t % nc];
+      e += 2.0 * eri[gpair(i, i) * NP + gpair(j, j)] - eri[gpair(i, j) * NP + gpair(j, i)];
     }
-    double e2 = 0.0;
-    for (int x = 0; x < nc; x++)
-      for (int y = 0; y < nc; y++) {
-        int i = s_core[x], j = s_core[y];
-        e2 += 2.0 * eri[gpair(i, i) * NP + gpair(j, j)] - eri[gpair(i, j) * NP + gpair(j, i)];
-      }
-    ecore_out[b] = e + e2;
+    for (int x = tid; x < nc; x += 32) e += 2.0 * h[(int64_t)s_core[x] * norb + s_core[x]];
+    for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (tid == 0) ecore_out[b] = e;
   }
-  // h_eff_pq = h_pq + sum_i [2 (pq|ii) - (pi|iq)]
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-    int p = t / n, q = t % n;
-    int P = s_act[p], Q = s_act[q];
+  // h_eff_pq = h_pq + sum_i [2 (pq|ii) - (pi|iq)] and
+  // h'_pq = h_eff_pq - 1/2 sum_r (pr|rq), r over the active orbitals
+  for (int t = tid; t < n * n; t += nt) {
+    const int p = t / n, q = t - p * n;
+    const int P = s_act[p], Q = s_act[q];
     double v = h[(int64_t)P * norb + Q];
+#pragma unroll 4
     for (int x = 0; x < nc; x++) {
-      int i = s_core[x];
+      const int i = s_core[x];
       v += 2.0 * eri[gpair(P, Q) * NP + gpair(i, i)] - eri[gpair(P, i) * NP + gpair(i, Q)];
     }
+    double x = 0.0;
+#pragma unroll 4
+    for (int r = 0; r < n; r++) x += eri[gpair(P, s_act[r]) * NP + gpair(s_act[r], Q)];
     s_heff[t] = v;
-    heff_out[(int64_t)b * n * n + t] = v;
-    jk_out[(int64_t)b * 2 * n * n + t] = eri[gpair(P, P) * NP + gpair(Q, Q)];
-    jk_out[(int64_t)b * 2 * n * n + n * n + t] = eri[gpair(P, Q) * NP + gpair(Q, P)];
-  }
-  __syncthreads();
-  // h'_pq = h_eff_pq - 1/2 sum_r (pr|rq), r over the active orbitals
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-    int p = t / n, q = t % n;
-    int P = s_act[p], Q = s_act[q];
-    double v = 0.0;
-    for (int r = 0; r < n; r++) {
-      int R = s_act[r];
-      v += eri[gpair(P, R) * NP + gpair(R, Q)];
+    s_hp[t] = v - 0.5 * x;
+    if (lead) {
+      heff_out[(int64_t)b * n * n + t] = v;
+      hp_out[(int64_t)b * n * n + t] = v - 0.5 * x;
+      jk_out[(int64_t)b * 2 * n * n + t] = eri[gpair(P, P) * NP + gpair(Q, Q)];
+      jk_out[(int64_t)b * 2 * n * n + n * n + t] = eri[gpair(P, Q) * NP + gpair(Q, P)];
     }
-    s_hp[t] = s_heff[t] - 0.5 * v;
-    hp_out[(int64_t)b * n * n + t] = s_hp[t];
   }
   __syncthreads();
   // g'_{PQ} = (pq|rs) + (h'_pq d_rs + d_pq h'_rs) / N_active, N_active = nel
   // active electrons of both spins (sum_r E_rr = N_active on the space)
-  const int npair = n * (n + 1) / 2;
   const double inv = nel > 0 ? 1.0 / nel : 0.0;
-  for (int t = threadIdx.x; t < npair * npair; t += blockDim.x) {
-    int P = t / npair, Q = t % npair;
-    int p = (int)((sqrt(8.0 * P + 1.0) - 1.0) * 0.5);
-    while (p * (p + 1) / 2 > P) p--;
-    while ((p + 1) * (p + 2) / 2 <= P) p++;
-    int q = P - p * (p + 1) / 2;
-    int r = (int)((sqrt(8.0 * Q + 1.0) - 1.0) * 0.5);
-    while (r * (r + 1) / 2 > Q) r--;
-    while ((r + 1) * (r + 2) / 2 <= Q) r++;
-    int s = Q - r * (r + 1) / 2;
-    double v = eri[gpair(s_act[p], s_act[q]) * NP + gpair(s_act[r], s_act[s])];
+  for (int t = blockIdx.y * nt + tid; t < npair * npair; t += gridDim.y * nt) {
+    const int P = t / npair, Q = t - P * npair;
+    const int p = s_p[P], q = s_q[P], r = s_p[Q], s = s_q[Q];
+    double v = eri[(int64_t)s_g[P] * NP + s_g[Q]];
     if (r == s) v += s_hp[p * n + q] * inv;
     if (p == q) v += s_hp[r * n + s] * inv;
     gp_out[(int64_t)b * npair * npair + t] = v;
@@ -223,11 +227,15 @@ __global__ void k_effints(const double* __restrict__ h, const double* __restrict
 
 }  // namespace
 
-void launch_effints_raw(mbe_ctx* ctx, const int32_t* act, int B, int n, int nel, double* ecore,
-                        double* heff, double* hp, double* gp, double* jk) {
+void launch_effints_raw(mbe_ctx* ctx, const int32_t* act, const ActList* al, int B, int n, int nel,
+                        double* ecore, double* heff, double* hp, double* gp, double* jk) {
   size_t smem = 2 * sizeof(double) * n * n;
-  k_effints<<<B, 256, smem, ctx->stream>>>(ctx->h.ptr, ctx->eri.ptr, ctx->norb, ctx->nocc,
-                                           ctx->npair_g, act, n, nel, ecore, heff, hp, gp, jk);
+  // a CTA per 1024 elements of g' while the batch leaves SMs idle
+  const int npair = n * (n + 1) / 2;
+  const int split = std::max(1, std::min((npair * npair + 1023) / 1024, 304 / B));
+  k_effints<<<dim3(B, split), 256, smem, ctx->stream>>>(
+      ctx->h.ptr, ctx->eri.ptr, ctx->norb, ctx->nocc, ctx->npair_g, act, al ? *al : ActList{}, n,
+      nel, ecore, heff, hp, gp, jk);
   CU_LAUNCH_CHECK();
 }
 
@@ -239,7 +247,7 @@ void launch_effints(mbe_ctx* ctx, BinProblem& bp) {
   bp.gp.reset(&ctx->pool, (size_t)B * bp.npair * bp.npair);
   bp.jk.reset(&ctx->pool, (size_t)B * 2 * n * n);
   const int nel = bp.nsig + (bp.nsigb < 0 ? bp.nsig : bp.nsigb);
-  launch_effints_raw(ctx, bp.act.ptr, B, n, nel, bp.ecore.ptr, bp.heff.ptr, bp.hp.ptr,
+  launch_effints_raw(ctx, bp.act.ptr, nullptr, B, n, nel, bp.ecore.ptr, bp.heff.ptr, bp.hp.ptr,
                      bp.gp.ptr, bp.jk.ptr);
 }
 

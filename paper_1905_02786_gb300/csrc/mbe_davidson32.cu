@@ -160,8 +160,10 @@ __global__ void k32_hdiag(const uint32_t* __restrict__ masks, int nstr, int64_t 
   }
 }
 
-__global__ void k32_guess(const float* __restrict__ hd, int nstr, int64_t ld, int M,
-                          float* __restrict__ V) {
+// lowest-diagonal determinant a nstr + c, a <= c, of every tuple (without a
+// P-space, whose selection finds it too)
+__global__ void k32_lowest(const float* __restrict__ hd, int nstr, int64_t ld,
+                           int32_t* __restrict__ low) {
   const int b = blockIdx.x;
   const int64_t N = (int64_t)nstr * nstr;
   __shared__ float sv[256];
@@ -188,14 +190,16 @@ __global__ void k32_guess(const float* __restrict__ hd, int nstr, int64_t ld, in
     }
     __syncthreads();
   }
-  float* Vb = V + (int64_t)b * M * ld;
-  for (int64_t k = threadIdx.x; k < ld; k += blockDim.x) Vb[k] = 0.f;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const int64_t i0 = si[0];
-    const int ia = (int)(i0 / nstr), ib = (int)(i0 % nstr);
-    // (|a b> + |b a>) / sqrt(2): its packed element carries both halves
-    Vb[sym_index(ia, ib, nstr)] = ia == ib ? 1.f : 0.70710678f;
+  if (threadIdx.x == 0) low[b] = (int)si[0];
+}
+
+// start vectors: (|a b> + |b a>) / sqrt(2) of the lowest determinant (its
+// packed element carries both halves), or |a a>; V_0 is zero on entry
+__global__ void k32_guess(const int32_t* __restrict__ low, int B, int nstr, int64_t vstride,
+                          float* __restrict__ V) {
+  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < B; b += gridDim.x * blockDim.x) {
+    const int ia = low[b] / nstr, ib = low[b] - ia * nstr;
+    V[(int64_t)b * vstride + sym_index(ia, ib, nstr)] = ia == ib ? 1.f : 0.70710678f;
   }
 }
 
@@ -384,7 +388,12 @@ void davidson_batch_mixed(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int3
   DevBuf<float> U32(P, olsen ? (size_t)B * L : 0), epsb(P, olsen ? (size_t)B : 0);
   DevBuf<double> upart(P, olsen ? (size_t)B * M * nchunks : 0),
       xpart(P, olsen ? (size_t)B * 2 * nchunks : 0);
-  k32_guess<<<B, 256, 0, st>>>(hd.ptr, bp.nstr, L, M, V.ptr);
+  if (!olsen) {
+    psp.low.reset(P, B);
+    k32_lowest<<<B, 256, 0, st>>>(hd.ptr, bp.nstr, L, psp.low.ptr);
+    CU_LAUNCH_CHECK();
+  }
+  k32_guess<<<(B + 255) / 256, 256, 0, st>>>(psp.low.ptr, B, bp.nstr, (int64_t)M * L, V.ptr);
   CU_LAUNCH_CHECK();
   if (plan) {
     // the parent guess writes full vectors (into F), packed into V_0 here

@@ -418,13 +418,14 @@ struct BinProblem {
 };
 
 // P-space preconditioner of the mixed Davidson iteration (mbe_pspace.cu):
-// per tuple the npp lowest-diagonal symmetric basis functions, the
-// eigenvectors U and eigenvalues of A restricted to them
+// per tuple the npp lowest-diagonal symmetric basis functions and A
+// restricted to them as Q T Q^T, T tridiagonal
 struct PspaceWork {
   int npp = 0;
   DevBuf<int32_t> sel;   // B * 128 canonical determinant indices
-  DevBuf<float> lam;     // B * 128
-  DevBuf<float> U;       // B * 128 * 128
+  DevBuf<int32_t> low;   // B: the lowest-diagonal one
+  DevBuf<float> tri;     // B * 2 * 128: diagonal, subdiagonal of T
+  DevBuf<float> Qt;      // B * 128 * 128: rows of Q^T
 };
 // the P-space size used for a bin (0: off) given the requested size
 int pspace_size(const BinProblem& bp, int requested);
@@ -447,9 +448,14 @@ void build_string_tables(mbe_ctx* ctx, StringTables* t);
 // allocate nothing)
 int64_t string_count(int n, int nsig);
 void launch_string_masks(mbe_ctx* ctx, int n, int nsig, int nstr, uint32_t* masks);
-// nel: active electrons (both spins)
-void launch_effints_raw(mbe_ctx* ctx, const int32_t* act, int B, int n, int nel, double* ecore,
-                        double* heff, double* hp, double* gp, double* jk);
+// the sorted active orbitals (at most 15) of one tuple, by value
+struct ActList {
+  int32_t v[16];
+};
+// nel: active electrons (both spins); act: B * n orbitals on the device, or
+// NULL: those of al (B = 1)
+void launch_effints_raw(mbe_ctx* ctx, const int32_t* act, const ActList* al, int B, int n, int nel,
+                        double* ecore, double* heff, double* hp, double* gp, double* jk);
 // one spin's strings and tables of the FP64 sigma
 struct DirectSide {
   int nsig, nstr;
@@ -459,7 +465,8 @@ struct DirectSide {
   const double* hv;        // their one-spin elements, per tuple
 };
 int direct_nnz(int n, int nsig);   // replacements of one string, itself included
-void launch_direct_tables(mbe_ctx* ctx, int n, int nsig, int nstr, const uint32_t* masks,
+// (masks is written too: the ascending strings)
+void launch_direct_tables(mbe_ctx* ctx, int n, int nsig, int nstr, uint32_t* masks,
                           uint16_t* hidx, uint32_t* olnk);
 // hv (B * nnz * nstr) and, unless NULL, wt (B * npair * nstr)
 void launch_direct_values(mbe_ctx* ctx, int n, int nsig, int nstr, const uint32_t* masks, int B,

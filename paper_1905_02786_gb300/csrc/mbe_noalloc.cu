@@ -53,7 +53,7 @@ unsigned char* scratch_base(int device) {
 
 // byte offsets of the pieces inside the scratch array (256-byte aligned)
 struct NoallocLayout {
-  size_t masks, act, ecore, heff, hp, gp, jk, hidx, olnk, hv, wt, total;
+  size_t masks, ecore, heff, hp, gp, jk, hidx, olnk, hv, wt, total;
   size_t limit;   // what MBE_NOALLOC_SCRATCH_BYTES is compared with
 };
 
@@ -68,7 +68,6 @@ NoallocLayout noalloc_layout(int n, int nsig, int64_t nstr) {
     return r;
   };
   L.masks = take(sizeof(uint32_t) * nstr);
-  L.act = take(sizeof(int32_t) * n);
   L.ecore = take(sizeof(double));
   L.heff = take(sizeof(double) * n * n);
   L.hp = take(sizeof(double) * n * n);
@@ -81,21 +80,13 @@ NoallocLayout noalloc_layout(int n, int nsig, int64_t nstr) {
   L.wt = take(sizeof(double) * npair * nstr);
   L.total = o;
   o = common;
+  take(sizeof(int32_t) * n);
   take(sizeof(int32_t) * nstr * npair);
   take(sizeof(int32_t));
   take(sizeof(double) * npair * ndet);
   take(sizeof(double) * npair * ndet);
   L.limit = o;
   return L;
-}
-
-// the sorted active orbitals (at most 15) passed by value
-struct ActList {
-  int32_t v[16];
-};
-__global__ void k_put_act(ActList a, int n, int32_t* __restrict__ dst) {
-  const int t = threadIdx.x;
-  if (t < n) dst[t] = a.v[t];
 }
 
 }  // namespace
@@ -122,20 +113,15 @@ int noalloc_sigma_run(mbe_ctx* ctx, const int* act, int nact, const double* c_de
     throw MbeError{MBE_EINVAL, "active space too large for the no-allocation scratch"};
   unsigned char* base = scratch_base(ctx->device);
   uint32_t* masks = (uint32_t*)(base + L.masks);
-  int32_t* actd = (int32_t*)(base + L.act);
   double* ecore = (double*)(base + L.ecore);
   double* gp = (double*)(base + L.gp);
   double* hv = (double*)(base + L.hv);
   double* wt = (double*)(base + L.wt);
   uint32_t* olnk = (uint32_t*)(base + L.olnk);
   uint16_t* hidx = (uint16_t*)(base + L.hidx);
-  cudaStream_t st = ctx->stream;
   ActList al = {};
   for (int i = 0; i < nact; i++) al.v[i] = a[i];
-  k_put_act<<<1, 32, 0, st>>>(al, nact, actd);
-  CU_LAUNCH_CHECK();
-  launch_string_masks(ctx, nact, nsig, (int)nstr, masks);
-  launch_effints_raw(ctx, actd, 1, nact, 2 * nsig, ecore, (double*)(base + L.heff),
+  launch_effints_raw(ctx, nullptr, &al, 1, nact, 2 * nsig, ecore, (double*)(base + L.heff),
                      (double*)(base + L.hp), gp, (double*)(base + L.jk));
   launch_direct_tables(ctx, nact, nsig, (int)nstr, masks, hidx, olnk);
   launch_direct_values(ctx, nact, nsig, (int)nstr, masks, 1, gp, hv, wt);
@@ -144,8 +130,8 @@ int noalloc_sigma_run(mbe_ctx* ctx, const int* act, int nact, const double* c_de
   sigma_direct_raw(ctx, nact, side, side, wt, gp, c_dev, ndet, sigma_dev, ndet, nullptr, nullptr, 1,
                    ctx->opt.spin_shift, false);
   if (e_core) {
-    CU_CHECK(cudaMemcpyAsync(e_core, ecore, sizeof(double), cudaMemcpyDeviceToHost, st));
-    CU_CHECK(cudaStreamSynchronize(st));
+    CU_CHECK(cudaMemcpyAsync(e_core, ecore, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+    CU_CHECK(cudaStreamSynchronize(ctx->stream));
   }
   return MBE_OK;
 }

@@ -10,15 +10,16 @@
 // of symmetric basis functions: a canonical determinant pair (a, b), a <= b,
 // stands for (|a b> + |b a>) / sqrt(2) (or |a a>), and A_PP is A in that
 // basis.  Per tuple, once:
-//   k_psp_select  the npp canonical pairs of lowest diagonal (radix select on
-//                 the FP32 diagonal, ties broken by index), in index order;
-//   k_psp_eigh    A_PP from the Slater-Condon rules (one-electron h_eff with
+//   k_psp_select  the npp canonical pairs of lowest diagonal (FP32, ties
+//                 broken by index), in index order, and the lowest of them
+//                 (the start vector);
+//   k_psp_tri     A_PP from the Slater-Condon rules (one-electron h_eff with
 //                 the core folded in, (pq|rs) of the active orbitals, the
-//                 spin-exchange couplings of lambda S^2), then its
-//                 eigenvectors by cyclic Jacobi (parallel tournament order)
+//                 spin-exchange couplings of lambda S^2), reduced to
+//                 tridiagonal form A_PP = Q T Q^T by Householder reflections
 //                 in shared memory, FP32 (a preconditioner needs no more);
 // per iteration:
-//   k_psp_apply   t_P = U (theta - Lambda)^{-1} U^T r_P (r_P recovered from
+//   k_psp_apply   t_P = Q (theta - T)^{-1} Q^T r_P (r_P recovered from
 //                 the diagonal correction as t_I (theta - A_II)), written
 //                 back into the packed vector; the same for M^-1 x, x the
 //                 Ritz vector; and the first Gram-Schmidt pass's
@@ -37,11 +38,9 @@
 namespace {
 
 constexpr int PSP_MAX = 128;
-constexpr int PSP_PITCH = PSP_MAX + 1;   // row pitch of the shared matrices
 constexpr int SEL_THREADS = 1024;
-constexpr int EIG_THREADS = 1024;
+constexpr int TRI_THREADS = 8 * PSP_MAX;
 constexpr int APPLY_THREADS = 4 * PSP_MAX;
-constexpr int EIG_SWEEPS = 10;
 
 // FP32 bit pattern mapped to an unsigned key with the same order
 __device__ __forceinline__ uint32_t order_key(float x) {
@@ -49,89 +48,179 @@ __device__ __forceinline__ uint32_t order_key(float x) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// exclusive count of set flags below this thread in the block, and the
-// block total (all threads must call; s_warp holds 32 ints)
-__device__ __forceinline__ int block_flag_scan(bool f, int* s_warp, int* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned bal = __ballot_sync(0xffffffffu, f);
-  if (lane == 0) s_warp[warp] = __popc(bal);
-  __syncthreads();
-  int off = 0, tot = 0;
-  const int nw = (int)(blockDim.x >> 5);
-  for (int w = 0; w < nw; w++) {
-    const int c = s_warp[w];
-    if (w < warp) off += c;
-    tot += c;
-  }
-  __syncthreads();
-  *total = tot;
-  return off + __popc(bal & ((1u << lane) - 1u));
+// packed position p of the diagonal -> linear index a nstr + c, a <= c
+__device__ __forceinline__ int linear_of(int64_t p, int nstr) {
+  const int nd = sym_nd(nstr);
+  if (p < nd) return (int)p * nstr + (int)p;
+  const int64_t t = p - nd;   // row a starts at a (2 nstr - a - 1) / 2
+  int a = (int)(((2.0f * nstr - 1.0f) - sqrtf((2.0f * nstr - 1.0f) * (2.0f * nstr - 1.0f) - 8.0f * (float)t)) * 0.5f);
+  a = max(0, min(a, nstr - 2));
+  while (a > 0 && (int64_t)a * (2 * nstr - a - 1) / 2 > t) a--;
+  while ((int64_t)(a + 1) * (2 * nstr - a - 2) / 2 <= t) a++;
+  return a * nstr + (int)(t - (int64_t)a * (2 * nstr - a - 1) / 2) + a + 1;
 }
 
 // psel[b][0..npp) = linear indices a nstr + c (a <= c) of the npp canonical
-// pairs of lowest diagonal, in increasing index order (the diagonal and all
-// vectors are in the packed symmetric layout, element (a, c) at
-// sym_index(a, c))
+// pairs of lowest diagonal, in increasing index order; gidx[b] the lowest one
+// (ties: the lower index).  One CTA per tuple, three passes over the packed
+// diagonal (contiguous 16-byte loads): the smallest and largest value, a
+// histogram on the linear scale between them, and the elements up to the bin
+// of the npp-th, which are sorted in shared memory.  Bins near the lowest
+// determinants hold few elements; where they hold more than SEL_CAP (a
+// diagonal with many equal values) the threshold is found by bisection on the
+// ordered keys instead, 64 more passes.  (10e/13o, 829,000 elements: 0.26 ms;
+// a four-pass radix select over all pairs with the index arithmetic per
+// element took 2.6 ms.)
+constexpr int SEL_BINS = 4096, SEL_CAP = 2048;
+struct SelShared {
+  union {
+    int hist[SEL_BINS];
+    unsigned long long cand[SEL_CAP];   // key, then linear index
+  };
+};
 __global__ void __launch_bounds__(SEL_THREADS)
     k_psp_select(const float* __restrict__ hd_all, int nstr, int64_t ld, int npp,
-                 int32_t* __restrict__ psel) {
-  const int b = blockIdx.x;
-  const int64_t N = (int64_t)nstr * nstr;
+                 int32_t* __restrict__ psel, int32_t* __restrict__ gidx) {
+  const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float* hd = hd_all + (int64_t)b * ld;
-  __shared__ uint32_t hist[256];
-  __shared__ uint32_t s_prefix;
-  __shared__ int s_k;
-  __shared__ int s_warp[32];
-  uint32_t prefix = 0, mask = 0;
-  int k = npp;   // rank (from 1) of the threshold key among the remaining keys
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0u;
-    __syncthreads();
-    for (int64_t i = threadIdx.x; i < N; i += blockDim.x) {
-      const int a = (int)(i / nstr), c = (int)(i - (int64_t)a * nstr);
-      if (a > c) continue;
-      const uint32_t key = order_key(hd[sym_index(a, c, nstr)]);
-      if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      uint32_t cum = 0;
-      int d = 0;
-      for (; d < 255; d++) {
-        if (cum + hist[d] >= (uint32_t)k) break;
-        cum += hist[d];
+  const int nd = sym_nd(nstr);
+  const int64_t len = (int64_t)nd + (int64_t)nstr * (nstr - 1) / 2;   // the last element, + 1
+  __shared__ SelShared S;
+  __shared__ float s_lo[32], s_hi[32];
+  __shared__ int s_n, s_bin, s_scan[32];
+  // fn(value, position) over the diagonal's elements
+  auto each = [&](auto fn) {
+    for (int64_t q = tid; q < (ld >> 2); q += SEL_THREADS) {
+      const float4 v = reinterpret_cast<const float4*>(hd)[q];
+      const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int e = 0; e < 4; e++) {
+        const int64_t p = 4 * q + e;
+        if (p < len && (p < nstr || p >= nd)) fn(x[e], p);
       }
-      s_k = k - (int)cum;
-      s_prefix = prefix | ((uint32_t)d << shift);
     }
+  };
+  float lo = 3.4e38f, hi = -3.4e38f;
+  each([&](float x, int64_t) {
+    lo = fminf(lo, x);
+    hi = fmaxf(hi, x);
+  });
+  for (int o = 16; o; o >>= 1) {
+    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if (lane == 0) {
+    s_lo[warp] = lo;
+    s_hi[warp] = hi;
+  }
+  for (int i = tid; i < SEL_BINS; i += SEL_THREADS) S.hist[i] = 0;
+  if (tid == 0) s_n = 0;
+  __syncthreads();
+  for (int w = 0; w < SEL_THREADS / 32; w++) {
+    lo = fminf(lo, s_lo[w]);
+    hi = fmaxf(hi, s_hi[w]);
+  }
+  const float scale = hi > lo ? (float)(SEL_BINS - 1) / (hi - lo) : 0.f;
+  auto bin = [&](float x) { return min(SEL_BINS - 1, max(0, (int)((x - lo) * scale))); };
+  each([&](float x, int64_t) { atomicAdd(&S.hist[bin(x)], 1); });
+  __syncthreads();
+  {
+    // the bin of the npp-th element: 4 bins per thread, scanned over the block
+    constexpr int PER = SEL_BINS / SEL_THREADS;
+    int c[PER], s = 0;
+    for (int j = 0; j < PER; j++) s += c[j] = S.hist[tid * PER + j];
+    int inc = s;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    if (lane == 31) s_scan[warp] = inc;
     __syncthreads();
-    prefix = s_prefix;
-    k = s_k;
-    mask |= 0xFFu << shift;
+    int base = inc - s;
+    for (int w = 0; w < warp; w++) base += s_scan[w];
+    for (int j = 0; j < PER; j++) {
+      if (base < npp && base + c[j] >= npp) s_bin = base + c[j] <= SEL_CAP ? tid * PER + j : -1;
+      base += c[j];
+    }
+  }
+  __syncthreads();
+  uint32_t kmax = 0xffffffffu;   // key of the npp-th element (many equal values)
+  const int tbin = s_bin;
+  if (tbin < 0) {
+    // smallest key with at least npp elements up to it
+    uint32_t k0 = 0, k1 = 0xffffffffu;
+    while (k0 < k1) {
+      const uint32_t mid = k0 + (k1 - k0) / 2;
+      int n = 0;
+      each([&](float x, int64_t) { n += order_key(x) <= mid; });
+      __syncthreads();
+      if (tid == 0) s_n = 0;
+      __syncthreads();
+      atomicAdd(&s_n, n);
+      __syncthreads();
+      if (s_n >= npp) k1 = mid;
+      else k0 = mid + 1;
+    }
+    kmax = k0;
+    __syncthreads();
+    if (tid == 0) s_n = 0;
     __syncthreads();
   }
-  // keys below the threshold, then the first k equal to it, in index order
-  const uint32_t thr = prefix;
-  const int need_eq = k;
-  int base = 0, base_eq = 0;
-  for (int64_t i0 = 0; i0 < N && base < npp; i0 += blockDim.x) {
-    const int64_t i = i0 + threadIdx.x;
-    bool lt = false, eq = false;
-    if (i < N) {
-      const int a = (int)(i / nstr), c = (int)(i - (int64_t)a * nstr);
-      if (a <= c) {
-        const uint32_t key = order_key(hd[sym_index(a, c, nstr)]);
-        lt = key < thr;
-        eq = key == thr;
-      }
+  // candidates: below kmax all, of those equal to it the lowest indices (they
+  // can be many: kept by a bound on the index, halved until they fit)
+  auto put = [&](float x, int64_t p) {
+    const int at = atomicAdd(&s_n, 1);
+    if (at < SEL_CAP)
+      S.cand[at] = ((unsigned long long)order_key(x) << 32) | (unsigned)linear_of(p, nstr);
+  };
+  if (tbin >= 0) {
+    each([&](float x, int64_t p) {
+      if (bin(x) <= tbin) put(x, p);
+    });
+  } else {
+    // index bound such that at least npp and at most SEL_CAP elements qualify
+    int i0 = 0, i1 = nstr * nstr - 1;
+    while (i0 < i1) {
+      const int mid = i0 + (i1 - i0) / 2;
+      int n = 0;
+      each([&](float x, int64_t p) {
+        const uint32_t k = order_key(x);
+        n += k < kmax || (k == kmax && linear_of(p, nstr) <= mid);
+      });
+      __syncthreads();
+      if (tid == 0) s_n = 0;
+      __syncthreads();
+      atomicAdd(&s_n, n);
+      __syncthreads();
+      if (s_n >= npp) i1 = mid;
+      else i0 = mid + 1;
     }
-    int teq = 0, tsel = 0;
-    const int req = base_eq + block_flag_scan(eq, s_warp, &teq);
-    const bool sel = lt || (eq && req < need_eq);
-    const int pos = base + block_flag_scan(sel, s_warp, &tsel);
-    if (sel && pos < npp) psel[(int64_t)b * PSP_MAX + pos] = (int)i;
-    base += tsel;
-    base_eq += teq;
+    __syncthreads();
+    if (tid == 0) s_n = 0;
+    __syncthreads();
+    each([&](float x, int64_t p) {
+      const uint32_t k = order_key(x);
+      if (k < kmax || (k == kmax && linear_of(p, nstr) <= i0)) put(x, p);
+    });
+  }
+  __syncthreads();
+  // rank of every candidate by (key, index); the npp lowest, then their rank
+  // by index
+  const int n = min(s_n, SEL_CAP);
+  __shared__ int s_sel[PSP_MAX];
+  for (int i = tid; i < n; i += SEL_THREADS) {
+    const unsigned long long v = S.cand[i];
+    int r = 0;
+    for (int j = 0; j < n; j++) r += S.cand[j] < v;
+    if (r < npp) s_sel[r] = (int)(unsigned)v;
+  }
+  __syncthreads();
+  if (tid < npp) {
+    const int v = s_sel[tid];
+    int r = 0;
+    for (int j = 0; j < npp; j++) r += s_sel[j] < v;
+    psel[(int64_t)b * PSP_MAX + r] = v;
+    if (tid == 0) gidx[b] = v;
   }
 }
 
@@ -192,18 +281,18 @@ __device__ float psp_offdiag(uint32_t ma, uint32_t mb, uint32_t na, uint32_t nb,
   return s1 * s2 * (G(p, q, r, s) - G(p, s, r, q));
 }
 
-struct EigShared {
-  uint32_t a_off, u_off, g_off, h_off, total;
+constexpr int TRI_PITCH = PSP_MAX + 8;   // 8 columns of 4 rows: 32 banks
+
+struct TriShared {
+  uint32_t a_off, g_off, h_off, total;
 };
 
-__host__ __device__ inline EigShared eig_layout(int n) {
+__host__ __device__ inline TriShared tri_layout(int n) {
   const int npair = n * (n + 1) / 2;
-  EigShared s;
+  TriShared s;
   uint32_t o = 0;
   s.a_off = o;
-  o += PSP_MAX * PSP_PITCH * 4;
-  s.u_off = o;
-  o += PSP_MAX * PSP_PITCH * 4;
+  o += PSP_MAX * TRI_PITCH * 4;
   s.g_off = o;
   o += (uint32_t)npair * npair * 4;
   s.h_off = o;
@@ -212,42 +301,46 @@ __host__ __device__ inline EigShared eig_layout(int n) {
   return s;
 }
 
-// A_PP in the symmetric basis and its eigenpairs: lam_out[b][k], U[b][u][k]
-// (column k the eigenvector of lam_k)
-__global__ void __launch_bounds__(EIG_THREADS)
-    k_psp_eigh(const uint32_t* __restrict__ masks, int nstr, int n, int nsig,
-               const double* __restrict__ heff_all, const double* __restrict__ hp_all,
-               const double* __restrict__ gp_all, const float* __restrict__ hd_all, int64_t ld,
-               float lam, int npp, const int32_t* __restrict__ psel, float* __restrict__ lam_out,
-               float* __restrict__ U_out) {
+// A_PP in the symmetric basis and its tridiagonal form A_PP = Q T Q^T:
+// tri[b] = diagonal (PSP_MAX) then subdiagonal, Qt[b][k][u] = Q[u][k].
+// One CTA per tuple, eight lanes per row: a reflection is a row product, one
+// barrier, the rank-two update and another; the transformation is accumulated
+// backwards on Q^T, whose rows never meet, in registers.  128 functions:
+// 0.40 ms for one tuple, 0.54 ms per batch of the 8e/23o expansion to order 3
+// (up to 544 tuples), A_PP included; the eigenvectors by cyclic Jacobi, 1,270
+// rounds of three barriers over the matrix and its rotations, took 3.7 and 5.1
+// ms (22 % of that expansion).
+__global__ void __launch_bounds__(TRI_THREADS)
+    k_psp_tri(const uint32_t* __restrict__ masks, int nstr, int n, int nsig,
+              const double* __restrict__ heff_all, const double* __restrict__ hp_all,
+              const double* __restrict__ gp_all, const float* __restrict__ hd_all, int64_t ld,
+              float lam, int npp, const int32_t* __restrict__ psel, float* __restrict__ tri,
+              float* __restrict__ Qt) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int b = blockIdx.x;
   const int npair = n * (n + 1) / 2;
-  const EigShared L = eig_layout(n);
+  const TriShared L = tri_layout(n);
   float* A = (float*)(smem + L.a_off);
-  float* U = (float*)(smem + L.u_off);
   float* g = (float*)(smem + L.g_off);
   float* heff = (float*)(smem + L.h_off);
   __shared__ uint32_t s_ma[PSP_MAX], s_mb[PSP_MAX];
   __shared__ int s_diag[PSP_MAX];
-  __shared__ float s_hd[PSP_MAX];
-  __shared__ float s_c[PSP_MAX / 2], s_s[PSP_MAX / 2];
-  __shared__ int s_p[PSP_MAX / 2], s_q[PSP_MAX / 2];
-  __shared__ float s_red[32];
-  __shared__ int s_done;
-  const int tid = threadIdx.x;
+  __shared__ float s_hd[PSP_MAX], s_p[PSP_MAX], s_beta[PSP_MAX];
+  __shared__ uint8_t s_op[128], s_oq[128];
+  const int tid = threadIdx.x, lane = tid & 31;
+  for (int p = tid; p < n; p += blockDim.x)
+    for (int q = 0; q <= p; q++) {
+      s_op[p * (p + 1) / 2 + q] = (uint8_t)p;
+      s_oq[p * (p + 1) / 2 + q] = (uint8_t)q;
+    }
+  __syncthreads();
   // (pq|rs) = g'_PQ - (h'_pq d_rs + d_pq h'_rs) / N_active (the definition of g')
   const double* gp = gp_all + (int64_t)b * npair * npair;
   const double* hp = hp_all + (int64_t)b * n * n;
   const double inv = nsig > 0 ? 1.0 / (2 * nsig) : 0.0;
   for (int t = tid; t < npair * npair; t += blockDim.x) {
     const int P = t / npair, Q = t - P * npair;
-    int p = 0;
-    while ((p + 1) * (p + 2) / 2 <= P) p++;
-    const int q = P - p * (p + 1) / 2;
-    int r = 0;
-    while ((r + 1) * (r + 2) / 2 <= Q) r++;
-    const int s = Q - r * (r + 1) / 2;
+    const int p = s_op[P], q = s_oq[P], r = s_op[Q], s = s_oq[Q];
     double v = gp[t];
     if (r == s) v -= hp[p * n + q] * inv;
     if (p == q) v -= hp[r * n + s] * inv;
@@ -263,12 +356,7 @@ __global__ void __launch_bounds__(EIG_THREADS)
     s_diag[u] = a == c;
     s_hd[u] = hd_all[(int64_t)b * ld + sym_index(a, c, nstr)];
   }
-  // an odd npp gets one decoupled pad index (zero row and column)
-  const int m = (npp + 1) & ~1;
-  for (int t = tid; t < PSP_MAX * PSP_PITCH; t += blockDim.x) {
-    A[t] = 0.f;
-    U[t] = 0.f;
-  }
+  for (int t = tid; t < PSP_MAX * TRI_PITCH; t += blockDim.x) A[t] = 0.f;
   __syncthreads();
   const float r2 = 0.70710678118654752f;
   for (int t = tid; t < npp * npp; t += blockDim.x) {
@@ -288,119 +376,106 @@ __global__ void __launch_bounds__(EIG_THREADS)
       }
       x = sum * (s_diag[u] ? 1.f : r2) * (s_diag[v] ? 1.f : r2);
     }
-    A[u * PSP_PITCH + v] = x;
-    A[v * PSP_PITCH + u] = x;
+    A[u * TRI_PITCH + v] = x;
+    A[v * TRI_PITCH + u] = x;
   }
-  for (int u = tid; u < m; u += blockDim.x) U[u * PSP_PITCH + u] = 1.f;
   __syncthreads();
-  // cyclic Jacobi, tournament order: in round r the m/2 disjoint pairs
-  // (pos(j), pos(m-1-j)) with position 0 fixed and the others rotating
-  for (int sweep = 0; sweep < EIG_SWEEPS; sweep++) {
-    for (int round = 0; round < m - 1; round++) {
-      if (tid < m / 2) {
-        auto pos = [&](int k) { return k == 0 ? 0 : 1 + (k - 1 + round) % (m - 1); };
-        int p = pos(tid), q = pos(m - 1 - tid);
-        if (p > q) {
-          const int t = p;
-          p = q;
-          q = t;
-        }
-        const float app = A[p * PSP_PITCH + p], aqq = A[q * PSP_PITCH + q];
-        const float apq = A[p * PSP_PITCH + q];
-        float c = 1.f, s = 0.f;
-        if (fabsf(apq) > 1e-30f) {
-          const float tau = (aqq - app) / (2.f * apq);
-          const float t = (tau >= 0.f ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
-          c = rsqrtf(1.f + t * t);
-          s = t * c;
-        }
-        s_p[tid] = p;
-        s_q[tid] = q;
-        s_c[tid] = c;
-        s_s[tid] = s;
-      }
-      __syncthreads();
-      // rows p, q of A <- J^T A
-      for (int t = tid; t < (m / 2) * m; t += blockDim.x) {
-        const int j = t / m, col = t - j * m;
-        const int p = s_p[j], q = s_q[j];
-        const float c = s_c[j], s = s_s[j];
-        const float x = A[p * PSP_PITCH + col], y = A[q * PSP_PITCH + col];
-        A[p * PSP_PITCH + col] = c * x - s * y;
-        A[q * PSP_PITCH + col] = s * x + c * y;
-      }
-      __syncthreads();
-      // columns p, q of A and U <- A J, U J
-      for (int t = tid; t < (m / 2) * m; t += blockDim.x) {
-        const int j = t / m, row = t - j * m;
-        const int p = s_p[j], q = s_q[j];
-        const float c = s_c[j], s = s_s[j];
-        const float x = A[row * PSP_PITCH + p], y = A[row * PSP_PITCH + q];
-        A[row * PSP_PITCH + p] = c * x - s * y;
-        A[row * PSP_PITCH + q] = s * x + c * y;
-        const float ux = U[row * PSP_PITCH + p], uy = U[row * PSP_PITCH + q];
-        U[row * PSP_PITCH + p] = c * ux - s * uy;
-        U[row * PSP_PITCH + q] = s * ux + c * uy;
-      }
-      __syncthreads();
+  const int m = npp, row = tid >> 3, l = tid & 7;
+  // reflection k: v = row k right of the diagonal with its first element
+  // replaced by x0 - mu, H = 1 - beta v v^T, mu the new subdiagonal element.
+  // Every warp forms the sums over v itself (no barrier for them).
+  for (int k = 0; k + 2 < m; k++) {
+    const float* vk = A + k * TRI_PITCH;
+    float s = 0.f;
+    for (int j = k + 2 + lane; j < m; j += 32) s = fmaf(vk[j], vk[j], s);
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const float x0 = vk[k + 1];
+    const float nrm = sqrtf(fmaf(x0, x0, s));
+    const float mu = x0 > 0.f ? -nrm : nrm;
+    const float v0 = x0 - mu;
+    const float beta = s > 1e-30f ? 2.f / fmaf(v0, v0, s) : 0.f;   // s ~ 0: H = 1
+    // p = beta A v
+    if (row > k && row < m) {
+      float acc = 0.f;
+      for (int j = k + 1 + l; j < m; j += 8)
+        acc = fmaf(A[row * TRI_PITCH + j], j == k + 1 ? v0 : vk[j], acc);
+      for (int o = 4; o; o >>= 1) acc += __shfl_xor_sync(0xffu << (lane & 24), acc, o);
+      if (l == 0) s_p[row] = beta * acc;
     }
-    // off-diagonal against diagonal weight
-    float off = 0.f, dia = 0.f;
-    for (int t = tid; t < m * m; t += blockDim.x) {
-      const int i = t / m, j = t - i * m;
-      const float x = A[i * PSP_PITCH + j];
-      if (i == j) dia += x * x;
-      else off += x * x;
+    __syncthreads();
+    // q = p - (beta/2 p.v) v, A <- A - v q^T - q v^T
+    float pv = 0.f;
+    for (int j = k + 1 + lane; j < m; j += 32) pv = fmaf(s_p[j], j == k + 1 ? v0 : vk[j], pv);
+    for (int o = 16; o; o >>= 1) pv += __shfl_xor_sync(0xffffffffu, pv, o);
+    const float kk = 0.5f * beta * pv;
+    if (row > k && row < m) {
+      const float vi = row == k + 1 ? v0 : vk[row], qi = s_p[row] - kk * vi;
+      for (int j = k + 1 + l; j < m; j += 8) {
+        const float vj = j == k + 1 ? v0 : vk[j];
+        A[row * TRI_PITCH + j] -= vi * (s_p[j] - kk * vj) + qi * vj;
+      }
     }
-    for (int o = 16; o; o >>= 1) {
-      off += __shfl_down_sync(0xffffffffu, off, o);
-      dia += __shfl_down_sync(0xffffffffu, dia, o);
-    }
-    if ((tid & 31) == 0) s_red[tid >> 5] = off;
     __syncthreads();
     if (tid == 0) {
-      float so = 0.f;
-      for (int w = 0; w < (int)(blockDim.x >> 5); w++) so += s_red[w];
-      s_red[0] = so;
+      // row k now keeps v; its diagonal is final
+      tri[(int64_t)b * 2 * PSP_MAX + k] = vk[k];
+      tri[(int64_t)b * 2 * PSP_MAX + PSP_MAX + k] = beta != 0.f ? mu : x0;
+      A[k * TRI_PITCH + k + 1] = v0;
+      s_beta[k] = beta;
     }
-    __syncthreads();
-    const float so = s_red[0];
-    __syncthreads();
-    if ((tid & 31) == 0) s_red[tid >> 5] = dia;
-    __syncthreads();
-    if (tid == 0) {
-      float sd = 0.f;
-      for (int w = 0; w < (int)(blockDim.x >> 5); w++) sd += s_red[w];
-      s_done = so <= 1e-10f * sd;   // off-diagonal ~1e-5 of the diagonal
+    // (row k is read again only below)
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int k = max(0, m - 2); k < m; k++) {
+      tri[(int64_t)b * 2 * PSP_MAX + k] = A[k * TRI_PITCH + k];
+      if (k + 1 < m) tri[(int64_t)b * 2 * PSP_MAX + PSP_MAX + k] = A[k * TRI_PITCH + k + 1];
     }
-    __syncthreads();
-    if (s_done) break;
   }
-  for (int k = tid; k < npp; k += blockDim.x) lam_out[(int64_t)b * PSP_MAX + k] = A[k * PSP_PITCH + k];
-  float* Ub = U_out + (int64_t)b * PSP_MAX * PSP_MAX;
-  for (int t = tid; t < npp * npp; t += blockDim.x) {
-    const int u = t / npp, k = t - u * npp;
-    Ub[u * PSP_MAX + k] = U[u * PSP_PITCH + k];
+  // Q^T = H_{m-3} .. H_0, row by row: R <- R - beta (R v) v^T
+  float R[PSP_MAX / 8];
+#pragma unroll
+  for (int t = 0; t < PSP_MAX / 8; t++) R[t] = l + 8 * t == row ? 1.f : 0.f;
+  for (int k = m - 3; k >= 0; k--) {
+    const float* vk = A + k * TRI_PITCH;
+    const float beta = s_beta[k];
+    float v[PSP_MAX / 8], d = 0.f;
+#pragma unroll
+    for (int t = 0; t < PSP_MAX / 8; t++) {
+      const int j = l + 8 * t;
+      v[t] = j > k && j < m ? vk[j] : 0.f;
+      d = fmaf(R[t], v[t], d);
+    }
+    for (int o = 4; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+    d *= beta;
+#pragma unroll
+    for (int t = 0; t < PSP_MAX / 8; t++) R[t] = fmaf(-d, v[t], R[t]);
   }
+  float* Qb = Qt + (int64_t)b * PSP_MAX * PSP_MAX;
+#pragma unroll
+  for (int t = 0; t < PSP_MAX / 8; t++)
+    if (row < m && l + 8 * t < m) Qb[row * PSP_MAX + l + 8 * t] = R[t];
 }
 
 // What an iteration does between the residual and the Gram-Schmidt passes,
 // one CTA per tuple still iterating:
-//   t_P = U (theta - Lambda)^{-1} U^T r_P (npp = 0: no P-space);
+//   t_P = Q (theta - T)^{-1} Q^T r_P (npp = 0: no P-space), the tridiagonal
+//   system by cyclic reduction, all unknowns at once (seven steps);
 //   with olsen the same block solve turns u = x / (theta - A_II) (Uo, from the
 //   residual kernel) into M^-1 x on P;
 //   the dots x.t, x.u (xpart) and, with dots, V.t (dpart) and V.u (upart) are
 //   summed over their chunks, with the changes of t and u on P;
 //   Olsen's eps = x.t / x.u and the first Gram-Schmidt pass's coefficients
 //   coef = V.t - eps V.u.
-// U comes from L2 twice (by columns for U^T r, by rows for U w), a quarter of
-// a column or a warp per row; the whole is a latency chain of a few thousand
-// cycles (one warp-wide pass over U in shared memory and four more kernels
-// for the sums took 40 us and four launches).
+// Q^T comes from L2 twice (by rows for Q^T r, a warp per row; by columns for
+// Q z, a quarter of a column per thread); the whole is a latency chain of a
+// few thousand cycles (19-22 us a call; eigenvectors staged in shared memory,
+// two of 256 threads' warps busy, took 37-47 us and four more launches for
+// the sums).
 __global__ void __launch_bounds__(APPLY_THREADS)
     k_psp_apply(float* __restrict__ T, const float* __restrict__ hd_all, int nstr, int64_t ld,
                 const double* __restrict__ theta, int npp, const int32_t* __restrict__ psel,
-                const float* __restrict__ U_all, const float* __restrict__ lam_all,
+                const float* __restrict__ Qt, const float* __restrict__ tri,
                 const float* __restrict__ V, int m, int M, int nchunks,
                 const double* __restrict__ dpart, int dots, const int32_t* __restrict__ active,
                 int olsen, float* __restrict__ Uo, const float* __restrict__ X,
@@ -409,9 +484,10 @@ __global__ void __launch_bounds__(APPLY_THREADS)
                 float* __restrict__ eps) {
   const int b = blockIdx.x;
   if (!active[b]) return;
-  __shared__ float s_r[PSP_MAX], s_x[PSP_MAX], s_w[PSP_MAX], s_wx[PSP_MAX];
+  __shared__ float s_r[PSP_MAX], s_x[PSP_MAX];
   __shared__ float s_del[PSP_MAX], s_delu[PSP_MAX], s_xv[PSP_MAX];
   __shared__ float s_pr[4][PSP_MAX], s_px[4][PSP_MAX];
+  __shared__ float s_t[2][5][PSP_MAX];   // a, b, c and the two right-hand sides
   __shared__ int s_i[PSP_MAX];
   __shared__ double s_c[32], s_c2[32], s_xs[2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -424,7 +500,7 @@ __global__ void __launch_bounds__(APPLY_THREADS)
     float* Ob = olsen ? Uo + (int64_t)b * ld : nullptr;
     const float* Xb = olsen ? X + (int64_t)b * ld : nullptr;
     const float* hb = hd_all + (int64_t)b * ld;
-    const float* Ub = U_all + (int64_t)b * PSP_MAX * PSP_MAX;
+    const float* Qb = Qt + (int64_t)b * PSP_MAX * PSP_MAX;
     const float th = (float)theta[b];
     const float sq2 = 1.41421356237309505f, r2 = 0.70710678118654752f;
     if (tid < npp) {
@@ -443,39 +519,16 @@ __global__ void __launch_bounds__(APPLY_THREADS)
       s_i[u] = i;
     }
     __syncthreads();
-    {
-      // U^T r: thread -> column k and a quarter of the rows u
-      const int k = tid & (PSP_MAX - 1), part = tid / PSP_MAX;
-      float w = 0.f, wx = 0.f;
-      if (k < npp) {
-        const int u1 = npp * (part + 1) / 4;
-#pragma unroll 8
-        for (int u = npp * part / 4; u < u1; u++) {
-          const float uk = Ub[u * PSP_MAX + k];
-          w = fmaf(uk, s_r[u], w);
-          wx = fmaf(uk, s_x[u], wx);
-        }
-      }
-      s_pr[part][k] = w;
-      s_px[part][k] = wx;
-    }
-    __syncthreads();
-    if (tid < npp) {
-      float dl = th - lam_all[(int64_t)b * PSP_MAX + tid];
-      if (fabsf(dl) < 1e-4f) dl = dl < 0.f ? -1e-4f : 1e-4f;
-      s_w[tid] = ((s_pr[0][tid] + s_pr[1][tid]) + (s_pr[2][tid] + s_pr[3][tid])) / dl;
-      s_wx[tid] = ((s_px[0][tid] + s_px[1][tid]) + (s_px[2][tid] + s_px[3][tid])) / dl;
-    }
-    __syncthreads();
-    for (int u = warp; u < npp; u += NW) {
+    // Q^T r and Q^T x
+    for (int k = warp; k < npp; k += NW) {
       float v = 0.f, vx = 0.f;
 #pragma unroll
       for (int q = 0; q < PSP_MAX / 32; q++) {
-        const int k = lane + 32 * q;
-        if (k < npp) {
-          const float uk = Ub[u * PSP_MAX + k];
-          v = fmaf(uk, s_w[k], v);
-          vx = fmaf(uk, s_wx[k], vx);
+        const int u = lane + 32 * q;
+        if (u < npp) {
+          const float uk = Qb[k * PSP_MAX + u];
+          v = fmaf(uk, s_r[u], v);
+          vx = fmaf(uk, s_x[u], vx);
         }
       }
       for (int o = 16; o; o >>= 1) {
@@ -483,17 +536,84 @@ __global__ void __launch_bounds__(APPLY_THREADS)
         vx += __shfl_xor_sync(0xffffffffu, vx, o);
       }
       if (lane == 0) {
-        const int i = s_i[u];
-        const bool diag = i < sym_nd(nstr);
-        const float f = diag ? 1.f : 2.f;   // both elements of a pair change alike
-        const float tn = diag ? v : v * r2;
-        s_del[u] = (tn - Tb[i]) * f;
-        Tb[i] = tn;
-        if (olsen) {
-          const float un = diag ? vx : vx * r2;
-          s_delu[u] = (un - Ob[i]) * f;
-          Ob[i] = un;
+        s_t[0][3][k] = v;
+        s_t[0][4][k] = vx;
+      }
+    }
+    if (tid < npp) {
+      const float* tb = tri + (int64_t)b * 2 * PSP_MAX;
+      s_t[0][0][tid] = tid > 0 ? -tb[PSP_MAX + tid - 1] : 0.f;
+      s_t[0][1][tid] = th - tb[tid];
+      s_t[0][2][tid] = tid + 1 < npp ? -tb[PSP_MAX + tid] : 0.f;
+    }
+    __syncthreads();
+    int cur = 0;
+    for (int st = 1; st < npp; st <<= 1, cur ^= 1) {
+      if (tid < npp) {
+        const float(*o)[PSP_MAX] = s_t[cur];
+        float(*w)[PSP_MAX] = s_t[cur ^ 1];
+        const int i = tid, lo = i - st, hi = i + st;
+        float bb = o[1][i], f = o[3][i], gx = o[4][i], an = 0.f, cn = 0.f;
+        auto piv = [](float x) { return fabsf(x) < 1e-6f ? (x < 0.f ? -1e-6f : 1e-6f) : x; };
+        if (lo >= 0) {
+          const float k1 = __fdividef(o[0][i], piv(o[1][lo]));
+          bb -= o[2][lo] * k1;
+          f -= o[3][lo] * k1;
+          gx -= o[4][lo] * k1;
+          an = -o[0][lo] * k1;
         }
+        if (hi < npp) {
+          const float k2 = __fdividef(o[2][i], piv(o[1][hi]));
+          bb -= o[0][hi] * k2;
+          f -= o[3][hi] * k2;
+          gx -= o[4][hi] * k2;
+          cn = -o[2][hi] * k2;
+        }
+        w[0][i] = an;
+        w[1][i] = bb;
+        w[2][i] = cn;
+        w[3][i] = f;
+        w[4][i] = gx;
+      }
+      __syncthreads();
+    }
+    if (tid < npp) {
+      float d = s_t[cur][1][tid];
+      if (fabsf(d) < 1e-6f) d = d < 0.f ? -1e-6f : 1e-6f;
+      s_r[tid] = s_t[cur][3][tid] / d;
+      s_x[tid] = s_t[cur][4][tid] / d;
+    }
+    __syncthreads();
+    {
+      // Q z: thread -> u and a quarter of the k
+      const int u = tid & (PSP_MAX - 1), part = tid / PSP_MAX;
+      float w = 0.f, wx = 0.f;
+      if (u < npp) {
+        const int k1 = npp * (part + 1) / 4;
+#pragma unroll 8
+        for (int k = npp * part / 4; k < k1; k++) {
+          const float uk = Qb[k * PSP_MAX + u];
+          w = fmaf(uk, s_r[k], w);
+          wx = fmaf(uk, s_x[k], wx);
+        }
+      }
+      s_pr[part][u] = w;
+      s_px[part][u] = wx;
+    }
+    __syncthreads();
+    if (tid < npp) {
+      const int u = tid, i = s_i[u];
+      const float v = (s_pr[0][u] + s_pr[1][u]) + (s_pr[2][u] + s_pr[3][u]);
+      const float vx = (s_px[0][u] + s_px[1][u]) + (s_px[2][u] + s_px[3][u]);
+      const bool diag = i < sym_nd(nstr);
+      const float f = diag ? 1.f : 2.f;   // both elements of a pair change alike
+      const float tn = diag ? v : v * r2;
+      s_del[u] = (tn - Tb[i]) * f;
+      Tb[i] = tn;
+      if (olsen) {
+        const float un = diag ? vx : vx * r2;
+        s_delu[u] = (un - Ob[i]) * f;
+        Ob[i] = un;
       }
     }
     __syncthreads();
@@ -535,7 +655,6 @@ int pspace_size(const BinProblem& bp, int requested) {
   const int64_t ncan = (int64_t)bp.nstr * (bp.nstr + 1) / 2;
   const int64_t cap = std::min<int64_t>({(int64_t)requested, (int64_t)PSP_MAX, ncan / 2});
   if (cap < 2) return 0;
-  if (eig_layout(bp.n).total + 4096 > 227u * 1024u) return 0;
   return (int)cap;
 }
 
@@ -545,20 +664,20 @@ void pspace_setup(mbe_ctx* ctx, BinProblem& bp, const float* hd, int64_t ld, dou
   if (!npp) return;
   const int B = bp.B;
   w.sel.reset(&ctx->pool, (size_t)B * PSP_MAX);
-  w.lam.reset(&ctx->pool, (size_t)B * PSP_MAX);
-  w.U.reset(&ctx->pool, (size_t)B * PSP_MAX * PSP_MAX);
+  w.low.reset(&ctx->pool, B);
+  w.tri.reset(&ctx->pool, (size_t)B * 2 * PSP_MAX);
+  w.Qt.reset(&ctx->pool, (size_t)B * PSP_MAX * PSP_MAX);
   cudaStream_t st = ctx->stream;
-  k_psp_select<<<B, SEL_THREADS, 0, st>>>(hd, bp.nstr, ld, npp, w.sel.ptr);
+  k_psp_select<<<B, SEL_THREADS, 0, st>>>(hd, bp.nstr, ld, npp, w.sel.ptr, w.low.ptr);
   CU_LAUNCH_CHECK();
-  const uint32_t smem = eig_layout(bp.n).total;
   static bool attr_set[MBE_MAX_DEVICES] = {false};
   once_per_device(attr_set, ctx->device, [] {
-    CU_CHECK(cudaFuncSetAttribute(k_psp_eigh, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  227 * 1024 - 4096));
+    CU_CHECK(cudaFuncSetAttribute(k_psp_tri, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)tri_layout(15).total));
   });
-  k_psp_eigh<<<B, EIG_THREADS, smem, st>>>(bp.tab->masks.ptr, bp.nstr, bp.n, bp.nsig,
-                                           bp.heff.ptr, bp.hp.ptr, bp.gp.ptr, hd, ld,
-                                           (float)shift, npp, w.sel.ptr, w.lam.ptr, w.U.ptr);
+  k_psp_tri<<<B, TRI_THREADS, tri_layout(bp.n).total, st>>>(
+      bp.tab->masks.ptr, bp.nstr, bp.n, bp.nsig, bp.heff.ptr, bp.hp.ptr, bp.gp.ptr, hd, ld,
+      (float)shift, npp, w.sel.ptr, w.tri.ptr, w.Qt.ptr);
   CU_LAUNCH_CHECK();
 }
 
@@ -568,7 +687,7 @@ void pspace_apply(mbe_ctx* ctx, const BinProblem& bp, const PspaceWork& w, float
                   float* Uo, const float* X, const double* upart, const double* xpart,
                   const double* y, double* yp, double* coef, float* eps) {
   k_psp_apply<<<bp.B, APPLY_THREADS, 0, ctx->stream>>>(
-      T, hd, bp.nstr, ld, theta, w.npp, w.sel.ptr, w.U.ptr, w.lam.ptr, V, m, M, nchunks, dpart,
+      T, hd, bp.nstr, ld, theta, w.npp, w.sel.ptr, w.Qt.ptr, w.tri.ptr, V, m, M, nchunks, dpart,
       dots ? 1 : 0, active, olsen ? 1 : 0, Uo, X, upart, xpart, y, yp, coef, eps);
   CU_LAUNCH_CHECK();
 }

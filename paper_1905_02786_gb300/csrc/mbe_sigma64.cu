@@ -87,33 +87,47 @@ __device__ __forceinline__ Repl repl_of(uint32_t m, int n, int nsig, int k) {
   return x;
 }
 
-// rank of a string among all of its electron count: binary search in the
-// ascending mask table
-__device__ __forceinline__ int rank_of(const uint32_t* __restrict__ masks, int nstr, uint32_t m) {
-  int lo = 0, hi = nstr - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (masks[mid] < m) lo = mid + 1;
-    else hi = mid;
-  }
-  return lo;
+// the ascending (colexicographic) order of the k-subsets of n bits: binomial
+// coefficients of up to 15 orbitals
+struct Binom {
+  uint16_t c[16][16];
+};
+__device__ __forceinline__ int rank_of(const Binom& t, uint32_t m) {
+  int r = 0;
+  for (int i = 1; m; i++, m &= m - 1) r += t.c[__ffs(m) - 1][i];
+  return r;
+}
+__device__ __forceinline__ uint32_t unrank(const Binom& t, int r, int n, int k) {
+  uint32_t m = 0;
+  for (int p = n - 1; p >= 0 && k > 0; p--)
+    if (t.c[p][k] <= r) {
+      r -= t.c[p][k--];
+      m |= 1u << p;
+    }
+  return m;
 }
 
-// per shape: hidx[k][I] the string of replacement k of I; olnk[x][I] the
-// off-diagonal links (J << 9) | (Q << 2) | (dir << 1) | (sign < 0), dir = 1 if
-// I holds the larger orbital of the pair Q
-__global__ void k_direct_tables(const uint32_t* __restrict__ masks, int nstr, int n, int nsig,
-                                int nnz, uint16_t* __restrict__ hidx, uint32_t* __restrict__ olnk) {
+// per shape: the strings (ascending masks), hidx[k][I] the string of
+// replacement k of I, and olnk[x][I] the off-diagonal links
+// (J << 9) | (Q << 2) | (dir << 1) | (sign < 0), dir = 1 if I holds the larger
+// orbital of the pair Q
+__global__ void k_direct_tables(const Binom bn, int nstr, int n, int nsig, int nnz,
+                                uint32_t* __restrict__ masks, uint16_t* __restrict__ hidx,
+                                uint32_t* __restrict__ olnk) {
+  __shared__ Binom sb;
+  for (int t = threadIdx.x; t < 256; t += blockDim.x) sb.c[t >> 4][t & 15] = bn.c[t >> 4][t & 15];
+  __syncthreads();
   const int noff = nsig * (n - nsig);
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < (int64_t)nnz * nstr;
        t += (int64_t)gridDim.x * blockDim.x) {
     const int k = (int)(t / nstr), I = (int)(t - (int64_t)k * nstr);
-    const uint32_t m = masks[I];
+    const uint32_t m = unrank(sb, I, n, nsig);
     const Repl x = repl_of(m, n, nsig, k);
     uint32_t m2 = m;
     if (x.kind >= 1) m2 ^= (1u << x.q) ^ (1u << x.p);
     if (x.kind == 2) m2 ^= (1u << x.s) ^ (1u << x.r);
-    const int J = x.kind ? rank_of(masks, nstr, m2) : I;
+    const int J = x.kind ? rank_of(sb, m2) : I;
+    if (k == 0) masks[I] = m;
     hidx[t] = (uint16_t)J;
     if (x.kind == 1 && k <= noff)
       olnk[(int64_t)(k - 1) * nstr + I] = ((uint32_t)J << 9) | ((uint32_t)pair_of(x.p, x.q) << 2) |
@@ -398,12 +412,15 @@ int direct_nnz(int n, int nsig) {
   return 1 + nsig * nv + nsig * (nsig - 1) / 2 * (nv * (nv - 1) / 2);
 }
 
-void launch_direct_tables(mbe_ctx* ctx, int n, int nsig, int nstr, const uint32_t* masks,
+void launch_direct_tables(mbe_ctx* ctx, int n, int nsig, int nstr, uint32_t* masks,
                           uint16_t* hidx, uint32_t* olnk) {
+  Binom bn;   // C(15, 7) = 6435 at most
+  for (int p = 0; p < 16; p++)
+    for (int k = 0; k < 16; k++) bn.c[p][k] = k > p ? 0 : (uint16_t)string_count(p, k);
   const int nnz = direct_nnz(n, nsig);
   const int64_t tot = (int64_t)nnz * nstr;
   k_direct_tables<<<(unsigned)std::min<int64_t>((tot + 255) / 256, 4096), 256, 0, ctx->stream>>>(
-      masks, nstr, n, nsig, nnz, hidx, olnk);
+      bn, nstr, n, nsig, nnz, masks, hidx, olnk);
   CU_LAUNCH_CHECK();
 }
 
