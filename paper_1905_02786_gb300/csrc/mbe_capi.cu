@@ -202,7 +202,13 @@ void solve_jobs(mbe_ctx* ctx, const std::vector<std::vector<int>>& acts, double*
     const bool mixed_bin = ctx->opt.precision == MBE_MIXED_BF16X3 && N > 1 && closed &&
                            sigma_tc_supported(n, tab->nstr) && ozaki_supported(tab->npair);
     const int Mm = mixed_subspace_alloc(ctx->opt.max_subspace);
-    double per = (mixed_bin ? (double)(4 * Mm + 46) * N + 128.0 * 129.0 * 4.0
+    // and, where its two-spin kernel takes the shape, the row sums and the
+    // packed words of the operand
+    const double nm1 =
+        mixed_bin && sigma_nm1_supported(n, nsig, tab->nstr, 1)
+            ? 4.0 * ((double)sigma_nm1_slot_floats(n, nsig, tab->nstr) +
+                     (double)tab->nstr * sigma_nm1_ldw(tab->nstr)) : 0.0;
+    double per = (mixed_bin ? (double)(4 * Mm + 46) * N + nm1 + 128.0 * 128.0 * 4.0
                             : (double)(2 * M + 6) * N * 8.0 +
                                   8.0 * (direct_nnz(n, nsig) * (double)tab->nstr +
                                          (direct_nnz(n, nsigb) + tabb->npair) *

@@ -239,6 +239,7 @@ k_sigma_exact(const int32_t* __restrict__ link, int nstr, int npair, int kpad,
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base_sh;
   const int Z = s_maxep + 2 - 48;
+  const bool leader = warp == 0 && elect_one();   // issues the MMAs
   const uint32_t idesc = make_idesc(EX_M, kpad);
   const uint32_t sbo = (uint32_t)(kpad >> 3) * 128u;
   const int nkb = kpad >> 3;
@@ -321,7 +322,7 @@ k_sigma_exact(const int32_t* __restrict__ link, int nstr, int npair, int kpad,
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     // ---- group accumulators: acc_s = sum_{i + j = s} D_i g'_j^T (columns s kpad)
-    if (tid == 0) {
+    if (leader) {
       const uint32_t d0 = smem_u32(sD), g0 = smem_u32(sG);
       for (int ks = 0; ks < (kpad >> 4); ks++) {
         const uint32_t koff = (uint32_t)ks * 256u;

@@ -252,6 +252,13 @@ struct StringTables {
   // (poff, ntiles + 1 per string)
   DevBuf<int16_t> plist;
   DevBuf<int32_t> poff;
+  // two-spin kernel over (N-1)-electron strings (mbe_sigma_nm1.cu, built on
+  // first use): those strings, their one-electron additions (16 per string),
+  // the first string with a larger mask, and the slot row of every electron
+  // of every string
+  DevBuf<uint32_t> kmask;
+  DevBuf<int32_t> krow, kj0;
+  DevBuf<int2> srow;
   // FP64 sigma (mbe_sigma64.cu, built on first use): replacements of every
   // string and its off-diagonal links, string index fastest
   DevBuf<uint16_t> hidx;
@@ -411,6 +418,7 @@ struct BinProblem {
   DevBuf<double> gp;             // B * npair * npair
   DevBuf<double> jk;             // B * 2 * n * n  (J_pq = (pp|qq), K_pq = (pq|qp))
   DevBuf<uint8_t> gsplit;        // g'/2 as bf16 hi/lo rows (tensor-core sigma operand source)
+  DevBuf<uint8_t> nmop;          // operand M of the (N-1)-electron two-spin kernel
   DevBuf<uint8_t> haa;           // one-spin Hamiltonian H^alpha as bf16 hi/lo rows
   // FP64 sigma: non-zero one-spin elements of the alpha (and, for an open
   // shell, beta) strings and the pair integrals summed over a beta string
@@ -496,6 +504,8 @@ struct SigmaWork {
   DevBuf<double> D, E;           // scratch of the emulated FP64 path
   DevBuf<float> Xf;              // W rows of the tensor-core path (sigma = W + W^T)
   DevBuf<uint8_t> csplit;        // the vectors as bf16 hi/lo rows (tensor-core operands)
+  DevBuf<uint32_t> cw;           // and as hi | lo words (two-spin kernel's gathers)
+  DevBuf<float> slots;           // its finished row sums
   DevBuf<int32_t> err;           // timeout flag of the tensor-core path
   DevBuf<uint8_t> gex;           // g' digit planes of the fused exact sigma
   DevBuf<int32_t> gexp;          // their row exponents
@@ -510,6 +520,21 @@ void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, float* c, int64_t c_st
               float* out, int64_t out_stride, const int32_t* active, double spin_shift,
               bool packed = false, const float* T = nullptr, const double* inv = nullptr);
 int32_t sigma_tc_error(mbe_ctx* ctx, SigmaWork& w);
+// two-spin part over pairs of (N-1)-electron strings (mbe_sigma_nm1.cu): the
+// shapes it takes, the floats of row sums per tuple, its TMEM operand stages
+bool sigma_nm1_supported(int n, int nsig, int nstr, int B);
+int64_t sigma_nm1_slot_floats(int n, int nsig, int nstr);
+int sigma_nm1_stages(int n, int nsig, int nstr, int B);
+int sigma_nm1_ldw(int nstr);   // words per row of w.cw
+// tables, operand and buffers (w.cw is filled by the split of c)
+void sigma_nm1_prepare(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, double shift);
+// row sums from w.cw into w.slots; stages: 2.. (0: the most)
+void sigma_nm1(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, const int32_t* active, int nsm,
+               int stages);
+// sigma = X + X^T + shift nsig c, X = w.Xf + row sums
+void sigma_nm1_finish(mbe_ctx* ctx, const BinProblem& bp, const SigmaWork& w, int64_t w_stride,
+                      const float* c, int64_t c_stride, double shift, const int32_t* active,
+                      float* out, int64_t out_stride, bool packed);
 // subspace vectors allocated per tuple by the mixed Davidson: max_subspace
 // (clamped to 4..32) for its first stage and its refinement rounds, up to 12
 // more (at most 32) for the rounds after one that filled its subspace

@@ -29,7 +29,10 @@
 //                n_link pairs that link a, the same count for every string);
 //                the product for 128 column strings lands in TMEM and the
 //                scatter through the link table of the column strings adds
-//                it into row a of W (columns J >= a) in shared memory;
+//                it into row a of W (columns J >= a) in shared memory; for 4,
+//                13 and more orbitals.  For 5 to 12 the two-spin part is
+//                k_sigma_nm1 over (N-1)-electron strings (mbe_sigma_nm1.cu),
+//                2 to 2.7 times faster;
 //   k_sigma_tc_finish  sigma = W + W^T + shift S^2 c.
 // Both products run as split-BF16x3 (hi*hi + lo*hi + hi*lo, FP32
 // accumulation in TMEM): ~16 significant bits per operand, sigma to ~1e-4 of
@@ -75,13 +78,15 @@ __device__ __forceinline__ bool bar_red_or(int id, int n, bool pred) {
 
 // ------------------------------------------------------------ c split
 // c (rows of nstr FP32) -> bf16 hi rows then lo rows of ldc elements (zeros
-// beyond nstr); cs_stride elements between tuples
+// beyond nstr); cs_stride elements between tuples; cw (unless NULL): the same
+// as words hi | lo << 16, ldw per row
 __global__ void k_split_c(const float* __restrict__ c, int64_t c_stride, int nstr, int ldc,
                           const int32_t* __restrict__ active, bf16* __restrict__ cs,
-                          int64_t cs_stride) {
+                          int64_t cs_stride, uint32_t* __restrict__ cw, int ldw) {
   const int b = blockIdx.y;
   if (active && !active[b]) return;
   const float* cb = c + (int64_t)b * c_stride;
+  uint32_t* wb = cw ? cw + (int64_t)b * nstr * ldw : nullptr;
   bf16* hi = cs + (int64_t)b * cs_stride;
   bf16* lo = hi + (int64_t)nstr * ldc;
   const int chunks = ldc >> 3;
@@ -100,6 +105,10 @@ __global__ void k_split_c(const float* __restrict__ c, int64_t c_stride, int nst
     }
     *reinterpret_cast<uint4*>(hi + (int64_t)r * ldc + k0) = hv;
     *reinterpret_cast<uint4*>(lo + (int64_t)r * ldc + k0) = lv;
+    if (wb)
+      for (int q = 0; q < 8 && k0 + q < nstr; q++)
+        wb[(int64_t)r * ldw + k0 + q] =
+            __byte_perm(hw[q >> 1], lw[q >> 1], (q & 1) ? 0x7632 : 0x5410);
   }
 }
 
@@ -112,9 +121,19 @@ __global__ void k_split_c(const float* __restrict__ c, int64_t c_stride, int nst
 __global__ void k_split_c_sym(float* __restrict__ c, int64_t c_stride, const float* __restrict__ T,
                               int64_t t_stride, const double* __restrict__ inv, int nstr, int ldc,
                               const int32_t* __restrict__ active, bf16* __restrict__ cs,
-                              int64_t cs_stride) {
+                              int64_t cs_stride, uint32_t* __restrict__ cw, int ldw) {
   const int b = blockIdx.y;
   if (active && !active[b]) return;
+  uint32_t* wb = cw ? cw + (int64_t)b * nstr * ldw : nullptr;
+  auto put = [&](bf16* hi, bf16* lo, int r, int k, float x) {
+    const bf16 h = __float2bfloat16_rn(x);
+    const bf16 l = __float2bfloat16_rn(x - __bfloat162float(h));
+    hi[(int64_t)r * ldc + k] = h;
+    lo[(int64_t)r * ldc + k] = l;
+    if (wb && k < nstr)
+      wb[(int64_t)r * ldw + k] =
+          (uint32_t)__bfloat16_as_ushort(h) | ((uint32_t)__bfloat16_as_ushort(l) << 16);
+  };
   const int nt = (nstr + 31) / 32;
   int t = blockIdx.x, I = 0;
   while (t >= nt - I) {
@@ -146,23 +165,13 @@ __global__ void k_split_c_sym(float* __restrict__ c, int64_t c_stride, const flo
   // rows of tile I, columns of tile J (zeros from nstr up to ldc)
   for (int i = ty; i < 32; i += ny) {
     const int r = I * 32 + i, k = J * 32 + tx;
-    if (r < nstr && k < ldc) {
-      const float x = sC[i][tx];
-      const bf16 h = __float2bfloat16_rn(x);
-      hi[(int64_t)r * ldc + k] = h;
-      lo[(int64_t)r * ldc + k] = __float2bfloat16_rn(x - __bfloat162float(h));
-    }
+    if (r < nstr && k < ldc) put(hi, lo, r, k, sC[i][tx]);
   }
   if (I == J) return;
   // rows of tile J, columns of tile I (all below nstr)
   for (int i = ty; i < 32; i += ny) {
     const int r = J * 32 + i, k = I * 32 + tx;
-    if (r < nstr) {
-      const float x = sC[tx][i];
-      const bf16 h = __float2bfloat16_rn(x);
-      hi[(int64_t)r * ldc + k] = h;
-      lo[(int64_t)r * ldc + k] = __float2bfloat16_rn(x - __bfloat162float(h));
-    }
+    if (r < nstr) put(hi, lo, r, k, sC[tx][i]);
   }
 }
 
@@ -279,6 +288,7 @@ k_gemm_haa(const bf16* __restrict__ haa, const bf16* __restrict__ cs, int64_t hs
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tbase;
   const uint32_t sbase = smem_u32(sm);
+  const bool leader = warp == 0 && elect_one();   // issues the MMAs
   // one K block into a stage: 2 operands x 2 halves x 128 rows x 4 chunks
   auto load = [&](int kb, int s) {
     const uint32_t st = sbase + (uint32_t)s * G_STAGE;
@@ -320,7 +330,7 @@ k_gemm_haa(const bf16* __restrict__ haa, const bf16* __restrict__ cs, int64_t hs
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (tid == 0) {
+    if (leader) {
       const uint32_t st = sbase + (uint32_t)(kc % G_STAGES) * G_STAGE;
 #pragma unroll
       for (int kk = 0; kk < GK_T / 16; kk++) {
@@ -336,7 +346,7 @@ k_gemm_haa(const bf16* __restrict__ haa, const bf16* __restrict__ cs, int64_t hs
     }
   }
   cp_async_wait<0>();
-  if (tid == 0) mma_commit(&mdone);
+  if (leader) mma_commit(&mdone);
   bool done = ok && mbar_wait(&mdone, 0, wait_limit);
   if (__syncthreads_or(!done)) {
     if (tid == 0) atomicExch(err, MBE_ETIMEOUT);
@@ -557,7 +567,7 @@ k_sigma_ab(const int32_t* __restrict__ lnk, const int16_t* __restrict__ plist,
 
   if (warp == 0) {
     // ------------------------------------------------ MMA issue
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = make_idesc_mn(AB_M, KP);
       const uint32_t a_lbo = (AB_M / 8) * 128, b_lbo = (uint32_t)(KP / 8) * 128;
       const uint32_t a_lo = (uint32_t)kl * AB_M * 2, b_lo = (uint32_t)kl * KP * 2;
@@ -1072,9 +1082,20 @@ void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, float* c, int64_t c_st
   const int64_t hs = 2 * (int64_t)nstr * p.ldc;      // bf16 elements per tuple (hi + lo)
   const int ntiles = (nstr + AB_M - 1) / AB_M;
   cudaStream_t st = ctx->stream;
-  // per bin shape: compacted links and the pull lists of the scatter
   StringTables* tab = get_tables(ctx, bp.n, bp.nsig);
-  if (tab->nlink != p.nlink) {
+  // the two-spin part over (N-1)-electron strings where that kernel takes the
+  // shape: 5 to 12 orbitals, whose operand and one string's row sums fit in
+  // shared memory (64 x 8e/12o 804 -> 326 us, 8 x 10e/12o 452 -> 249 us).  At 13
+  // the operand alone is 130 KB; there and beyond, over the rows of c
+  const bool nm1 = p.nlink > 0 && sigma_nm1_supported(bp.n, bp.nsig, nstr, B);
+  int nm_stages = 0;
+  if (nm1) {
+    sigma_nm1_prepare(ctx, bp, w, spin_shift);
+    auto it = ctx->tune_ab.find({bp.n, bp.nsig});
+    if (ctx->opt.autotune && it != ctx->tune_ab.end()) nm_stages = it->second[0];
+  }
+  // per bin shape: compacted links and the pull lists of the scatter
+  if (!nm1 && tab->nlink != p.nlink) {
     tab->lnk.reset(&ctx->pool, (size_t)nstr * std::max(p.nlink, 1));
     tab->plist.reset(&ctx->pool, (size_t)nstr * std::max(p.nlink, 1));
     tab->poff.reset(&ctx->pool, (size_t)nstr * (ntiles + 1));
@@ -1098,7 +1119,7 @@ void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, float* c, int64_t c_st
   if (w.csplit.n < (size_t)B * hs * 2) w.csplit.reset(&ctx->pool, (size_t)B * hs * 2);
   // per batch (constant over the Davidson iteration): g'/2 split and H^a
   const size_t gbytes = (size_t)B * 2 * p.kp * p.kp * 2;
-  if (bp.gsplit.n != gbytes) {
+  if (!nm1 && bp.gsplit.n != gbytes) {
     bp.gsplit.reset(&ctx->pool, gbytes);
     k_prep_gh<<<dim3(8, B), 256, 0, st>>>(bp.gp.ptr, npair, p.kp, (bf16*)bp.gsplit.ptr);
     CU_LAUNCH_CHECK();
@@ -1120,18 +1141,53 @@ void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, float* c, int64_t c_st
   if (packed) {
     const int ntp = (nstr + 31) / 32;
     k_split_c_sym<<<dim3((unsigned)(ntp * (ntp + 1) / 2), B), 256, 0, st>>>(
-        c, c_stride, T, sym_len(nstr), inv, nstr, p.ldc, active, cs, hs);
+        c, c_stride, T, sym_len(nstr), inv, nstr, p.ldc, active, cs, hs, nm1 ? w.cw.ptr : nullptr, sigma_nm1_ldw(nstr));
     CU_LAUNCH_CHECK();
   } else {
     const int64_t work = (int64_t)nstr * (p.ldc / 8);
     const unsigned gx = (unsigned)std::min<int64_t>((work + 255) / 256, 1024);
-    k_split_c<<<dim3(gx, B), 256, 0, st>>>(c, c_stride, nstr, p.ldc, active, cs, hs);
+    k_split_c<<<dim3(gx, B), 256, 0, st>>>(c, c_stride, nstr, p.ldc, active, cs, hs,
+                                           nm1 ? w.cw.ptr : nullptr, sigma_nm1_ldw(nstr));
     CU_LAUNCH_CHECK();
   }
   const long long wl = ctx->opt.wait_limit;
   const int nt_g = (nstr + GM_T - 1) / GM_T;
   const int grid_ab = (int)std::min<int64_t>((int64_t)B * nstr, nsm);
-  if (tune_now) {
+  if (tune_now && nm1) {
+    // its TMEM operand stages, timed on this call's data (the row sums are
+    // the same whatever the count)
+    cudaEvent_t e0, e1;
+    CU_CHECK(cudaEventCreate(&e0));
+    CU_CHECK(cudaEventCreate(&e1));
+    float best = 1e30f;
+    const int most = sigma_nm1_stages(bp.n, bp.nsig, nstr, B);
+    for (int nst = 2; nst <= most; nst++) {
+      float t = 1e30f;
+      for (int rep = 0; rep < 3; rep++) {
+        CU_CHECK(cudaEventRecord(e0, st));
+        sigma_nm1(ctx, bp, w, active, nsm, nst);
+        CU_CHECK(cudaEventRecord(e1, st));
+        CU_CHECK(cudaEventSynchronize(e1));
+        float ms = 0.f;
+        CU_CHECK(cudaEventElapsedTime(&ms, e0, e1));
+        if (rep > 0) t = std::min(t, ms);
+      }
+      if (ctx->opt.verbose)
+        fprintf(stderr, "[mbe autotune] n=%d nsig=%d stages=%d (N-1 strings) %.4f ms\n", bp.n,
+                bp.nsig, nst, t);
+      if (t < best) {
+        best = t;
+        nm_stages = nst;
+      }
+    }
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    ctx->tune_ab[{bp.n, bp.nsig}] = {nm_stages, 0, 1};
+    if (!ctx->tune_file.empty()) {
+      std::ofstream out(ctx->tune_file, std::ios::app);
+      out << "sigma_ab " << bp.n << " " << bp.nsig << " " << nm_stages << " 0 1 " << best << "\n";
+    }
+  } else if (tune_now) {
     // every plan that fits, timed on this call's data (H^a c rewritten
     // before each, so W ends correct whichever runs last); the best of two
     // timed launches per plan counts
@@ -1199,13 +1255,19 @@ void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, float* c, int64_t c_st
         (const bf16*)bp.haa.ptr, cs, hs, nstr, p.ldc, active, w.Xf.ptr, N, wl, w.err.ptr);
     CU_LAUNCH_CHECK();
   }
-  if (p.nlink > 0) {
+  if (nm1) {
+    sigma_nm1(ctx, bp, w, active, nsm, nm_stages);
+  } else if (p.nlink > 0) {
     launch_ab(ctx->device, grid_ab, p, st, tab->lnk.ptr, tab->plist.ptr, tab->poff.ptr, nstr,
               (const bf16*)bp.gsplit.ptr, cs, hs, active, B, w.Xf.ptr, N, wl, w.err.ptr);
     CU_LAUNCH_CHECK();
   }
   ctx->dom_timer.end(st, ev);
   ctx->stats.dom_launches += 1;
+  if (nm1) {
+    sigma_nm1_finish(ctx, bp, w, N, c, c_stride, spin_shift, active, out, out_stride, packed);
+    return;
+  }
   const int ntl = (nstr + 31) / 32;
   k_sigma_tc_finish<<<dim3((unsigned)(ntl * (ntl + 1) / 2), B), 256, 0, st>>>(w.Xf.ptr, N, bp.tab->link.ptr, bp.tab->masks.ptr,
                                                 nstr, bp.n, bp.nsig, c, c_stride,

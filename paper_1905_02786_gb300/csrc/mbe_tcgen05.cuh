@@ -56,6 +56,20 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t da, uint64_t 
       "l"(da), "l"(db), "r"(idesc), "r"(accumulate));
 }
 
+// One lane of a converged warp (the same one each time).  The thread that
+// issues MMAs is chosen with it and not by a lane number: under a branch on
+// elect.sync's predicate the compiler keeps the issue in uniform registers
+// (56-112 cycles per MMA of N = 96-208 with A in tensor memory, the tensor
+// pipe's own pace), under `lane == 0` every MMA took 174-180 cycles whatever N.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}\n"
+      : "=r"(e));
+  return e != 0;
+}
+
 __device__ __forceinline__ void mma_commit(uint64_t* mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                    smem_u32(mbar))
