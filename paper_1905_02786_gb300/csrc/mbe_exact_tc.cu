@@ -28,6 +28,12 @@
 // Layout of a tile, as in the tensor-core sigma: M = 128 determinants
 // (R rows a of X per CTA, W = 128 / R column strings k), N = kpad pairs,
 // A = D digits (K-major), B = g' digits (K-major), accumulator = E^T.
+//
+// Instruction issue and shared-memory atomics bound it (75 MMAs are a third of
+// a tile's time), so: digits by FP32 additions and byte permutes instead of
+// 64-bit shifts and conversions, the small groups' integers likewise, 64-bit
+// sums as two 32-bit atomics, and the next tile's global reads behind the MMAs.
+// 64 x 8e/12o: 10.19 -> 7.31 ms, 8 x 10e/12o 4.06 -> 3.18 ms per call.
 #include "mbe_internal.cuh"
 #include "mbe_tcgen05.cuh"
 #include <cuda_bf16.h>
@@ -41,7 +47,8 @@ constexpr int EX_THREADS = 640;
 constexpr int EX_M = 128;
 constexpr int EX_SLICES = 5;
 constexpr int EX_GROUPS = 6;
-constexpr int EX_MAXK = 80;            // 6 groups x kpad columns <= 512
+constexpr int EX_MAXK = 80;            // 6 groups x kpad columns <= 512: up to 12 orbitals
+constexpr int EX_R = 2;                // rows a of X per CTA
 constexpr uint32_t EX_TMEM_COLS = 512;
 
 __host__ __device__ inline int ex_link_stride(int kpad) { return 8 * ((kpad >> 3) | 1); }
@@ -58,17 +65,29 @@ __device__ __forceinline__ int exp_f32(float x) {
   return be == 0 ? -1000 : be - 126;
 }
 
-// round(x 2^(39 - e)) for |x| < 2^e, from the FP32 bit pattern (integer ops)
-__device__ __forceinline__ long long fixed39_f32(float x, int e) {
-  const uint32_t bits = __float_as_uint(x);
-  const int be = (int)((bits >> 23) & 0xFF);
-  if (be == 0) return 0;
-  const long long M = (long long)((bits & 0x7FFFFFu) | 0x800000u);
-  const int sh = be - 150 + 39 - e;            // x = M 2^(be - 150)
-  long long F = 0;
-  if (sh >= 0) F = M << sh;
-  else if (sh > -40) F = (M + (1LL << (-sh - 1))) >> (-sh);
-  return (bits >> 31) ? -F : F;
+// Digits of F = round(d1 2^(39 - e)) + round(d2 2^(39 - e)), |d| < 2^e, without
+// conversions (16 per clock and SM against 128 additions): with sc = 2^(39 - e)
+// and y = d sc (exact), y = h 2^20 + l, |h| <= 2^19, |l| <= 2^19, and adding
+// 1.5 2^23 rounds h and l to integers that stand in the low bits of the sum.
+// F + 0x80808080 then has the balanced digits plus 128 as its low four bytes,
+// the first digit above them; a byte u becomes the float 2^23 + u by PRMT and
+// u - 128 by one addition (exact, and its upper half is the bf16 value).
+__device__ __forceinline__ void split39(float d, float sc, uint32_t& h, uint32_t& l) {
+  constexpr float M = 12582912.f;   // 1.5 2^23, 0x4B400000
+  const float y = d * sc, t = fmaf(y, 0x1p-20f, M);
+  h += __float_as_uint(t);
+  l += __float_as_uint(fmaf(t - M, -0x1p20f, y) + M);
+}
+__device__ __forceinline__ void digits_f32(float d1, float d2, float sc, float* f) {
+  uint32_t h = 0u - 2u * 0x4B400000u, l = 0x80808080u - 2u * 0x4B400000u;
+  split39(d1, sc, h, l);
+  split39(d2, sc, h, l);
+  const long long G = (long long)(int)h * (1 << 20) + (long long)l;
+  const uint32_t u = (uint32_t)G;
+#pragma unroll
+  for (int i = 1; i < EX_SLICES; i++)
+    f[i] = __uint_as_float(__byte_perm(u, 0x4B000000u, 0x7440 | (4 - i))) - 8388736.f;
+  f[0] = __int_as_float((int)(G >> 32) + 0x4B400000) - 12582912.f;
 }
 
 // round(x 2^(39 - e)) for an FP64 x, |x| < 2^e (integer ops)
@@ -153,8 +172,8 @@ struct ExShared {
   uint32_t g, d, c_rows, x_rows, link_k, link_a, ep, em, total;
 };
 
-__host__ __device__ inline ExShared ex_layout(int kpad, int R, int nstr) {
-  const int W = EX_M / R;
+__host__ __device__ inline ExShared ex_layout(int kpad, int nstr) {
+  constexpr int R = EX_R, W = EX_M / R;
   ExShared s;
   uint32_t o = 0;
   auto take = [&](uint32_t bytes) {
@@ -165,8 +184,8 @@ __host__ __device__ inline ExShared ex_layout(int kpad, int R, int nstr) {
   s.g = take((uint32_t)EX_SLICES * kpad * kpad * 2);
   s.d = take((uint32_t)EX_SLICES * EX_M * kpad * 2);
   s.c_rows = take((uint32_t)R * (nstr + 1) * 4);
-  s.x_rows = take((uint32_t)R * nstr * 8);
-  s.link_k = take((uint32_t)W * ex_link_stride(kpad) * 2);
+  s.x_rows = take((uint32_t)R * (nstr + 1) * 8);
+  s.link_k = take((uint32_t)2 * W * ex_link_stride(kpad) * 2);
   s.link_a = take((uint32_t)R * kpad * 4);
   s.ep = take((uint32_t)kpad * 4);
   s.em = take((uint32_t)EX_M * 4);
@@ -174,14 +193,13 @@ __host__ __device__ inline ExShared ex_layout(int kpad, int R, int nstr) {
   return s;
 }
 
-template <int R>
 __global__ void __launch_bounds__(EX_THREADS, 1)
 k_sigma_exact(const int32_t* __restrict__ link, int nstr, int npair, int kpad,
               const uint8_t* __restrict__ gslices, const int32_t* __restrict__ ge,
               const float* __restrict__ c, int64_t c_stride, const float* __restrict__ rmax,
               const int32_t* __restrict__ active, double* __restrict__ X, int64_t x_stride,
               long long wait_limit, int32_t* __restrict__ err) {
-  constexpr int W = EX_M / R;
+  constexpr int R = EX_R, W = EX_M / R;
   const int LS = ex_link_stride(kpad);
   const int b = blockIdx.y;
   if (active && !active[b]) return;
@@ -191,12 +209,13 @@ k_sigma_exact(const int32_t* __restrict__ link, int nstr, int npair, int kpad,
   __shared__ uint64_t mbar;
   __shared__ uint32_t tmem_base_sh;
   __shared__ int s_maxep;
-  const ExShared L = ex_layout(kpad, R, nstr);
+  const ExShared L = ex_layout(kpad, nstr);
   const uint32_t gplane = (uint32_t)kpad * kpad * 2, dplane = (uint32_t)EX_M * kpad * 2;
   uint8_t* sG = smem + L.g;
   uint8_t* sD = smem + L.d;
   float* sC = (float*)(smem + L.c_rows);
-  long long* sX = (long long*)(smem + L.x_rows);
+  // X rows, nstr + 1 words of the low and as many of the high halves
+  uint32_t* sX = (uint32_t*)(smem + L.x_rows);
   uint16_t* sLk = (uint16_t*)(smem + L.link_k);
   int32_t* sLa = (int32_t*)(smem + L.link_a);
   int* sEP = (int*)(smem + L.ep);
@@ -222,7 +241,7 @@ k_sigma_exact(const int32_t* __restrict__ link, int nstr, int npair, int kpad,
     const int a = a0 + r;
     sC[it] = (a < nstr && k < nstr) ? cb[a * nstr + k] : 0.f;
   }
-  for (int it = tid; it < R * nstr; it += EX_THREADS) sX[it] = 0;
+  for (int it = tid; it < 2 * R * (nstr + 1); it += EX_THREADS) sX[it] = 0;
   for (int it = tid; it < R * kpad; it += EX_THREADS) {
     const int r = it / kpad, P = it - r * kpad;
     const int a = a0 + r;
@@ -239,7 +258,6 @@ k_sigma_exact(const int32_t* __restrict__ link, int nstr, int npair, int kpad,
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_base_sh;
   const int Z = s_maxep + 2 - 48;
-  const bool leader = warp == 0 && elect_one();   // issues the MMAs
   const uint32_t idesc = make_idesc(EX_M, kpad);
   const uint32_t sbo = (uint32_t)(kpad >> 3) * 128u;
   const int nkb = kpad >> 3;
@@ -249,7 +267,6 @@ k_sigma_exact(const int32_t* __restrict__ link, int nstr, int npair, int kpad,
   // thread -> determinant m = tid % 128 and P-blocks tid / 128 + 5 i (gather),
   // warp -> TMEM lanes 32 (w mod 4) and 8-column chunks w / 4 + 5 i (epilogue):
   // the ten blocks and chunks of kpad = 80 in two even rounds
-  // (20 warps: 28.65 ms against 29.0 with 24 on the 64 x 8e/12o batch)
   const int gm = tid & (EX_M - 1);
   const int gr = gm / W, gj = gm % W;
   const int ga = a0 + gr;
@@ -257,60 +274,85 @@ k_sigma_exact(const int32_t* __restrict__ link, int nstr, int npair, int kpad,
   const float* crow = sC + gr * (nstr + 1);
   const int em_ = 32 * (warp & 3) + lane;
   const int er = em_ / W, ej = em_ % W;
-  long long* xrow = sX + er * nstr;
+  uint32_t* xlo = sX + er * (nstr + 1);
+  int* xhi = (int*)(xlo + R * (nstr + 1));
 
+  // What a tile reads from global memory is fetched while the MMAs of the one
+  // before it run: the elements c(J_a, k) of this thread's blocks and the row
+  // maximum of k into registers, the link rows into the other of two buffers
+  constexpr int NB = (EX_MAXK / 8 + EX_THREADS / EX_M - 1) / (EX_THREADS / EX_M);
+  float xa[NB][8], rk;
+  auto fetch = [&](int k0, uint16_t* lk) {
+    const int k = k0 + gj;
+    const bool col_ok = ga < nstr && k < nstr;
+    const float* ccol = cb + (col_ok ? k : 0);   // column 0 stands in for an invalid one
+    rk = col_ok ? rmax[(int64_t)b * nstr + k] : 0.f;
+#pragma unroll
+    for (int i = 0; i < NB; i++) {
+      const int kb = (tid >> 7) + i * (EX_THREADS / EX_M);
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        const int t = kb < nkb ? la[kb * 8 + q] : -1;
+        xa[i][q] = ccol[t >= 0 ? (t >> 1) : 0];
+      }
+    }
+    // link rows of the tile's column strings (pad-encoded, as in the
+    // tensor-core sigma)
+    for (int j = warp; j < W; j += EX_THREADS / 32) {
+      uint16_t* dst = lk + j * LS;
+      const int32_t* src = link + (int64_t)(k0 + j) * npair;
+      for (int P = lane; P < kpad; P += 32) {
+        const int t = (k0 + j < nstr && P < npair) ? src[P] : -1;
+        dst[P] = (uint16_t)(t < 0 ? nstr : ((t >> 1) | ((t & 1) << 15)));
+      }
+    }
+  };
   // the two FP32 terms of D_P(m) for the 8 pairs of block pb
-  auto terms = [&](int k, bool col_ok, int pb, const uint16_t* lkg, float* d1, float* d2) {
+  auto terms = [&](const float* x1, bool col_ok, int pb, const uint16_t* lkg, float* d1,
+                   float* d2) {
     const int4 a0v = *reinterpret_cast<const int4*>(la + pb);
     const int4 a1v = *reinterpret_cast<const int4*>(la + pb + 4);
     const int4 kv = *reinterpret_cast<const int4*>(lkg + pb);
     const int ta[8] = {a0v.x, a0v.y, a0v.z, a0v.w, a1v.x, a1v.y, a1v.z, a1v.w};
     const uint32_t kw[4] = {(uint32_t)kv.x, (uint32_t)kv.y, (uint32_t)kv.z, (uint32_t)kv.w};
-    const float* ccol = cb + (col_ok ? k : 0);   // column 0 stands in for an invalid one
-    float xa[8];
-#pragma unroll
-    for (int q = 0; q < 8; q++) xa[q] = ccol[ta[q] >= 0 ? (ta[q] >> 1) : 0];
 #pragma unroll
     for (int q = 0; q < 8; q++) {
-      d1[q] = (col_ok && ta[q] >= 0) ? ((ta[q] & 1) ? -xa[q] : xa[q]) : 0.f;
+      d1[q] = (col_ok && ta[q] >= 0) ? ((ta[q] & 1) ? -x1[q] : x1[q]) : 0.f;
       const uint32_t e = (kw[q >> 1] >> (16 * (q & 1))) & 0xFFFFu;
       const float x = crow[e & 0x7FFFu];
       d2[q] = (e & 0x8000u) ? -x : x;
     }
   };
+  const float ra = ga < nstr ? rmax[(int64_t)b * nstr + ga] : 0.f;
+  fetch(0, sLk);
+  __syncthreads();
 
   for (int k0 = 0; k0 < nstr && ok; k0 += W) {
-    // ---- link rows of the tile's column strings (pad-encoded, as in the
-    // tensor-core sigma)
-    const int nc = min(W, nstr - k0);
-    for (int j = warp; j < W; j += EX_THREADS / 32) {
-      uint16_t* dst = sLk + j * LS;
-      const int32_t* src = link + (int64_t)(k0 + j) * npair;
-      for (int P = lane; P < kpad; P += 32) {
-        const int t = (j < nc && P < npair) ? src[P] : -1;
-        dst[P] = (uint16_t)(t < 0 ? nstr : ((t >> 1) | ((t & 1) << 15)));
-      }
-    }
-    __syncthreads();
     const int k = k0 + gj;
     const bool col_ok = ga < nstr && k < nstr;
-    const uint16_t* lkg = sLk + gj * LS;
+    uint16_t* lk = sLk + (k0 / W & 1) * W * LS;
+    const uint16_t* lkg = lk + gj * LS;
     // ---- digit planes of D (A operand), e_m from the row maxima of c
     {
-      const int e = col_ok ? exp_f32(rmax[(int64_t)b * nstr + ga] + rmax[(int64_t)b * nstr + k])
-                           : -1000;
+      // (below 2^-80 the terms round to zero units of X; d = 0 where !col_ok)
+      const int e = max(col_ok ? exp_f32(ra + rk) : -80, -80);
+      const float sc = __int_as_float((39 - e + 127) << 23);   // 2^(39 - e), e >= -80
       if (tid < EX_M) sEm[gm] = e;
-      for (int kb = tid >> 7; kb < nkb; kb += EX_THREADS / EX_M) {
+#pragma unroll
+      for (int r = 0; r < NB; r++) {
+        const int kb = (tid >> 7) + r * (EX_THREADS / EX_M);
+        if (kb >= nkb) break;
         float d1[8], d2[8];
-        terms(k, col_ok, kb * 8, lkg, d1, d2);
-        __align__(16) __nv_bfloat16 sl[EX_SLICES][8];
+        terms(xa[r], col_ok, kb * 8, lkg, d1, d2);
+        __align__(16) uint32_t sl[EX_SLICES][4];
 #pragma unroll
-        for (int q = 0; q < 8; q++) {
-          __nv_bfloat16 d[EX_SLICES];
-          const long long F = e > -1000 ? fixed39_f32(d1[q], e) + fixed39_f32(d2[q], e) : 0;
-          digits5(F, d);
+        for (int q = 0; q < 8; q += 2) {
+          float f0[EX_SLICES], f1[EX_SLICES];
+          digits_f32(d1[q], d2[q], sc, f0);
+          digits_f32(d1[q + 1], d2[q + 1], sc, f1);
 #pragma unroll
-          for (int i = 0; i < EX_SLICES; i++) sl[i][q] = d[i];
+          for (int i = 0; i < EX_SLICES; i++)
+            sl[i][q >> 1] = __byte_perm(__float_as_uint(f0[i]), __float_as_uint(f1[i]), 0x7632);
         }
         const uint32_t off = kmajor_offset(gm, kb * 8, kpad);
 #pragma unroll
@@ -322,7 +364,7 @@ k_sigma_exact(const int32_t* __restrict__ link, int nstr, int npair, int kpad,
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     // ---- group accumulators: acc_s = sum_{i + j = s} D_i g'_j^T (columns s kpad)
-    if (leader) {
+    if (warp == 0 && elect_one()) {
       const uint32_t d0 = smem_u32(sD), g0 = smem_u32(sG);
       for (int ks = 0; ks < (kpad >> 4); ks++) {
         const uint32_t koff = (uint32_t)ks * 256u;
@@ -340,6 +382,7 @@ k_sigma_exact(const int32_t* __restrict__ link, int nstr, int npair, int kpad,
       }
       mma_commit(&mbar);
     }
+    if (k0 + W < nstr) fetch(k0 + W, sLk + ((k0 / W & 1) ^ 1) * W * LS);
     const int timed_out = mbar_wait(&mbar, phase, wait_limit) ? 0 : 1;
     if (__syncthreads_or(timed_out)) {
       ok = false;
@@ -355,35 +398,55 @@ k_sigma_exact(const int32_t* __restrict__ link, int nstr, int npair, int kpad,
     // in units of 2^Z (a right shift by >= 7 bits, rounded)
     if (ok) {
       const int e_m = sEm[em_];
-      const uint16_t* lke = sLk + ej * LS;
+      const uint16_t* lke = lk + ej * LS;
       const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
 #pragma unroll 1
       for (int ch = warp >> 2; ch < nkb; ch += EX_THREADS / EX_M) {
-        long long I[8];
+        uint32_t u[EX_GROUPS][8];
 #pragma unroll
-        for (int q = 0; q < 8; q++) I[q] = 0;
-#pragma unroll
-        for (int s = 0; s < EX_GROUPS; s++) {
-          float v[8];
-          tmem_ld8(tmem + lane_off + (uint32_t)(s * kpad + ch * 8), v);
-#pragma unroll
-          for (int q = 0; q < 8; q++)
-            I[q] += (long long)__float2int_rn(v[q]) * (1LL << (8 * (EX_GROUPS - 1 - s)));
-        }
+        for (int s = 0; s < EX_GROUPS; s++)
+          tmem_ld8_nowait(tmem + lane_off + (uint32_t)(s * kpad + ch * 8), u[s]);
         const int4 kv = *reinterpret_cast<const int4*>(lke + ch * 8);
         const uint32_t kw[4] = {(uint32_t)kv.x, (uint32_t)kv.y, (uint32_t)kv.z, (uint32_t)kv.w};
-        if (e_m > -1000) {
+        tmem_wait_ld();
 #pragma unroll
-          for (int q = 0; q < 8; q++) {
-            const uint32_t t = (kw[q >> 1] >> (16 * (q & 1))) & 0xFFFFu;
-            const uint32_t J = t & 0x7FFFu;
-            if (J == (uint32_t)nstr) continue;
-            const int sh = Z + 54 + 1 - (sEP[ch * 8 + q] + e_m);   // >= 7
-            long long v = sh < 63 ? (I[q] + (1LL << (sh - 1))) >> sh : 0;
-            if (t & 0x8000u) v = -v;
-            atomicAdd((unsigned long long*)&xrow[J], (unsigned long long)v);
+        for (int s = 0; s < EX_GROUPS; s++)
+#pragma unroll
+          for (int q = 0; q < 8; q++) asm volatile("" : "+r"(u[s][q]));
+        uint32_t lo[8], J[8];
+        int hi[8];
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+          // the groups of at most three products stay below 2^22 (3 x 80 x 2^14):
+          // adding 1.5 2^23 leaves the integer in the low bits
+          long long I = 0;
+#pragma unroll
+          for (int s = 0; s < EX_GROUPS; s++) {
+            const float a = __uint_as_float(u[s][q]);
+            const int v = s < 3 ? __float_as_int(a + 12582912.f) - 0x4B400000 : __float2int_rn(a);
+            I += (long long)v * (1LL << (8 * (EX_GROUPS - 1 - s)));
           }
+          const uint32_t t = (kw[q >> 1] >> (16 * (q & 1))) & 0xFFFFu;
+          J[q] = t & 0x7FFFu;
+          // >= 7; 63 and more: zero
+          const int sh = min(63, Z + 54 + 1 - (sEP[ch * 8 + q] + e_m));
+          long long v = ((I >> (sh - 1)) + 1) >> 1;
+          if (t & 0x8000u) v = -v;
+          lo[q] = (uint32_t)v;
+          hi[q] = (int)(v >> 32);
         }
+        // 64-bit sums as two 32-bit atomics: the low words wrap, and each wrap
+        // adds one to the high word, in whatever order (a 64-bit shared atomic
+        // is a compare-and-swap loop); unlinked pairs (J = nstr) are predicated
+        // off (adding them to a spare column serialises on its one address)
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+          const uint32_t old = J[q] < (uint32_t)nstr ? atomicAdd(&xlo[J[q]], lo[q]) : 0u;
+          hi[q] += old + lo[q] < old ? 1 : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; q++)
+          if (J[q] < (uint32_t)nstr) atomicAdd(&xhi[J[q]], hi[q]);
       }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -395,7 +458,9 @@ k_sigma_exact(const int32_t* __restrict__ link, int nstr, int npair, int kpad,
   for (int it = tid; it < R * nstr; it += EX_THREADS) {
     const int r = it / nstr, kk = it - r * nstr;
     const int a = a0 + r;
-    if (a < nstr) X[(int64_t)b * x_stride + (int64_t)a * nstr + kk] = (double)sX[it] * scale;
+    const int at = r * (nstr + 1) + kk;
+    const long long v = (long long)(((unsigned long long)sX[R * (nstr + 1) + at] << 32) | sX[at]);
+    if (a < nstr) X[(int64_t)b * x_stride + (int64_t)a * nstr + kk] = (double)v * scale;
   }
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, EX_TMEM_COLS);
@@ -406,15 +471,13 @@ k_sigma_exact(const int32_t* __restrict__ link, int nstr, int npair, int kpad,
 bool sigma_exact_supported(int npair, int nstr) {
   const int kpad = ((npair + 15) / 16) * 16;
   if (kpad > EX_MAXK) return false;
-  const int R = nstr <= 2048 ? 2 : 1;
-  return ex_layout(kpad, R, nstr).total + 2048 <= 227 * 1024;
+  return ex_layout(kpad, nstr).total + 2048 <= 227 * 1024;
 }
 
 void sigma_exact_prepare(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w) {
   const int npair = bp.npair, nstr = bp.nstr;
   const int kpad = ((npair + 15) / 16) * 16;
-  const int R = nstr <= 2048 ? 2 : 1;
-  const ExShared L = ex_layout(kpad, R, nstr);
+  const ExShared L = ex_layout(kpad, nstr);
   if (kpad > EX_MAXK || L.total + 2048 > 227 * 1024)
     throw MbeError{MBE_EINVAL, "active space too large for the fused exact sigma"};
   if (!w.err.ptr) {
@@ -433,9 +496,7 @@ void sigma_exact_prepare(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w) {
   if (w.rmax.n < (size_t)bp.B * nstr) w.rmax.reset(&ctx->pool, (size_t)bp.B * nstr);
   static bool attr_done[MBE_MAX_DEVICES] = {false};
   once_per_device(attr_done, ctx->device, [] {
-    CU_CHECK(cudaFuncSetAttribute(k_sigma_exact<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  227 * 1024 - 1024));
-    CU_CHECK(cudaFuncSetAttribute(k_sigma_exact<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    CU_CHECK(cudaFuncSetAttribute(k_sigma_exact, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   227 * 1024 - 1024));
   });
 }
@@ -444,24 +505,18 @@ void sigma_exact(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, const float* c, int
                  double* X, int64_t x_stride, const int32_t* active) {
   const int npair = bp.npair, nstr = bp.nstr;
   const int kpad = ((npair + 15) / 16) * 16;
-  const int R = nstr <= 2048 ? 2 : 1;
-  const ExShared L = ex_layout(kpad, R, nstr);
+  const ExShared L = ex_layout(kpad, nstr);
   // one-time set-up of the batch (allocations, g' digit planes)
   sigma_exact_prepare(ctx, bp, w);
-  const dim3 grid((unsigned)((nstr + R - 1) / R), bp.B);
+  const dim3 grid((unsigned)((nstr + EX_R - 1) / EX_R), bp.B);
   cudaEvent_t ev;
   ctx->fp64_timer.begin(ctx->stream, ctx->opt.timing != 0, &ev);
   k_rowmax<<<dim3((unsigned)((nstr + 7) / 8), bp.B), 256, 0, ctx->stream>>>(c, c_stride, nstr,
                                                                           active, w.rmax.ptr);
   CU_LAUNCH_CHECK();
-  if (R == 2)
-    k_sigma_exact<2><<<grid, EX_THREADS, L.total, ctx->stream>>>(
-        bp.tab->link.ptr, nstr, npair, kpad, w.gex.ptr, w.gexp.ptr, c, c_stride, w.rmax.ptr,
-        active, X, x_stride, ctx->opt.wait_limit, w.err.ptr);
-  else
-    k_sigma_exact<1><<<grid, EX_THREADS, L.total, ctx->stream>>>(
-        bp.tab->link.ptr, nstr, npair, kpad, w.gex.ptr, w.gexp.ptr, c, c_stride, w.rmax.ptr,
-        active, X, x_stride, ctx->opt.wait_limit, w.err.ptr);
+  k_sigma_exact<<<grid, EX_THREADS, L.total, ctx->stream>>>(
+      bp.tab->link.ptr, nstr, npair, kpad, w.gex.ptr, w.gexp.ptr, c, c_stride, w.rmax.ptr, active,
+      X, x_stride, ctx->opt.wait_limit, w.err.ptr);
   CU_LAUNCH_CHECK();
   ctx->fp64_timer.end(ctx->stream, ev);
   ctx->stats.fp64_launches += 1;

@@ -153,7 +153,6 @@ k_contract_ozaki(const double* __restrict__ gp_all, int npair, int kpad,
   const uint32_t sbo = (uint32_t)(kpad >> 3) * 128u;
   uint32_t phase = 0;
 
-  const bool leader = warp == 0 && elect_one();   // issues the MMAs
   const int64_t ntiles = (ndet + OZ_N - 1) / OZ_N;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int64_t n0 = tile * OZ_N;
@@ -194,7 +193,7 @@ k_contract_ozaki(const double* __restrict__ gp_all, int npair, int kpad,
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     // ---- group accumulators acc_s (columns 64 s .. 64 s + 63)
-    if (leader) {
+    if (warp == 0 && elect_one()) {
       const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
       for (int ks = 0; ks < (kpad >> 4); ks++) {
         const uint32_t koff = (uint32_t)ks * 256u;

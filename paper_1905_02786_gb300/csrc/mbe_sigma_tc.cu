@@ -254,7 +254,9 @@ k_build_haa(const int32_t* __restrict__ link, int nstr, int npair, const double*
 // 0.7 % slower on the 64 x 8e/12o batch);
 // both operands K-major (8 rows x 16 bytes core matrices, LBO 128, SBO 512);
 // one elected thread issues the split-BF16x3 MMAs into a 128-column TMEM
-// accumulator.
+// accumulator.  43 of 64 x 8e/12o: 150 -> 109 us, 8 x 10e/12o 125 -> 103 us with
+// W stored as whole rows and the copies' addresses computed once; the tiles'
+// 32 KB per block from the L2 bound it (the MMAs alone: about 30 us).
 constexpr int GM_T = 128, GK_T = 32, G_STAGES = 3, G_AHEAD = 2, G_THREADS = 128;
 constexpr uint32_t G_OPB = GM_T * GK_T * 2;          // bytes of one operand half (8 KB)
 constexpr uint32_t G_STAGE = 4 * G_OPB;              // A hi, A lo, B hi, B lo
@@ -288,19 +290,34 @@ k_gemm_haa(const bf16* __restrict__ haa, const bf16* __restrict__ cs, int64_t hs
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tbase;
   const uint32_t sbase = smem_u32(sm);
-  const bool leader = warp == 0 && elect_one();   // issues the MMAs
-  // one K block into a stage: 2 operands x 2 halves x 128 rows x 4 chunks
+  // one K block into a stage: 2 operands x 2 halves x 128 rows x 4 chunks.
+  // A thread copies chunk tid % 4 of the rows tid / 4 + 32 j; everything but the
+  // block's k and the stage is computed once
+  constexpr int G_ROWS = G_THREADS / 4, G_J = GM_T / G_ROWS;
+  const int ch = tid & 3, r0 = tid >> 2;
+  uint32_t goff[2][G_J], rok = 0;
+#pragma unroll
+  for (int j = 0; j < 2 * G_J; j++) {
+    const int gr = (j < G_J ? m0 : n0) + r0 + (j % G_J) * G_ROWS;
+    goff[j / G_J][j % G_J] = (uint32_t)min(gr, nstr - 1) * (uint32_t)ldc;
+    rok |= (gr < nstr ? 1u : 0u) << j;
+  }
+  const uint32_t sdst =
+      sbase + (uint32_t)((r0 >> 3) * (GK_T >> 3) + ch) * 128u + (uint32_t)(r0 & 7) * 16u;
   auto load = [&](int kb, int s) {
-    const uint32_t st = sbase + (uint32_t)s * G_STAGE;
-    for (int it = tid; it < 4 * GM_T * 4; it += G_THREADS) {
-      const int ch = it & 3, row = (it >> 2) & (GM_T - 1), hl = (it >> 9) & 1, op = it >> 10;
-      const int gr = (op == 0 ? m0 : n0) + row;
-      const int k = kb * GK_T + ch * 8;
-      const bool ok = gr < nstr && k < ldc;
-      const bf16* src = (op == 0 ? A : Bm) + hl * half + (ok ? (int64_t)gr * ldc + k : 0);
-      const uint32_t dst = st + (uint32_t)(op * 2 + hl) * G_OPB +
-                           (uint32_t)(((row >> 3) * (GK_T >> 3) + ch) * 128 + (row & 7) * 16);
-      cp_async16(dst, src, ok ? 16u : 0u);
+    const int k = kb * GK_T + ch * 8;
+    const bool kok = k < ldc;
+    const uint32_t ko = kok ? (uint32_t)k : 0u, st = sdst + (uint32_t)s * G_STAGE;
+#pragma unroll
+    for (int op = 0; op < 2; op++) {
+      const bf16* p = (op == 0 ? A : Bm) + ko;
+#pragma unroll
+      for (int j = 0; j < G_J; j++) {
+        const uint32_t n = kok && ((rok >> (op * G_J + j)) & 1u) ? 16u : 0u;
+        const uint32_t dst = st + (uint32_t)(op * 2) * G_OPB + (uint32_t)(j * G_ROWS * GK_T * 2);
+        cp_async16(dst, p + goff[op][j], n);
+        cp_async16(dst + G_OPB, p + half + goff[op][j], n);
+      }
     }
   };
   for (int s = 0; s < G_AHEAD; s++) {
@@ -330,7 +347,7 @@ k_gemm_haa(const bf16* __restrict__ haa, const bf16* __restrict__ cs, int64_t hs
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (leader) {
+    if (warp == 0 && elect_one()) {
       const uint32_t st = sbase + (uint32_t)(kc % G_STAGES) * G_STAGE;
 #pragma unroll
       for (int kk = 0; kk < GK_T / 16; kk++) {
@@ -346,7 +363,7 @@ k_gemm_haa(const bf16* __restrict__ haa, const bf16* __restrict__ cs, int64_t hs
     }
   }
   cp_async_wait<0>();
-  if (leader) mma_commit(&mdone);
+  if (warp == 0 && elect_one()) mma_commit(&mdone);
   bool done = ok && mbar_wait(&mdone, 0, wait_limit);
   if (__syncthreads_or(!done)) {
     if (tid == 0) atomicExch(err, MBE_ETIMEOUT);
@@ -356,18 +373,29 @@ k_gemm_haa(const bf16* __restrict__ haa, const bf16* __restrict__ cs, int64_t hs
   }
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (done) {
-    const int row = m0 + 32 * warp + lane;
-    float* wr = W + (int64_t)b * w_stride + (int64_t)row * nstr;
+    // a lane holds a row: through shared memory (the stages are free), so that
+    // the stores to W are whole rows (from the lanes, 32 rows per store, they
+    // took more of the load/store unit than the loads)
+    constexpr int GP = GM_T + 4;
+    float* so = reinterpret_cast<float*>(sm) + 32 * warp * GP;
     const uint32_t ta = tmem + ((uint32_t)(32 * warp) << 16);
-#pragma unroll 1
+#pragma unroll 2
     for (int cc = 0; cc < GM_T; cc += 16) {
       float v[16];
       tmem_ld8x2(ta + (uint32_t)cc, ta + (uint32_t)(cc + 8), v);
-      if (row < nstr) {
 #pragma unroll
-        for (int j = 0; j < 16; j++)
-          if (n0 + cc + j < nstr) wr[n0 + cc + j] = v[j];
-      }
+      for (int j = 0; j < 16; j += 4)
+        *reinterpret_cast<float4*>(so + lane * GP + cc + j) =
+            make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    }
+    __syncwarp();
+    const int r1 = min(32, nstr - m0 - 32 * warp), c1 = nstr - n0;
+    float* wr = W + (int64_t)b * w_stride + (int64_t)(m0 + 32 * warp) * nstr + n0;
+#pragma unroll 4
+    for (int r = 0; r < r1; r++, wr += nstr) {
+#pragma unroll
+      for (int j = 0; j < GM_T; j += 32)
+        if (lane + j < c1) wr[lane + j] = so[r * GP + lane + j];
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
