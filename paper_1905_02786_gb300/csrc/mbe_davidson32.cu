@@ -559,8 +559,12 @@ void davidson_batch_mixed(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int3
     }
     return false;
   };
-  // the exact-point sigma: fused on the tensor cores where it fits (kpad <= 80)
+  // the exact-point sigma: fused on the tensor cores where it fits (up to 12
+  // orbitals: 64 x 8e/12o 7.31 ms against 24.3), beyond that FP64 from the string
+  // links (10e/13o: 3.96 ms against 8.5 for the sliced contraction through D and
+  // E, which stays where a row of c is too long for the FP64 kernel)
   const bool exact_fused = sigma_exact_supported(bp.npair, bp.nstr);
+  const bool exact_direct = !exact_fused && sigma_direct_supported(bp.n, bp.nsig, bp.nstr);
   // exact point of the tuples in `mask`: V0 = x/|x|, exact A V0, theta_x,
   // r_x and its norm; G = [[V0.AV0]]
   auto exact_point = [&]() {
@@ -574,6 +578,8 @@ void davidson_batch_mixed(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int3
     if (exact_fused) {
       sigma_exact(ctx, bp, sw, F.ptr, Lf, S64.ptr, Lf, active.ptr);
       launch_finish_sym_fp64(ctx, bp, S64.ptr, Lf, C64.ptr, Lf, shift, active.ptr);
+    } else if (exact_direct) {
+      sigma_direct(ctx, bp, C64.ptr, Lf, S64.ptr, Lf, active.ptr, shift, true, false);
     } else {
       sigma_emulated(ctx, bp, sw, C64.ptr, Lf, S64.ptr, Lf, active.ptr, shift, true);
     }
@@ -589,6 +595,7 @@ void davidson_batch_mixed(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int3
 
   // the exact path's set-up before any of its calls is captured
   if (exact_fused) sigma_exact_prepare(ctx, bp, sw);
+  if (exact_direct) sigma_direct_prepare(ctx, bp);
   // stage A
   stage(1, 150, 1, false, B, Ms);
   // refinement rounds
@@ -598,14 +605,14 @@ void davidson_batch_mixed(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int3
   int round_cap = Ms;
   for (int round = 0; round < 12; round++) {
     // the exact point and the selection of the tuples above their targets
-    // (one graph; the unfused FP64 path stages host data and runs plain)
+    // (one graph; the sliced contraction stages host data and runs plain)
     auto point = [&] {
       exact_point();
       k32_select<<<1, 256, 0, st>>>(rnorm.ptr, mask.ptr, thx.ptr, B, abs_target, rel_target,
                                     ctx->opt.mixed_round_drop, active.ptr, tolr.ptr, nact.ptr);
       CU_LAUNCH_CHECK();
     };
-    if (use_graphs && exact_fused)
+    if (use_graphs && (exact_fused || exact_direct))
       gr.run(16, point);
     else
       point();

@@ -482,7 +482,7 @@ void launch_direct_values(mbe_ctx* ctx, int n, int nsig, int nstr, const uint32_
 void sigma_direct_raw(mbe_ctx* ctx, int n, const DirectSide& al, const DirectSide& be,
                       const double* wt, const double* gp, const double* c, int64_t c_stride,
                       double* out, int64_t out_stride, const int32_t* active,
-                      const int32_t* bmap, int nb, double spin_shift, bool symmetric);
+                      const int32_t* bmap, int nb, double spin_shift, int symmetric);   // 2: full
 StringTables* get_tables(mbe_ctx* ctx, int n, int nsig);
 // active electrons of each spin: alpha (orbitals below nocc_a), beta (below nocc)
 int count_sig(const mbe_ctx* ctx, const std::vector<int>& act);
@@ -550,10 +550,13 @@ void convert_f64_to_f32(mbe_ctx* ctx, const double* src, float* dst, int64_t n);
 // with their parents' vectors (exactly one of V32 / V64 non-null)
 void launch_parent_guess(mbe_ctx* ctx, const GuessPlan& plan, int n, int nsig, int nstr,
                          float* V32, double* V64, int64_t vstride);
-// FP64 on the CUDA cores (symmetric: c(a,b) = c(b,a) for every tuple and the
-// result in the packed layout; otherwise any c and the full result):
+// FP64 on the CUDA cores (symmetric: c(a,b) = c(b,a) for every tuple, the upper
+// triangle is computed and the result packed or full; otherwise any c and the
+// full result):
 void sigma_direct(mbe_ctx* ctx, BinProblem& bp, const double* c, int64_t c_stride, double* out,
-                  int64_t out_stride, const int32_t* active, double spin_shift, bool symmetric);
+                  int64_t out_stride, const int32_t* active, double spin_shift, bool symmetric,
+                  bool packed = true);
+bool sigma_direct_supported(int n, int nsig, int nstr);
 // its tables and values (sigma_direct makes them on its first call otherwise)
 void sigma_direct_prepare(mbe_ctx* ctx, BinProblem& bp);
 // FP64-grade: gather, sliced tensor-core GEMM, scatter (symmetric: c(a,b) =

@@ -401,7 +401,12 @@ k_sigma_direct(const DirArgs A, const DirPlan L) {
   for (int k = tid; k < nb; k += nt) {
     double s = sPart[k];
     for (int part = 1; part < S; part++) s += sPart[part * nb + k];
-    ob[A.sym ? sym_index(a, b0 + k, nstrb) : (int64_t)a * nstrb + k] = s;
+    if (A.sym == 1) {
+      ob[sym_index(a, b0 + k, nstrb)] = s;
+    } else {
+      ob[(int64_t)a * nstrb + b0 + k] = s;
+      if (A.sym) ob[(int64_t)(b0 + k) * nstrb + a] = s;
+    }
   }
 }
 
@@ -438,7 +443,7 @@ void launch_direct_values(mbe_ctx* ctx, int n, int nsig, int nstr, const uint32_
 void sigma_direct_raw(mbe_ctx* ctx, int n, const DirectSide& al, const DirectSide& be,
                       const double* wt, const double* gp, const double* c, int64_t c_stride,
                       double* out, int64_t out_stride, const int32_t* active,
-                      const int32_t* bmap, int nb, double spin_shift, bool symmetric) {
+                      const int32_t* bmap, int nb, double spin_shift, int symmetric) {
   DirArgs A;
   A.n = n;
   A.npair = n * (n + 1) / 2;
@@ -448,7 +453,7 @@ void sigma_direct_raw(mbe_ctx* ctx, int n, const DirectSide& al, const DirectSid
   A.nsigb = be.nsig;
   A.nnz = direct_nnz(n, al.nsig);
   A.nnzb = direct_nnz(n, be.nsig);
-  A.sym = symmetric ? 1 : 0;
+  A.sym = symmetric;
   A.masks = al.masks;
   A.masksb = be.masks;
   A.olnk = al.olnk;
@@ -482,6 +487,12 @@ void sigma_direct_raw(mbe_ctx* ctx, int n, const DirectSide& al, const DirectSid
   ctx->stats.fp64_launches += 1;
 }
 
+// the closed-shell shape fits the kernel's shared memory
+bool sigma_direct_supported(int n, int nsig, int nstr) {
+  return direct_plan(n * (n + 1) / 2, nsig * (n - nsig), direct_nnz(n, nsig), nstr).total <=
+         DIR_SMEM;
+}
+
 // the shape's tables (once) and the batch's values (once per batch)
 void sigma_direct_prepare(mbe_ctx* ctx, BinProblem& bp) {
   const int n = bp.n;
@@ -511,12 +522,13 @@ void sigma_direct_prepare(mbe_ctx* ctx, BinProblem& bp) {
 }
 
 void sigma_direct(mbe_ctx* ctx, BinProblem& bp, const double* c, int64_t c_stride, double* out,
-                  int64_t out_stride, const int32_t* active, double spin_shift, bool symmetric) {
+                  int64_t out_stride, const int32_t* active, double spin_shift, bool symmetric,
+                  bool packed) {
   sigma_direct_prepare(ctx, bp);
   const DirectSide al = {bp.nsig, bp.nstr, bp.tab->masks.ptr, bp.tab->olnk.ptr, bp.tab->hidx.ptr,
                          bp.hv.ptr};
   const DirectSide be = {bp.nsigb, bp.nstrb, bp.tabb->masks.ptr, bp.tabb->olnk.ptr,
                          bp.tabb->hidx.ptr, bp.closed() ? bp.hv.ptr : bp.hvb.ptr};
   sigma_direct_raw(ctx, bp.n, al, be, bp.wt.ptr, bp.gp.ptr, c, c_stride, out, out_stride, active,
-                   nullptr, bp.B, spin_shift, symmetric && bp.closed());
+                   nullptr, bp.B, spin_shift, !symmetric || !bp.closed() ? 0 : packed ? 1 : 2);
 }
