@@ -11,7 +11,7 @@
 //        y <- y - sum_{j != k} z_j (z_j . s) / (lambda_j - theta),
 //      each step multiplying the error by ~ (FP32 residual of Z) / gap, and
 //      theta = y.G.y is the FP64 Rayleigh quotient of the normalised y.
-// m <= 32; G is read symmetrised, (G + G^T) / 2.
+// m <= 32; G is symmetric.
 //
 // The step is a chain of short dependent phases, so its latency is what
 // counts.  A thread owns column (lane) and four rows of A and Z; it forms the
@@ -20,8 +20,10 @@
 // Jacobi step.  When the subspace has grown by one vector since the last call
 // the sweeps start from Z_prev^T G Z_prev, an arrow matrix whose border is
 // small near convergence (2-3 sweeps instead of 6).  FP64 sums run in one
-// warp (each of the others would take the same 16 cycles of the SM's FP64
-// unit per instruction).
+// warp: an FP64 instruction of a warp takes 64 cycles of its sub-partition's
+// unit, a division or root about 1,200.  So the refinement stops once its
+// update is below 2e-10 (mostly the second; four always took 17,000 cycles), y.Gy
+// and y.y share one reduction, and y.y, 1 to about 1e-6, is inverted by a series.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -54,7 +56,7 @@ static __device__ void ritz_lowest(const double* __restrict__ Gb, int m, int M, 
   const int tid = threadIdx.x, r = tid & 31, w = tid >> 5;
   for (int i = w; i < 32; i += 8) {
     double g = 0.0;
-    if (i < m && r < m) g = 0.5 * (Gb[(int64_t)i * M + r] + Gb[(int64_t)r * M + i]);
+    if (i < m && r < m) g = Gb[(int64_t)i * M + r];
     S.G[i][r] = g;
     S.A[0][i][r] = (float)g;
     S.Z[0][i][r] = warm && i < m - 1 && r < m - 1 ? Zk[i * 32 + r] : (i == r) ? 1.f : 0.f;
@@ -159,8 +161,11 @@ static __device__ void ritz_lowest(const double* __restrict__ Gb, int m, int M, 
   // ---- 2. FP64 Newton refinement of the lowest pair (y unnormalised; warp 0
   // keeps it, lane = component); row products are spread over 8 threads
   double y = r < m ? (double)Z[r][k] : 0.0;
-  double theta = 0.0;
+  double theta = 0.0, n = 1.0;
   const int row = tid >> 3, part = tid & 7;
+  // s (FP32) drives the update; with the update at c, the error left in y is
+  // about c^2 (both are the FP32 residual of Z over the gap), that of theta and
+  // of |y|^2 smaller still
   for (int it = 0; it < 4; it++) {
     if (w == 0) S.y[r] = y;
     __syncthreads();
@@ -173,18 +178,24 @@ static __device__ void ritz_lowest(const double* __restrict__ Gb, int m, int M, 
     __syncthreads();
     if (w == 0) {
       const double g = r < m ? S.gy[r] : 0.0;
-      double a = y * g, n = y * y;
-      for (int o = 16; o; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        n += __shfl_xor_sync(0xffffffffu, n, o);
-      }
-      theta = a / n;
+      // lanes below 16 sum y.gy, the others y.y
+      const double a0 = y * g, n0 = y * y;
+      double v = r < 16 ? a0 : n0;
+      v += __shfl_xor_sync(0xffffffffu, r < 16 ? n0 : a0, 16);
+      for (int o = 8; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      const double a = __shfl_sync(0xffffffffu, v, 0);
+      n = __shfl_sync(0xffffffffu, v, 16);
+      const double d = n - 1.0;
+      if (fabs((float)d) < 1e-4f)   // 1 / (1 + d), to d^5
+        theta = a * fma(-d, fma(-d, fma(-d, 1.0 - d, 1.0), 1.0), 1.0);
+      else
+        theta = a / n;
       S.s32[r] = (float)(g - theta * y);
       if (r == 0) S.theta = (float)theta;
-      if (it == 3) y /= sqrt(n);
     }
     if (it == 3) break;
     __syncthreads();
+    bool more = false;
     if (4 * w < m) {
       float d = 0.f;
       for (int j = part; j < m; j += 8) d = fmaf(Z[j][row], S.s32[j], d);
@@ -196,9 +207,10 @@ static __device__ void ritz_lowest(const double* __restrict__ Gb, int m, int M, 
           if (fabsf(den) > 1e-6f * fmaxf(1.f, fabsf(th))) cf = d / den;
         }
         S.coef[row] = cf;
+        more = !(fabsf(cf) < 2e-10f);
       }
     }
-    __syncthreads();
+    const bool go = __syncthreads_or(more);
     if (4 * w < m) {
       float c = 0.f;
       for (int j = part; j < m; j += 8) c = fmaf(Z[row][j], S.coef[j], c);
@@ -206,7 +218,19 @@ static __device__ void ritz_lowest(const double* __restrict__ Gb, int m, int M, 
       if (part == 0) S.lam[row] = c;
     }
     __syncthreads();
-    if (w == 0 && r < m) y -= (double)S.lam[r];
+    if (w == 0) {
+      const double c = r < m ? (double)S.lam[r] : 0.0;
+      if (!go) n -= 2.0 * (double)ritz_warp_sumf((float)y * (float)c);   // |y - c|^2, c^2 < 1e-18
+      y -= c;
+    }
+    if (!go) break;
+  }
+  if (w == 0) {   // y / |y|
+    const double d = n - 1.0;
+    if (fabs((float)d) < 1e-4f)   // (1 + d)^(-1/2), to d^5
+      y *= fma(d, fma(d, fma(d, fma(d, 35.0 / 128.0, -5.0 / 16.0), 3.0 / 8.0), -0.5), 1.0);
+    else
+      y /= sqrt(n);
   }
   if (tid == 0) *theta_out = theta;
   if (w == 0 && r < m) y_out[r] = y;
