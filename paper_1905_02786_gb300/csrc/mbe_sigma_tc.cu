@@ -248,16 +248,15 @@ k_build_haa(const int32_t* __restrict__ link, int nstr, int npair, const double*
 
 // ------------------------------------------------------------ W = H^a c
 // Tiles of 128 x 128 (rows a of H^a x rows b of c = columns b of c), K in
-// blocks of 32 through a 3-stage cp.async ring loaded two blocks ahead (a
-// stage is refilled once the MMAs of the block before have completed; 97 KB
-// of shared memory, so two CTAs share an SM: 4 stages, one CTA per SM, were
-// 0.7 % slower on the 64 x 8e/12o batch);
-// both operands K-major (8 rows x 16 bytes core matrices, LBO 128, SBO 512);
-// one elected thread issues the split-BF16x3 MMAs into a 128-column TMEM
-// accumulator.  43 of 64 x 8e/12o: 150 -> 109 us, 8 x 10e/12o 125 -> 103 us with
-// W stored as whole rows and the copies' addresses computed once; the tiles'
-// 32 KB per block from the L2 bound it (the MMAs alone: about 30 us).
-constexpr int GM_T = 128, GK_T = 32, G_STAGES = 3, G_AHEAD = 2, G_THREADS = 128;
+// blocks of 32 through two cp.async stages, the next block loaded while the MMAs
+// of this one run; both operands K-major (8 rows x 16 bytes core matrices, LBO
+// 128, SBO 512); one elected thread issues the split-BF16x3 MMAs into a
+// 128-column TMEM accumulator.  The latency of a block's 32 KB from the L2 bounds
+// it (the MMAs alone: about 30 us), so three CTAs share an SM (65 KB each): 43
+// of 64 x 8e/12o 150 -> 107 us, 8 x 10e/12o 125 -> 80 us, with W stored as whole
+// rows; three stages and two CTAs take 109 and 103 us, K blocks of 64 and one
+// CTA of 256 threads 116 and 97 us.
+constexpr int GM_T = 128, GK_T = 32, G_STAGES = 2, G_AHEAD = 1, G_THREADS = 128;
 constexpr uint32_t G_OPB = GM_T * GK_T * 2;          // bytes of one operand half (8 KB)
 constexpr uint32_t G_STAGE = 4 * G_OPB;              // A hi, A lo, B hi, B lo
 constexpr uint32_t G_SMEM = G_STAGES * G_STAGE + 1024;
@@ -332,7 +331,7 @@ k_gemm_haa(const bf16* __restrict__ haa, const bf16* __restrict__ cs, int64_t hs
     if (kb < nk) {
       const int s = kb % G_STAGES;
       if (kb >= G_STAGES) {
-        // the MMAs of block kb - G_STAGES (issued at kc - 2) used this stage
+        // the MMAs of block kb - G_STAGES (issued at kc - 1) used this stage
         const bool got = mbar_wait(&mbar[s], (uint32_t)((kb / G_STAGES) - 1) & 1u, wait_limit);
         if (__syncthreads_or(!got)) {
           ok = false;
@@ -376,26 +375,30 @@ k_gemm_haa(const bf16* __restrict__ haa, const bf16* __restrict__ cs, int64_t hs
     // a lane holds a row: through shared memory (the stages are free), so that
     // the stores to W are whole rows (from the lanes, 32 rows per store, they
     // took more of the load/store unit than the loads)
-    constexpr int GP = GM_T + 4;
+    constexpr int GH = GM_T / 2, GP = GH + 4;   // half the columns at a time
     float* so = reinterpret_cast<float*>(sm) + 32 * warp * GP;
     const uint32_t ta = tmem + ((uint32_t)(32 * warp) << 16);
+    const int r1 = min(32, nstr - m0 - 32 * warp);
+    for (int h = 0; h < GM_T; h += GH) {
 #pragma unroll 2
-    for (int cc = 0; cc < GM_T; cc += 16) {
-      float v[16];
-      tmem_ld8x2(ta + (uint32_t)cc, ta + (uint32_t)(cc + 8), v);
+      for (int cc = 0; cc < GH; cc += 16) {
+        float v[16];
+        tmem_ld8x2(ta + (uint32_t)(h + cc), ta + (uint32_t)(h + cc + 8), v);
 #pragma unroll
-      for (int j = 0; j < 16; j += 4)
-        *reinterpret_cast<float4*>(so + lane * GP + cc + j) =
-            make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-    }
-    __syncwarp();
-    const int r1 = min(32, nstr - m0 - 32 * warp), c1 = nstr - n0;
-    float* wr = W + (int64_t)b * w_stride + (int64_t)(m0 + 32 * warp) * nstr + n0;
+        for (int j = 0; j < 16; j += 4)
+          *reinterpret_cast<float4*>(so + lane * GP + cc + j) =
+              make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+      }
+      __syncwarp();
+      const int c1 = nstr - n0 - h;
+      float* wr = W + (int64_t)b * w_stride + (int64_t)(m0 + 32 * warp) * nstr + n0 + h;
 #pragma unroll 4
-    for (int r = 0; r < r1; r++, wr += nstr) {
+      for (int r = 0; r < r1; r++, wr += nstr) {
 #pragma unroll
-      for (int j = 0; j < GM_T; j += 32)
-        if (lane + j < c1) wr[lane + j] = so[r * GP + lane + j];
+        for (int j = 0; j < GH; j += 32)
+          if (lane + j < c1) wr[lane + j] = so[r * GP + lane + j];
+      }
+      __syncwarp();
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
