@@ -40,13 +40,9 @@ DEFAULT_WORKLOAD = "h2o_dz_8e23o"
 # DRAM traffic per launch of the dominant kernels from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum), per algorithmic flop
 # (2 N_det npair^2 per sigma vector), keyed by kernel; valid only while the
-# kernel definition is unchanged (sha256 prefix of its source text).  From
-# the captures of one launch over 64 active 8e/12o tuples (1.9081e+11 flop),
-# profiles/k_sigma_ab_8e12o_batch64.md.
-TRAFFIC = {"k_gemm_haa": {"bytes_per_flop": (126411008 + 33256448) / 1.9081e11,
-                          "sha": "230b4e42ae85e619"},
-           "k_sigma_ab": {"bytes_per_flop": (100085760 + 9144576) / 1.9081e11,
-                          "sha": "b562c774055038dc"}}
+# kernel definition is unchanged (sha256 prefix of its source text).  No capture
+# of the present kernels over a full batch has been taken: null.
+TRAFFIC = {}
 
 
 def peaks():
@@ -479,12 +475,12 @@ def main():
         peak_tf = fp_peaks["fp64_tflops"]
         peak_src = "FP64 FMA, measured by mbe_measure_peaks on this GPU"
         bound = "alu"
-        ksrc = "paper_1905_02786_gb300/csrc/mbe_ci.cu"
+        ksrc = "paper_1905_02786_gb300/csrc/mbe_sigma64.cu"
     else:
-        # the sigma contraction: k_gemm_haa (one-spin part) + k_sigma_ab
-        # (two-spin part), timed together with CUDA events on the library's
+        # the sigma contraction: k_gemm_haa (one-spin part) + k_sigma_nm1
+        # (two-spin part; k_sigma_ab outside 5 to 12 orbitals), timed together with CUDA events on the library's
         # stream; algorithmic flops 2 N_det npair^2 per sigma vector
-        kname = "k_gemm_haa+k_sigma_ab"
+        kname = "k_gemm_haa+k_sigma_nm1"
         peak_tf = pk.get("bf16_tflops_sustained", 1700.0)
         peak_src = f"bf16 dense sustained, {pk_kind}"
         bound = "tensor"

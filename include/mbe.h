@@ -59,7 +59,7 @@ enum {
 
 /* Precision of the sigma-vector contraction. */
 enum {
-  MBE_FP64 = 0,          /* every step in FP64 (CUDA-core FP64 contraction)  */
+  MBE_FP64 = 0,          /* every step in FP64 (sigma from the string links)  */
   MBE_MIXED_BF16X3 = 1,  /* Davidson vectors in FP32; their sigma vectors as
                             split-BF16x3 on tcgen05 tensor cores with FP32
                             accumulation; refinement rounds ("exact points")
@@ -140,18 +140,18 @@ typedef struct mbe_options {
   int autotune;            /* 1: the first sigma call of each bin shape
                               (n, n_sigma) of the mixed mode times every
                               operand plan of the two-spin tensor-core kernel
-                              that fits (A-operand stages 2..4, pull lists in
+                              that fits on its own data and keeps the fastest
+                              for the shape: stages 2..4 of the operand ring
+                              and, outside 5 to 12 orbitals, pull lists in
                               shared or global memory, one or two epilogue
-                              groups) on its own data and
-                              keeps the fastest for the shape; 0 (default):
-                              the most stages that fit, lists in shared
-                              memory when they fit.  All plans give the same
-                              bits.                                          */
+                              groups; 0 (default): the most stages that fit,
+                              lists in shared memory when they fit.  All plans
+                              give the same bits.                            */
   const char* tune_file;   /* autotune cache (may be NULL): read at
                               mbe_create, one line per tuned shape appended
                               as it is tuned ("sigma_ab n nsig nstages
                               pull_smem groups ms"); the string is copied    */
-  int graphs;              /* mixed mode: 1 (default) issues each Davidson
+  int graphs;              /* FP64 and mixed modes: 1 (default) issues each Davidson
                               iteration (sigma vector, subspace update, Ritz
                               step, residual, correction and its
                               orthogonalisation) as one CUDA graph, captured
@@ -347,16 +347,14 @@ int mbe_sigma(mbe_ctx* ctx, const int* act, int nact, const double* c,
  *  e_core      host; if non-NULL the inactive-core energy is written there
  *              and the call waits for the context stream; if NULL the call
  *              returns once the work is enqueued on the context stream.
- * All intermediates (string tables, effective integrals, the D and E
- * intermediates of the sigma) live in one file-scope device array of
+ * All intermediates (string tables, effective integrals, H's one-spin values)
+ * live in one file-scope device array of
  * MBE_NOALLOC_SCRATCH_BYTES per device; none of it needs to start at zero.
  * A problem that does not fit (roughly more than 9 active orbitals) returns
  * MBE_EINVAL and launches nothing.  Calls overlapping on one device race on
  * that array: issue them on one stream or wait for one before the next.
- * The first call on a device looks the array up (cudaGetSymbolAddress),
- * sets a kernel attribute and copies a small constant table with a
- * synchronous cudaMemcpyToSymbol (once per device, shared with the other
- * entry points); make it before any stream capture.  The active orbitals
+ * The first call on a device looks the array up (cudaGetSymbolAddress)
+ * and sets kernel attributes; make it before any stream capture.  The active orbitals
  * reach the device as a kernel argument; with e_core non-NULL the call
  * copies the core energy to the host and waits for the stream. */
 int mbe_sigma_noalloc(mbe_ctx* ctx, const int* act, int nact, const double* c_dev,
