@@ -196,7 +196,7 @@ void solve_jobs(mbe_ctx* ctx, const std::vector<std::vector<int>>& acts, double*
     // vectors each, N/2 FP32 elements) and five packed FP32 work vectors,
     // the full FP32 exact-point operand, two full FP64 exact-point vectors,
     // the FP32 W rows of the sigma, the bf16 hi/lo copies of the sigma
-    // operand and of H^alpha and the P-space eigenvectors; the FP64 one
+    // operand and of H^alpha and the P-space block; the FP64 one
     // 2M + 6 FP64 vectors and the one-spin tables of its sigma
     // the mixed path works on alpha<->beta symmetric vectors: closed shells
     const bool mixed_bin = ctx->opt.precision == MBE_MIXED_BF16X3 && N > 1 && closed &&
