@@ -263,6 +263,9 @@ struct StringTables {
   // string and its off-diagonal links, string index fastest
   DevBuf<uint16_t> hidx;
   DevBuf<uint32_t> olnk;
+  // both sets are complete (set last: an allocation in between may throw, and
+  // the next call then makes the set anew)
+  bool nm1_ready = false, direct_ready = false;
 };
 
 // ------------------------------------------------------------- context

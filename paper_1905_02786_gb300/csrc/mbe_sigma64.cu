@@ -498,10 +498,11 @@ void sigma_direct_prepare(mbe_ctx* ctx, BinProblem& bp) {
   const int n = bp.n;
   auto tables = [&](const StringTables* ct) {
     StringTables* t = const_cast<StringTables*>(ct);
-    if (t->hidx.ptr) return;
+    if (t->direct_ready) return;
     t->hidx.reset(&ctx->pool, (size_t)direct_nnz(n, t->nsig) * t->nstr);
     t->olnk.reset(&ctx->pool, std::max<size_t>(1, (size_t)t->nsig * (n - t->nsig) * t->nstr));
     launch_direct_tables(ctx, n, t->nsig, t->nstr, t->masks.ptr, t->hidx.ptr, t->olnk.ptr);
+    t->direct_ready = true;   // the tables outlive a call that runs out of memory half-way
   };
   tables(bp.tab);
   tables(bp.tabb);

@@ -929,7 +929,7 @@ void sigma_nm1_prepare(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, double shift)
     throw MbeError{MBE_EINVAL, "active space too large for the two-spin kernel"};
   StringTables* t = get_tables(ctx, n, nsig);
   cudaStream_t st = ctx->stream;
-  if (!t->krow.ptr) {
+  if (!t->nm1_ready) {
     t->kmask.reset(&ctx->pool, L.nK);
     t->kj0.reset(&ctx->pool, L.nK);
     t->srow.reset(&ctx->pool, (size_t)nstr * nsig);
@@ -941,6 +941,7 @@ void sigma_nm1_prepare(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, double shift)
                                                     t->kmask.ptr, t->krow.ptr, kcol, t->kj0.ptr,
                                                     t->srow.ptr);
     CU_LAUNCH_CHECK();
+    t->nm1_ready = true;
   }
   const size_t need = (size_t)bp.B * L.b_bytes;
   if (bp.nmop.n != need) {
