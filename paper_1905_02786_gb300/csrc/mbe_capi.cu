@@ -421,7 +421,9 @@ int mbe_load_integrals(mbe_ctx* ctx, int norb, int nelec, const double* h, const
       if (!std::isfinite(h[i])) return fail(ctx, MBE_EINVAL, "non-finite h");
     for (int64_t i = 0; i < np * np; i++)
       if (!std::isfinite(eri[i])) return fail(ctx, MBE_EINVAL, "non-finite eri");
-    ctx->norb = norb;
+    // no integrals until both arrays are on the device (an allocation may throw)
+    ctx->norb = 0;
+    ctx->have_ref = false;
     ctx->nelec = nelec;
     // lowest spin of the high-spin family: singlet or doublet
     ctx->two_sz = nelec % 2;
@@ -437,7 +439,7 @@ int mbe_load_integrals(mbe_ctx* ctx, int norb, int nelec, const double* h, const
     CU_CHECK(cudaMemcpyAsync(ctx->eri.ptr, eri, sizeof(double) * np * np, cudaMemcpyHostToDevice,
                              ctx->stream));
     CU_CHECK(cudaStreamSynchronize(ctx->stream));
-    ctx->have_ref = false;
+    ctx->norb = norb;
     ctx->kept.clear();
     ctx->kept_ref = false;
     ctx->rdm_blocks.clear();
@@ -495,6 +497,8 @@ int mbe_set_reference(mbe_ctx* ctx, const int* ref_orbs, int nref, const int* ex
       if (o < 0 || o >= ctx->norb || !seen.insert(o).second)
         return fail(ctx, MBE_EINVAL, "bad or duplicate expansion orbital");
     }
+    // no reference until its CASCI is solved and the tuple hash is there
+    ctx->have_ref = false;
     ctx->ref.assign(ref_orbs, ref_orbs + nref);
     std::sort(ctx->ref.begin(), ctx->ref.end());
     ctx->exp.assign(exp_orbs, exp_orbs + nexp);
@@ -526,7 +530,6 @@ int mbe_set_reference(mbe_ctx* ctx, const int* ref_orbs, int nref, const int* ex
       e = ec;
     }
     ctx->e_ref = e;
-    ctx->have_ref = true;
     if (ctx->opt.keep_ci && nref > 0) {
       ctx->ref_ci.order = 0;
       ctx->ref_ci.tuple.clear();
@@ -536,6 +539,7 @@ int mbe_set_reference(mbe_ctx* ctx, const int* ref_orbs, int nref, const int* ex
       ctx->kept_ref = true;
     }
     hash_init(ctx, 4096);
+    ctx->have_ref = true;
     ctx->history.clear();
     ctx->last_order = 0;
     ctx->cur_order = 0;
@@ -622,9 +626,19 @@ int mbe_increments(mbe_ctx* ctx, int order, double screen_thr, double* inc_out, 
       return fail(ctx, MBE_ESTATE, "increments must be processed order by order after solving");
     if (!(screen_thr >= 0.0)) return fail(ctx, MBE_EINVAL, "negative screening threshold");
     const int64_t ntup = (int64_t)ctx->cur_eps.size();
-    if (2 * (ctx->hash.count + ntup) > ctx->hash.cap) {
-      // grow the table and re-insert every processed order
-      hash_init(ctx, 4 * (ctx->hash.count + ntup));
+    if (2 * (ctx->hash.count + ntup) > ctx->hash.cap || ctx->hash.cap == 0) {
+      // grow the table and re-insert every processed order; complete stays
+      // false (the next call makes the table anew) if an allocation throws
+      int64_t total = ntup;
+      for (const OrderRec& r : ctx->history) total += (int64_t)r.inc.size();
+      hash_init(ctx, 4 * total);
+      struct Undo {
+        HashTable& h;
+        bool complete = false;
+        ~Undo() {
+          if (!complete) h.cap = 0;
+        }
+      } undo{ctx->hash};
       for (const OrderRec& r : ctx->history) {
         int64_t nt = (int64_t)r.inc.size();
         if (!nt) continue;
@@ -638,6 +652,7 @@ int mbe_increments(mbe_ctx* ctx, int order, double screen_thr, double* inc_out, 
         CU_CHECK(cudaMemcpyAsync(kb.ptr, r.keep.data(), nt, cudaMemcpyHostToDevice, ctx->stream));
         hash_insert(ctx, tb.ptr, r.order, nt, vb.ptr, kb.ptr);
       }
+      undo.complete = true;
     }
     DevBuf<double> inc(&ctx->pool, std::max<int64_t>(ntup, 1));
     DevBuf<uint8_t> keep(&ctx->pool, std::max<int64_t>(ntup, 1));

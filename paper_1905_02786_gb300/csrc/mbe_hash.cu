@@ -341,6 +341,7 @@ __global__ void k_gen_units(DevHash h, const int32_t* __restrict__ parents, int 
 }
 
 DevHash dev_hash(mbe_ctx* ctx) {
+  if (ctx->hash.cap == 0) throw MbeError{MBE_ESTATE, "no tuple hash (an allocation failed)"};
   DevHash h;
   h.keys = ctx->hash.keys.ptr;
   h.val = ctx->hash.val.ptr;
@@ -356,13 +357,14 @@ void hash_init(mbe_ctx* ctx, int64_t cap) {
   int64_t c = 1024;
   while (c < cap) c <<= 1;
   HashTable& H = ctx->hash;
-  H.cap = c;
+  H.cap = 0;   // no table if an allocation throws
   H.count = 0;
   H.keys.reset(&ctx->pool, 2 * c);
   H.val.reset(&ctx->pool, c);
   H.keep.reset(&ctx->pool, c);
   H.state.reset(&ctx->pool, c);
   CU_CHECK(cudaMemsetAsync(H.state.ptr, 0, sizeof(int32_t) * c, ctx->stream));
+  H.cap = c;
 }
 
 void hash_insert(mbe_ctx* ctx, const int32_t* tuples_dev, int order, int64_t ntup,

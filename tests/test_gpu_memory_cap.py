@@ -60,3 +60,59 @@ def test_sigma_after_failed_solve(lib, precision):
         if solved >= 3:
             break
     assert solved and failed_then_right
+
+
+@pytest.mark.parametrize("cap", [256, 512, 1024, 2048, 16 << 10, 24 << 10])
+def test_no_integrals_after_failed_load(lib, cap):
+    """10 orbitals take 1,024 and 24,320 bytes: none of these caps holds both."""
+    h, eri, _ = ms.gen_integrals(10, 4, 31)
+    m = lib.MBE(0, mem_cap_bytes=cap)
+    with pytest.raises(lib.MBEError) as ei:
+        m.load(h, eri, 8)
+    assert ei.value.code == lib.MBE_ENOMEM
+    for call in (lambda: lib.mbe_sigma(m.ctx, list(range(9)), np.ones(126 * 126)),
+                 lambda: lib.mbe_set_reference(m.ctx, [3], [4, 5]),
+                 lambda: lib.mbe_solve_tuples(m.ctx, np.array([[4]], dtype=np.int32), 1)):
+        with pytest.raises(lib.MBEError) as ei:
+            call()
+        assert ei.value.code == lib.MBE_ESTATE
+    m.close()
+
+
+def test_increments_after_failed_growth(lib):
+    """Order 2 of 64 expansion orbitals outgrows the tuple hash (4,096 slots for
+    2,080 tuples): where the larger one does not fit, the call says so every
+    time, and where it does the increments are right."""
+    norb = 65
+    rng = np.random.default_rng(4)
+    h, eri, _ = ms.gen_integrals(norb, 1, 7)
+    exp = list(range(1, norb))
+    t1 = np.array([[o] for o in exp], dtype=np.int32)
+    t2 = np.array([[a, b] for a in exp for b in exp if a < b], dtype=np.int32)
+    e1, e2 = rng.standard_normal(len(t1)), rng.standard_normal(len(t2))
+    base = eri.nbytes
+    seen = set()
+    for cap in range(base + (64 << 10), base + (2 << 20), 32 << 10):
+        m = lib.MBE(0, mem_cap_bytes=cap)
+        try:
+            m.load(h, eri, 2)
+            e0 = lib.mbe_set_reference(m.ctx, [0], exp)
+            lib.mbe_set_order_energies(m.ctx, t1, e1, 1)
+            inc1 = lib.mbe_increments(m.ctx, 1, 0.0, len(t1))[0]
+            lib.mbe_set_order_energies(m.ctx, t2, e2, 2)
+        except lib.MBEError as err:
+            assert err.code == lib.MBE_ENOMEM
+            m.close()
+            continue
+        want = e2 - e0 - inc1[t2[:, 0] - 1] - inc1[t2[:, 1] - 1]
+        for _ in range(2):
+            try:
+                inc2 = lib.mbe_increments(m.ctx, 2, 0.0, len(t2))[0]
+                assert np.abs(inc2 - want).max() < 1e-12
+                seen.add("right")
+                break
+            except lib.MBEError as err:
+                assert err.code == lib.MBE_ENOMEM
+                seen.add("full")
+        m.close()
+    assert seen == {"right", "full"}
