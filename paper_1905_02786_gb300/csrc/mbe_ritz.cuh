@@ -18,24 +18,30 @@
 // rotation of its own column's pair itself, takes those of its rows from the
 // other lanes by shuffles and writes into the other buffer: one barrier per
 // Jacobi step.  When the subspace has grown by one vector since the last call
-// the sweeps start from Z_prev^T G Z_prev, an arrow matrix whose border is
-// small near convergence (2-3 sweeps instead of 6).  FP64 sums run in one
-// warp: an FP64 instruction of a warp takes 64 cycles of its sub-partition's
-// unit, a division or root about 1,200.  So the refinement stops once its
-// update is below 2e-10 (mostly the second; four always took 17,000 cycles), y.Gy
-// and y.y share one reduction, and y.y, 1 to about 1e-6, is inverted by a series.
+// the sweeps start from Z^T G Z, an arrow matrix whose border is small near
+// convergence (2-3 sweeps instead of 6), Z the kept vectors after one
+// Newton-Schulz step, Z + Z (1 - Z^T Z) / 2: kept over 30 calls as they are,
+// they leave orthonormality by 1e-5, an error of |theta| 1e-5 in every
+// lambda_j - theta, and a root 1e-3 above the lowest cost up to half as many
+// iterations again.  FP64 sums run in one warp: an FP64 instruction of a warp
+// takes 64 cycles of its sub-partition's unit, a division or root about 1,200.
+// So the refinement stops once its update is below 2e-10 (mostly the second,
+// the fifth at a gap of 1e-3 below theta = -24; the error left is that times
+// the ratio above) or no longer halves (a gap lost in FP32), y.Gy and y.y share
+// one reduction, and y.y, 1 to about 1e-6, is inverted by a series.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 constexpr int RITZ_THREADS = 256;
+constexpr int RITZ_UPDATES = 12;   // of the FP64 refinement at most
 
 struct RitzShared {
   double G[32][33];
   double y[32], gy[32];
   float A[2][32][33];
   float Z[2][32][33];
-  float lam[32], s32[32], coef[32], theta;
+  float lam[32], s32[32], coef[32], wmax[8], theta;
 };
 
 __device__ __forceinline__ double ritz_warp_sum(double v) {
@@ -62,24 +68,37 @@ static __device__ void ritz_lowest(const double* __restrict__ Gb, int m, int M, 
     S.Z[0][i][r] = warm && i < m - 1 && r < m - 1 ? Zk[i * 32 + r] : (i == r) ? 1.f : 0.f;
   }
   __syncthreads();
+  int cur = 0;
   if (warm) {
-    // A <- Z^T A Z through Z[1]
+    // Z[1] <- Z + Z (1 - Z^T Z) / 2, then A[1] <- Z^T A Z (the product A Z in Z[0])
     for (int i = w; i < m; i += 8) {
-      float v = 0.f;
-      for (int j = 0; j < m; j++) v = fmaf(S.A[0][i][j], S.Z[0][j][r], v);
-      S.Z[1][i][r] = v;
+      float v = i == r ? 1.f : 0.f;
+      for (int j = 0; j < m; j++) v = fmaf(-S.Z[0][j][i], S.Z[0][j][r], v);
+      S.A[1][i][r] = v;
     }
     __syncthreads();
     for (int i = w; i < m; i += 8) {
       float v = 0.f;
-      for (int j = 0; j < m; j++) v = fmaf(S.Z[0][j][i], S.Z[1][j][r], v);
-      S.A[0][i][r] = v;
+      for (int j = 0; j < m; j++) v = fmaf(S.Z[0][i][j], S.A[1][j][r], v);
+      S.Z[1][i][r] = fmaf(0.5f, v, S.Z[0][i][r]);
     }
     __syncthreads();
+    for (int i = w; i < m; i += 8) {
+      float v = 0.f;
+      for (int j = 0; j < m; j++) v = fmaf(S.A[0][i][j], S.Z[1][j][r], v);
+      S.Z[0][i][r] = v;
+    }
+    __syncthreads();
+    for (int i = w; i < m; i += 8) {
+      float v = 0.f;
+      for (int j = 0; j < m; j++) v = fmaf(S.Z[1][j][i], S.Z[0][j][r], v);
+      S.A[1][i][r] = v;
+    }
+    __syncthreads();
+    cur = 1;
   }
   // ---- 1. FP32 tournament Jacobi
   const int n2 = m + (m & 1);
-  int cur = 0;
   for (int sweep = 0; sweep < 12 && m > 1; sweep++) {
     // every warp sums the whole matrix: the decision is the same in all
     float off = 0.f, dia = 0.f;
@@ -163,10 +182,11 @@ static __device__ void ritz_lowest(const double* __restrict__ Gb, int m, int M, 
   double y = r < m ? (double)Z[r][k] : 0.0;
   double theta = 0.0, n = 1.0;
   const int row = tid >> 3, part = tid & 7;
-  // s (FP32) drives the update; with the update at c, the error left in y is
-  // about c^2 (both are the FP32 residual of Z over the gap), that of theta and
-  // of |y|^2 smaller still
-  for (int it = 0; it < 4; it++) {
+  // s (FP32) drives the update; an update of c leaves an error of c times the
+  // ratio of the last two in y, and its square in theta and |y|^2
+  float cprev = 0.f;
+  bool last = false;   // the update before was the last one: theta and |y| only
+  for (int it = 0;; it++) {
     if (w == 0) S.y[r] = y;
     __syncthreads();
     if (4 * w < m) {   // the warps that hold rows below m
@@ -193,24 +213,28 @@ static __device__ void ritz_lowest(const double* __restrict__ Gb, int m, int M, 
       S.s32[r] = (float)(g - theta * y);
       if (r == 0) S.theta = (float)theta;
     }
-    if (it == 3) break;
+    if (last) break;
     __syncthreads();
-    bool more = false;
     if (4 * w < m) {
       float d = 0.f;
       for (int j = part; j < m; j += 8) d = fmaf(Z[j][row], S.s32[j], d);
       for (int o = 4; o; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-      if (part == 0) {
-        float cf = 0.f;
-        if (row < m && row != k) {
-          const float th = S.theta, den = S.A[cur][row][row] - th;
-          if (fabsf(den) > 1e-6f * fmaxf(1.f, fabsf(th))) cf = d / den;
-        }
-        S.coef[row] = cf;
-        more = !(fabsf(cf) < 2e-10f);
+      float cf = 0.f;
+      if (row < m && row != k) {
+        const float th = S.theta, den = S.A[cur][row][row] - th;
+        if (fabsf(den) > 1e-6f * fmaxf(1.f, fabsf(th))) cf = d / den;
       }
+      if (part == 0) S.coef[row] = cf;
+      // largest of the warp's four rows (bits of |x| order like |x|, NaN above)
+      const uint32_t c = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(cf)));
+      if (r == 0) S.wmax[w] = __uint_as_float(c);
     }
-    const bool go = __syncthreads_or(more);
+    __syncthreads();
+    float cm = 0.f;
+    for (int j = 0; 4 * j < m; j++) cm = S.wmax[j] <= cm ? cm : S.wmax[j];
+    const bool go = !(cm < 2e-10f);
+    last = it + 1 == RITZ_UPDATES || (it >= 2 && !(cm < 0.5f * cprev));
+    cprev = cm;
     if (4 * w < m) {
       float c = 0.f;
       for (int j = part; j < m; j += 8) c = fmaf(Z[row][j], S.coef[j], c);
