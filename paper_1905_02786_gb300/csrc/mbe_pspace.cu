@@ -19,8 +19,9 @@
 //                 tridiagonal form A_PP = Q T Q^T by Householder reflections
 //                 in shared memory, FP32 (a preconditioner needs no more);
 // per iteration:
-//   k_psp_apply   t_P = Q (theta - T)^{-1} Q^T r_P (r_P recovered from
-//                 the diagonal correction as t_I (theta - A_II)), written
+//   k_psp_apply   t_P = Q (theta - T)^{-1} Q^T r_P, the inverse bounded by 1e4
+//                 (mbe_tridiag.cuh; r_P recovered from the diagonal
+//                 correction as t_I (theta - A_II)), written
 //                 back into the packed vector; the same for M^-1 x, x the
 //                 Ritz vector; and the first Gram-Schmidt pass's
 //                 coefficients from the residual kernel's partial dots and
@@ -33,11 +34,13 @@
 // an inverse-iteration step in that case.  npp is capped at half the
 // canonical pairs.
 #include "mbe_internal.cuh"
+#include "mbe_tridiag.cuh"
 #include <algorithm>
 
 namespace {
 
 constexpr int PSP_MAX = 128;
+static_assert(PSP_MAX == TRI_MAX, "rows of the tridiagonal solve");
 constexpr int SEL_THREADS = 1024;
 constexpr int TRI_THREADS = 8 * PSP_MAX;
 constexpr int APPLY_THREADS = 4 * PSP_MAX;
@@ -459,8 +462,8 @@ __global__ void __launch_bounds__(TRI_THREADS)
 
 // What an iteration does between the residual and the Gram-Schmidt passes,
 // one CTA per tuple still iterating:
-//   t_P = Q (theta - T)^{-1} Q^T r_P (npp = 0: no P-space), the tridiagonal
-//   system by cyclic reduction, all unknowns at once (seven steps);
+//   t_P = Q Re (theta - T + i delta)^{-1} Q^T r_P (npp = 0: no P-space), the
+//   tridiagonal system by cyclic reduction, all unknowns at once (seven steps);
 //   with olsen the same block solve turns u = x / (theta - A_II) (Uo, from the
 //   residual kernel) into M^-1 x on P;
 //   the dots x.t, x.u (xpart) and, with dots, V.t (dpart) and V.u (upart) are
@@ -487,7 +490,7 @@ __global__ void __launch_bounds__(APPLY_THREADS)
   __shared__ float s_r[PSP_MAX], s_x[PSP_MAX];
   __shared__ float s_del[PSP_MAX], s_delu[PSP_MAX], s_xv[PSP_MAX];
   __shared__ float s_pr[4][PSP_MAX], s_px[4][PSP_MAX];
-  __shared__ float s_t[2][5][PSP_MAX];   // a, b, c and the two right-hand sides
+  __shared__ TriC s_t[2][5][TRI_MAX];   // a, b, c and the two right-hand sides
   __shared__ int s_i[PSP_MAX];
   __shared__ double s_c[32], s_c2[32], s_xs[2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -536,52 +539,25 @@ __global__ void __launch_bounds__(APPLY_THREADS)
         vx += __shfl_xor_sync(0xffffffffu, vx, o);
       }
       if (lane == 0) {
-        s_t[0][3][k] = v;
-        s_t[0][4][k] = vx;
+        s_t[0][3][k] = {v, 0.f};
+        s_t[0][4][k] = {vx, 0.f};
       }
     }
     if (tid < npp) {
       const float* tb = tri + (int64_t)b * 2 * PSP_MAX;
-      s_t[0][0][tid] = tid > 0 ? -tb[PSP_MAX + tid - 1] : 0.f;
-      s_t[0][1][tid] = th - tb[tid];
-      s_t[0][2][tid] = tid + 1 < npp ? -tb[PSP_MAX + tid] : 0.f;
+      s_t[0][0][tid] = {tid > 0 ? -tb[PSP_MAX + tid - 1] : 0.f, 0.f};
+      s_t[0][1][tid] = {th - tb[tid], TRI_DELTA};
+      s_t[0][2][tid] = {tid + 1 < npp ? -tb[PSP_MAX + tid] : 0.f, 0.f};
     }
     __syncthreads();
     int cur = 0;
     for (int st = 1; st < npp; st <<= 1, cur ^= 1) {
-      if (tid < npp) {
-        const float(*o)[PSP_MAX] = s_t[cur];
-        float(*w)[PSP_MAX] = s_t[cur ^ 1];
-        const int i = tid, lo = i - st, hi = i + st;
-        float bb = o[1][i], f = o[3][i], gx = o[4][i], an = 0.f, cn = 0.f;
-        auto piv = [](float x) { return fabsf(x) < 1e-6f ? (x < 0.f ? -1e-6f : 1e-6f) : x; };
-        if (lo >= 0) {
-          const float k1 = __fdividef(o[0][i], piv(o[1][lo]));
-          bb -= o[2][lo] * k1;
-          f -= o[3][lo] * k1;
-          gx -= o[4][lo] * k1;
-          an = -o[0][lo] * k1;
-        }
-        if (hi < npp) {
-          const float k2 = __fdividef(o[2][i], piv(o[1][hi]));
-          bb -= o[0][hi] * k2;
-          f -= o[3][hi] * k2;
-          gx -= o[4][hi] * k2;
-          cn = -o[2][hi] * k2;
-        }
-        w[0][i] = an;
-        w[1][i] = bb;
-        w[2][i] = cn;
-        w[3][i] = f;
-        w[4][i] = gx;
-      }
+      if (tid < npp) tri_level(s_t[cur], s_t[cur ^ 1], tid, st, npp);
       __syncthreads();
     }
     if (tid < npp) {
-      float d = s_t[cur][1][tid];
-      if (fabsf(d) < 1e-6f) d = d < 0.f ? -1e-6f : 1e-6f;
-      s_r[tid] = s_t[cur][3][tid] / d;
-      s_x[tid] = s_t[cur][4][tid] / d;
+      s_r[tid] = tri_div(s_t[cur][3][tid], s_t[cur][1][tid]).re;
+      s_x[tid] = tri_div(s_t[cur][4][tid], s_t[cur][1][tid]).re;
     }
     __syncthreads();
     {
