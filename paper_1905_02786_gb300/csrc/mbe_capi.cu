@@ -204,8 +204,9 @@ void solve_jobs(mbe_ctx* ctx, const std::vector<std::vector<int>>& acts, double*
     const int Mm = mixed_subspace_alloc(ctx->opt.max_subspace);
     // and, where its two-spin kernel takes the shape, the row sums and the
     // packed words of the operand
+    const int most = (int)std::min<int64_t>(ctx->opt.max_batch, (int64_t)kv.second.size());
     const double nm1 =
-        mixed_bin && sigma_nm1_supported(n, nsig, tab->nstr, 1)
+        mixed_bin && sigma_nm1_used(ctx->device, n, nsig, tab->nstr, std::max(1, most))
             ? 4.0 * ((double)sigma_nm1_slot_floats(n, nsig, tab->nstr) +
                      (double)tab->nstr * sigma_nm1_ldw(tab->nstr)) : 0.0;
     double per = (mixed_bin ? (double)(4 * Mm + 46) * N + nm1 + 128.0 * 128.0 * 4.0

@@ -422,6 +422,7 @@ struct BinProblem {
   DevBuf<double> jk;             // B * 2 * n * n  (J_pq = (pp|qq), K_pq = (pq|qp))
   DevBuf<uint8_t> gsplit;        // g'/2 as bf16 hi/lo rows (tensor-core sigma operand source)
   DevBuf<uint8_t> nmop;          // operand M of the (N-1)-electron two-spin kernel
+  int nm1 = -1;                  // two-spin kernel of this batch (1: that one; -1: not chosen yet)
   DevBuf<uint8_t> haa;           // one-spin Hamiltonian H^alpha as bf16 hi/lo rows
   // FP64 sigma: non-zero one-spin elements of the alpha (and, for an open
   // shell, beta) strings and the pair integrals summed over a beta string
@@ -526,6 +527,10 @@ int32_t sigma_tc_error(mbe_ctx* ctx, SigmaWork& w);
 // two-spin part over pairs of (N-1)-electron strings (mbe_sigma_nm1.cu): the
 // shapes it takes, the floats of row sums per tuple, its TMEM operand stages
 bool sigma_nm1_supported(int n, int nsig, int nstr, int B);
+int sigma_nm1_tiles(int n, int nsig, int nstr, int B);   // of one tuple (0: not supported)
+// the kernel of the two-spin part for B tuples of a shape (mbe_sigma_tc.cu):
+// sigma_nm1 where it is supported and the faster one, else over the rows of c
+bool sigma_nm1_used(int device, int n, int nsig, int nstr, int B);
 int64_t sigma_nm1_slot_floats(int n, int nsig, int nstr);
 int sigma_nm1_stages(int n, int nsig, int nstr, int B);
 int sigma_nm1_ldw(int nstr);   // words per row of w.cw

@@ -910,6 +910,11 @@ bool sigma_nm1_supported(int n, int nsig, int nstr, int B) {
   return nm_plan(n, nsig, nstr, B, L);
 }
 
+int sigma_nm1_tiles(int n, int nsig, int nstr, int B) {
+  NmPlan L;
+  return nm_plan(n, nsig, nstr, B, L) ? nm_tiles(L.nK, L.G) : 0;
+}
+
 int64_t sigma_nm1_slot_floats(int n, int nsig, int nstr) {
   return string_count(n, nsig - 1) * (n - nsig + 1) * nm_ld(nstr);
 }

@@ -30,9 +30,10 @@
 //                the product for 128 column strings lands in TMEM and the
 //                scatter through the link table of the column strings adds
 //                it into row a of W (columns J >= a) in shared memory; for 4,
-//                13 and more orbitals.  For 5 to 12 the two-spin part is
-//                k_sigma_nm1 over (N-1)-electron strings (mbe_sigma_nm1.cu),
-//                2 to 2.7 times faster;
+//                13 and more orbitals, small batches and strings more than half
+//                full.  Otherwise the two-spin part is k_sigma_nm1 over
+//                (N-1)-electron strings (mbe_sigma_nm1.cu; sigma_nm1_used), up to
+//                2.7 times faster;
 //   k_sigma_tc_finish  sigma = W + W^T + shift S^2 c.
 // Both products run as split-BF16x3 (hi*hi + lo*hi + hi*lo, FP32
 // accumulation in TMEM): ~16 significant bits per operand, sigma to ~1e-4 of
@@ -1091,6 +1092,30 @@ bool sigma_tc_supported(int n, int nstr) {
   return true;
 }
 
+// k_sigma_ab walks nstr rows in tiles of 128 columns, k_sigma_nm1 the pairs of
+// (N-1)-electron strings in tiles of 128 pairs, which take about three times as
+// long each (row sums) and 6 us more per call: it is the faster one where there
+// are several times fewer of them and enough work.  Strings more than half full
+// have more (N-1)-electron strings than strings: there it loses whatever the
+// batch.  The lines lie between the measured shapes (all of 5 to 12 orbitals, 1
+// to 64 tuples, whole iterations, k_sigma_ab over k_sigma_nm1; tiles per SM of
+// k_sigma_ab, ratio of tiles): 4e/7o x 56 1.05 (7.7, 21), 8e/11o x 1 1.04 (6.5,
+// 8.9), 8e/12o x 1 1.07, x 64 1.63 (13 and 834, 9.5), 10e/12o x 1 1.16 (36, 5.7),
+// 10e/10o x 12 0.92, x 56 1.04 (40 and 186, 2.9), 12e/11o x 12 0.94, x 56 1.01
+// (146 and 681, 2.2), 8e/9o x 12 0.96 (10, 4.3), 16e/12o x 35 0.64 (456, 0.8),
+// 18e/12o x 20 0.44 (58, 0.5).  Where the pull lists of k_sigma_ab do not fit in
+// shared memory (beyond 495 strings) its tiles cost half as much again: 14e/12o x
+// 1 0.84, x 12 1.01, x 56 1.39 (36, 438, 2,043; 1.65).
+bool sigma_nm1_used(int device, int n, int nsig, int nstr, int B) {
+  AbPlan p;
+  const int tiles = sigma_nm1_tiles(n, nsig, nstr, B);
+  if (tiles == 0 || !ab_plan(n, nsig, nstr, p) || p.nlink == 0) return false;
+  const int64_t ab = (int64_t)nstr * ((nstr + AB_M - 1) / AB_M);
+  const double ratio = (double)ab / tiles, per_sm = (double)B * ab / sm_count(device);
+  return ratio >= (p.L.pull_smem ? 2.8 : 1.0) &&
+         per_sm >= (ratio >= 8.0 ? 6.0 : ratio >= 4.0 ? 12.0 : 48.0);
+}
+
 void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, float* c, int64_t c_stride,
               float* out, int64_t out_stride, const int32_t* active, double spin_shift,
               bool packed, const float* T, const double* inv) {
@@ -1114,11 +1139,13 @@ void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, float* c, int64_t c_st
   const int ntiles = (nstr + AB_M - 1) / AB_M;
   cudaStream_t st = ctx->stream;
   StringTables* tab = get_tables(ctx, bp.n, bp.nsig);
-  // the two-spin part over (N-1)-electron strings where that kernel takes the
-  // shape: 5 to 12 orbitals, whose operand and one string's row sums fit in
-  // shared memory (64 x 8e/12o 804 -> 326 us, 8 x 10e/12o 452 -> 249 us).  At 13
-  // the operand alone is 130 KB; there and beyond, over the rows of c
-  const bool nm1 = p.nlink > 0 && sigma_nm1_supported(bp.n, bp.nsig, nstr, B);
+  // the two-spin part over (N-1)-electron strings where that is the faster one
+  // (a single sigma vector, mbe_sigma: the kernel that a full batch would take)
+  if (bp.nm1 < 0)
+    bp.nm1 = sigma_nm1_supported(bp.n, bp.nsig, nstr, B) &&
+             sigma_nm1_used(ctx->device, bp.n, bp.nsig, nstr,
+                            packed ? B : std::max(B, std::min(ctx->opt.max_batch, 256)));
+  const bool nm1 = bp.nm1 == 1;
   int nm_stages = 0;
   if (nm1) {
     sigma_nm1_prepare(ctx, bp, w, spin_shift);
