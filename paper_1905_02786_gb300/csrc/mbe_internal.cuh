@@ -127,6 +127,42 @@ __host__ __device__ inline int64_t sym_index(int a, int b, int nstr) {
                 : (int64_t)sym_nd(nstr) + (int64_t)a * (2 * nstr - a - 1) / 2 + (b - a - 1);
 }
 
+#ifdef __CUDACC__
+// (S^2 c)(ia, ib) of an Ms = 0 vector c = c^T in FP32 (packed or full rows of
+// nstr): (nsig - |a & b|) c(a, b) less, for q open in a and p open in b, the
+// signed c(a - q + p, b - p + q).  Evaluated for (min, max): both elements of a
+// pair get bitwise the same value.
+__device__ __forceinline__ float spin_square_sym(const int32_t* __restrict__ link,
+                                                 const uint32_t* __restrict__ masks, int nstr,
+                                                 int npair, int nsig, const float* __restrict__ cb,
+                                                 int packed, int ia, int ib) {
+  const int lo = min(ia, ib), hi = max(ia, ib);
+  const int32_t* la = link + (int64_t)lo * npair;
+  const int32_t* lb = link + (int64_t)hi * npair;
+  const uint32_t ma = masks[lo], mb = masks[hi];
+  float s2 = (float)(nsig - __popc(ma & mb)) *
+             cb[packed ? sym_index(lo, hi, nstr) : (int64_t)lo * nstr + hi];
+  // pairs {p, q}: q open in the alpha string, p open in the beta string
+  uint32_t oa = ma & ~mb;
+  const uint32_t obm = mb & ~ma;
+  while (oa) {
+    const int q = __ffs(oa) - 1;
+    oa &= oa - 1;
+    uint32_t ob2 = obm;
+    while (ob2) {
+      const int p = __ffs(ob2) - 1;
+      ob2 &= ob2 - 1;
+      const int P = p > q ? p * (p + 1) / 2 + q : q * (q + 1) / 2 + p;
+      const int32_t ta = la[P], tb = lb[P];
+      const float x = cb[packed ? sym_index(ta >> 1, tb >> 1, nstr)
+                                : (int64_t)(ta >> 1) * nstr + (tb >> 1)];
+      s2 -= ((ta ^ tb) & 1) ? -x : x;
+    }
+  }
+  return s2;
+}
+#endif
+
 // ------------------------------------------------------------ CUDA graphs
 // Replays a launch sequence as one CUDA graph.  run(key, issue) records the
 // launches issue() makes on the stream (stream capture), brings the

@@ -11,7 +11,9 @@
 //   Z(a, b) = sum_{p in a} sum_{r in b} sg(p, a-p) sg(r, b-r) U_pr(a-p, b-r).
 // (Zarrabian, Sarma & Paldus, Chem. Phys. Lett. 155, 183 (1989).)  For c = c^T
 // U_pr(Ka, Kb) = U_rp(Kb, Ka), so only the pairs Ka <= Kb are formed, with
-// weight 1/2 for Ka = Kb, and Z is the result plus its transpose.
+// weight 1/2 for Ka = Kb, and Z is the result plus its transpose.  Beyond the
+// default shift the spin term would carry more rounding into M and c than g'
+// does (k_sigma_nm1_finish adds it in FP32 there).
 //
 // This is one dense GEMM per tuple: rows = the nK (nK + 1) / 2 pairs, K = N =
 // n^2 orbital pairs, and its operand M is the same for every row.  Against
@@ -742,14 +744,23 @@ __global__ void k_nm1_ktables(const uint32_t* __restrict__ masks, int nstr, int 
   }
 }
 
+// The spin term goes through the split operand M up to the default shift: its
+// rms error against FP64 is then that of the FP32 term within 2 % (0.98-1.02 over
+// six shapes, 12 seeds each); at shifts of 1, 2 and 4 it would be 1.10, 1.34
+// and 2.04 times that, and worse in proportion beyond.
+inline bool nm_spin_in_operand(double shift) { return shift >= 0.0 && shift <= 0.5; }
+
 // sigma(a, b) = X(a, b) + X(b, a) + shift nsig c(a, b), X = W + the slots of
-// row a.  One CTA per 32 x 32 tile pair (I, J), I <= J; a warp reads 32
+// row a (SPIN: + shift (S^2 c)(a, b) in FP32 instead, M without the spin term).
+// One CTA per 32 x 32 tile pair (I, J), I <= J; a warp reads 32
 // consecutive columns of W and of each slot.  packed: c and sigma in the packed
 // symmetric layout, only tile (I, J) is written.
+template <bool SPIN>
 __global__ void __launch_bounds__(256)
 k_sigma_nm1_finish(const float* __restrict__ W, int64_t w_stride, const float* __restrict__ slots,
-                   int64_t s_stride, int ldS, const int2* __restrict__ srow, int nstr, int nsig,
-                   const float* __restrict__ c, int64_t c_stride, float dshift,
+                   int64_t s_stride, int ldS, const int2* __restrict__ srow,
+                   const int32_t* __restrict__ link, const uint32_t* __restrict__ masks, int npair,
+                   int nstr, int nsig, const float* __restrict__ c, int64_t c_stride, float shift,
                    const int32_t* __restrict__ active, float* __restrict__ out, int64_t out_stride,
                    int packed) {
   const int b = blockIdx.y;
@@ -796,7 +807,11 @@ k_sigma_nm1_finish(const float* __restrict__ W, int64_t w_stride, const float* _
     v[k] = 0.f;
     if (ia < nstr && ib < nstr) {
       const int64_t at = packed ? sym_index(ia, ib, nstr) : (int64_t)ia * nstr + ib;
-      v[k] = fmaf(dshift, cb[at], sX[0][i][tx] + sT[tx][i]);
+      const float x = sX[0][i][tx] + sT[tx][i];
+      if constexpr (SPIN)
+        v[k] = fmaf(shift, spin_square_sym(link, masks, nstr, npair, nsig, cb, packed, ia, ib), x);
+      else
+        v[k] = fmaf(shift * (float)nsig, cb[at], x);
       if (!packed || ia <= ib) ob[at] = v[k];
     }
   }
@@ -952,7 +967,8 @@ void sigma_nm1_prepare(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, double shift)
   if (bp.nmop.n != need) {
     bp.nmop.reset(&ctx->pool, need);
     k_nm1_operand<<<dim3(std::max(1, std::min(16, 2432 / bp.B)), bp.B), 256, 0, st>>>(
-        bp.gp.ptr, n, bp.npair, (n + 1) & ~1, L.cq, L.ck, L.KP, L.NP, shift, bp.nmop.ptr);
+        bp.gp.ptr, n, bp.npair, (n + 1) & ~1, L.cq, L.ck, L.KP, L.NP,
+        nm_spin_in_operand(shift) ? shift : 0.0, bp.nmop.ptr);
     CU_LAUNCH_CHECK();
   }
   const size_t sf = (size_t)bp.B * sigma_nm1_slot_floats(n, nsig, nstr);
@@ -986,9 +1002,10 @@ void sigma_nm1_finish(mbe_ctx* ctx, const BinProblem& bp, const SigmaWork& w, in
                       const float* c, int64_t c_stride, double shift, const int32_t* active,
                       float* out, int64_t out_stride, bool packed) {
   const int ntl = (bp.nstr + 31) / 32;
-  k_sigma_nm1_finish<<<dim3((unsigned)(ntl * (ntl + 1) / 2), bp.B), 256, 0, ctx->stream>>>(
+  auto kernel = nm_spin_in_operand(shift) ? k_sigma_nm1_finish<false> : k_sigma_nm1_finish<true>;
+  kernel<<<dim3((unsigned)(ntl * (ntl + 1) / 2), bp.B), 256, 0, ctx->stream>>>(
       w.Xf.ptr, w_stride, w.slots.ptr, sigma_nm1_slot_floats(bp.n, bp.nsig, bp.nstr),
-      nm_ld(bp.nstr), bp.tab->srow.ptr, bp.nstr, bp.nsig, c, c_stride,
-      (float)(shift * bp.nsig), active, out, out_stride, packed ? 1 : 0);
+      nm_ld(bp.nstr), bp.tab->srow.ptr, bp.tab->link.ptr, bp.tab->masks.ptr, bp.npair, bp.nstr,
+      bp.nsig, c, c_stride, (float)shift, active, out, out_stride, packed ? 1 : 0);
   CU_LAUNCH_CHECK();
 }

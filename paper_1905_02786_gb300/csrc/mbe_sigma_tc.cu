@@ -923,34 +923,8 @@ __global__ void k_sigma_tc_finish(const float* __restrict__ X, int64_t x_stride,
   for (int k = 0, i = ty; i < 32; i += ny, k++) {
     const int ia = I * 32 + i, ib = J * 32 + tx;    // element (ia, ib) and its transpose
     float s = sX[0][i][tx] + sX[1][tx][i];
-    if (shift != 0.f && ia < nstr && ib < nstr) {
-      // evaluated for (min, max): on the diagonal tile both elements of a
-      // pair get bitwise the same value
-      const int lo = min(ia, ib), hi = max(ia, ib);
-      const int32_t* la = link + (int64_t)lo * npair;
-      const int32_t* lb = link + (int64_t)hi * npair;
-      const uint32_t ma = masks[lo], mb = masks[hi];
-      float s2 = (float)(nsig - __popc(ma & mb)) *
-                 cb[packed ? sym_index(lo, hi, nstr) : (int64_t)lo * nstr + hi];
-      // pairs {p, q}: q open in the alpha string, p open in the beta string
-      uint32_t oa = ma & ~mb;
-      const uint32_t obm = mb & ~ma;
-      while (oa) {
-        const int q = __ffs(oa) - 1;
-        oa &= oa - 1;
-        uint32_t ob2 = obm;
-        while (ob2) {
-          const int p = __ffs(ob2) - 1;
-          ob2 &= ob2 - 1;
-          const int P = p > q ? p * (p + 1) / 2 + q : q * (q + 1) / 2 + p;
-          const int32_t ta = la[P], tb = lb[P];
-          const float x = cb[packed ? sym_index(ta >> 1, tb >> 1, nstr)
-                                    : (int64_t)(ta >> 1) * nstr + (tb >> 1)];
-          s2 -= ((ta ^ tb) & 1) ? -x : x;
-        }
-      }
-      s += shift * s2;
-    }
+    if (shift != 0.f && ia < nstr && ib < nstr)
+      s += shift * spin_square_sym(link, masks, nstr, npair, nsig, cb, packed, ia, ib);
     v[k] = s;
     if (ia < nstr && ib < nstr) {
       if (!packed)
