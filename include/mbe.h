@@ -341,7 +341,8 @@ int mbe_sigma(mbe_ctx* ctx, const int* act, int nact, const double* c,
  *  c_dev       nstr*nstr doubles, DEVICE memory of the context's device,
  *              caller-owned, read only
  *  sigma_dev   nstr*nstr doubles, DEVICE memory, caller-owned, fully
- *              overwritten (need not be zeroed)
+ *              overwritten (need not be zeroed); it may be c_dev or overlap it
+ *              (c is then copied into the scratch first)
  *  ndet        element count of c_dev and sigma_dev; MBE_EINVAL unless it
  *              equals nstr*nstr of the active space
  *  e_core      host; if non-NULL the inactive-core energy is written there

@@ -53,7 +53,7 @@ unsigned char* scratch_base(int device) {
 
 // byte offsets of the pieces inside the scratch array (256-byte aligned)
 struct NoallocLayout {
-  size_t masks, ecore, heff, hp, gp, jk, hidx, olnk, hv, wt, total;
+  size_t masks, ecore, heff, hp, gp, jk, hidx, olnk, hv, wt, c, total;
   size_t limit;   // what MBE_NOALLOC_SCRATCH_BYTES is compared with
 };
 
@@ -78,6 +78,7 @@ NoallocLayout noalloc_layout(int n, int nsig, int64_t nstr) {
   L.olnk = take(sizeof(uint32_t) * nsig * (n - nsig) * nstr);
   L.hv = take(sizeof(double) * nnz * nstr);
   L.wt = take(sizeof(double) * npair * nstr);
+  L.c = take(sizeof(double) * ndet);   // of c, where sigma overwrites it
   L.total = o;
   o = common;
   take(sizeof(int32_t) * n);
@@ -126,6 +127,13 @@ int noalloc_sigma_run(mbe_ctx* ctx, const int* act, int nact, const double* c_de
   launch_direct_tables(ctx, nact, nsig, (int)nstr, masks, hidx, olnk);
   launch_direct_values(ctx, nact, nsig, (int)nstr, masks, 1, gp, hv, wt);
   const int64_t ndet = nstr * nstr;
+  // the sigma kernel's CTAs read rows of c that others would overwrite
+  const uintptr_t c0 = (uintptr_t)c_dev, s0 = (uintptr_t)sigma_dev;
+  if (c0 < s0 + sizeof(double) * ndet && s0 < c0 + sizeof(double) * ndet) {
+    CU_CHECK(cudaMemcpyAsync(base + L.c, c_dev, sizeof(double) * ndet, cudaMemcpyDeviceToDevice,
+                             ctx->stream));
+    c_dev = (const double*)(base + L.c);
+  }
   const DirectSide side = {nsig, (int)nstr, masks, olnk, hidx, hv};
   sigma_direct_raw(ctx, nact, side, side, wt, gp, c_dev, ndet, sigma_dev, ndet, nullptr, nullptr, 1,
                    ctx->opt.spin_shift, false);
