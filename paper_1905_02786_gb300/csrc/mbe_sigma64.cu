@@ -440,6 +440,16 @@ void launch_direct_values(mbe_ctx* ctx, int n, int nsig, int nstr, const uint32_
   CU_LAUNCH_CHECK();
 }
 
+// the kernel's shared memory, once per device (before a capture: an attribute
+// loads the kernel)
+static void sigma_direct_attributes(int device) {
+  static bool attr_done[MBE_MAX_DEVICES] = {false};
+  once_per_device(attr_done, device, [] {
+    CU_CHECK(cudaFuncSetAttribute(k_sigma_direct, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)DIR_SMEM));
+  });
+}
+
 void sigma_direct_raw(mbe_ctx* ctx, int n, const DirectSide& al, const DirectSide& be,
                       const double* wt, const double* gp, const double* c, int64_t c_stride,
                       double* out, int64_t out_stride, const int32_t* active,
@@ -474,11 +484,7 @@ void sigma_direct_raw(mbe_ctx* ctx, int n, const DirectSide& al, const DirectSid
   A.msms = 0.25 * (al.nsig - be.nsig) * (al.nsig - be.nsig + 2);   // Ms(Ms+1)
   const DirPlan L = direct_plan(A.npair, al.nsig * (n - al.nsig), A.nnz, be.nstr);
   if (L.total > DIR_SMEM) throw MbeError{MBE_EINVAL, "active space too large for the FP64 sigma"};
-  static bool attr_done[MBE_MAX_DEVICES] = {false};
-  once_per_device(attr_done, ctx->device, [] {
-    CU_CHECK(cudaFuncSetAttribute(k_sigma_direct, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)DIR_SMEM));
-  });
+  sigma_direct_attributes(ctx->device);
   cudaEvent_t ev;
   ctx->fp64_timer.begin(ctx->stream, ctx->opt.timing != 0, &ev);
   k_sigma_direct<<<dim3((unsigned)al.nstr, (unsigned)nb), L.threads, L.total, ctx->stream>>>(A, L);
@@ -495,6 +501,7 @@ bool sigma_direct_supported(int n, int nsig, int nstr) {
 
 // the shape's tables (once) and the batch's values (once per batch)
 void sigma_direct_prepare(mbe_ctx* ctx, BinProblem& bp) {
+  sigma_direct_attributes(ctx->device);
   const int n = bp.n;
   auto tables = [&](const StringTables* ct) {
     StringTables* t = const_cast<StringTables*>(ct);
