@@ -142,15 +142,18 @@ typedef struct mbe_options {
                               operand plan of the two-spin tensor-core kernel
                               that fits on its own data and keeps the fastest
                               for the shape: stages 2..4 of the operand ring
-                              and, outside 5 to 12 orbitals, pull lists in
-                              shared or global memory, one or two epilogue
+                              and, in the kernel over the rows of c, pull lists
+                              in shared or global memory, one or two epilogue
                               groups; 0 (default): the most stages that fit,
                               lists in shared memory when they fit.  All plans
-                              give the same bits.                            */
+                              of a kernel give the same bits.                */
   const char* tune_file;   /* autotune cache (may be NULL): read at
                               mbe_create, one line per tuned shape appended
                               as it is tuned ("sigma_ab n nsig nstages
-                              pull_smem groups ms"); the string is copied    */
+                              pull_smem groups ms", nsig negated for the
+                              kernel over (N-1)-electron strings, which larger
+                              batches of a shape can take); the string is
+                              copied                                         */
   int graphs;              /* FP64 and mixed modes: 1 (default) issues each Davidson
                               iteration (sigma vector, subspace update, Ritz
                               step, residual, correction and its

@@ -369,6 +369,7 @@ int mbe_create(mbe_ctx** out, int device, const mbe_options* opt) {
   if (o.tune_file) {
     c->tune_file = o.tune_file;
     // cached plans: "sigma_ab n nsig nstages pull_smem groups ms" per line
+    // (nsig < 0: of the kernel over (N-1)-electron strings)
     std::ifstream in(c->tune_file);
     std::string line;
     while (std::getline(in, line)) {

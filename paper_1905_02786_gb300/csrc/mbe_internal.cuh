@@ -418,7 +418,8 @@ struct mbe_ctx {
   KeptRdm ref_ci;
   std::vector<RdmBlock> rdm_blocks;
   // autotuned operand plans of the two-spin tensor-core sigma:
-  // (n, nsig) -> {A stages, pull lists in shared memory, epilogue groups};
+  // (n, nsig) -> {A stages, pull lists in shared memory, epilogue groups}; of
+  // the kernel over (N-1)-electron strings (n, -nsig) -> {A stages, 0, 1};
   // tune_file is the cache (empty: none)
   std::map<std::pair<int, int>, std::array<int, 3>> tune_ab;
   std::string tune_file;

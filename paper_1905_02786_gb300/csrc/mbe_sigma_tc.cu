@@ -1098,16 +1098,6 @@ void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, float* c, int64_t c_st
   AbPlan p;
   if (!ab_plan(bp.n, bp.nsig, nstr, p))
     throw MbeError{MBE_EINVAL, "active space too large for the tensor-core sigma"};
-  // autotuned plan of this shape, if one is known
-  bool tune_now = false;
-  if (ctx->opt.autotune && p.nlink > 0) {
-    auto it = ctx->tune_ab.find({bp.n, bp.nsig});
-    AbPlan q;
-    if (it == ctx->tune_ab.end())
-      tune_now = true;
-    else if (ab_plan_with(bp.n, bp.nsig, nstr, it->second[0], it->second[1], it->second[2], q))
-      p = q;
-  }
   const int64_t N = bp.ndet;
   const int64_t hs = 2 * (int64_t)nstr * p.ldc;      // bf16 elements per tuple (hi + lo)
   const int ntiles = (nstr + AB_M - 1) / AB_M;
@@ -1120,11 +1110,21 @@ void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, float* c, int64_t c_st
              sigma_nm1_used(ctx->device, bp.n, bp.nsig, nstr,
                             packed ? B : std::max(B, std::min(ctx->opt.max_batch, 256)));
   const bool nm1 = bp.nm1 == 1;
+  if (nm1) sigma_nm1_prepare(ctx, bp, w, spin_shift);
+  // autotuned plan of this shape, if one is known (of each kernel its own: the
+  // batch decides which of them a shape takes)
+  const std::pair<int, int> tune_key = {bp.n, nm1 ? -bp.nsig : bp.nsig};
   int nm_stages = 0;
-  if (nm1) {
-    sigma_nm1_prepare(ctx, bp, w, spin_shift);
-    auto it = ctx->tune_ab.find({bp.n, bp.nsig});
-    if (ctx->opt.autotune && it != ctx->tune_ab.end()) nm_stages = it->second[0];
+  bool tune_now = false;
+  if (ctx->opt.autotune && p.nlink > 0) {
+    auto it = ctx->tune_ab.find(tune_key);
+    AbPlan q;
+    if (it == ctx->tune_ab.end())
+      tune_now = true;
+    else if (nm1)
+      nm_stages = it->second[0];
+    else if (ab_plan_with(bp.n, bp.nsig, nstr, it->second[0], it->second[1], it->second[2], q))
+      p = q;
   }
   // per bin shape: compacted links and the pull lists of the scatter
   if (!nm1 && tab->nlink != p.nlink) {
@@ -1214,10 +1214,10 @@ void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, float* c, int64_t c_st
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    ctx->tune_ab[{bp.n, bp.nsig}] = {nm_stages, 0, 1};
+    ctx->tune_ab[tune_key] = {nm_stages, 0, 1};
     if (!ctx->tune_file.empty()) {
       std::ofstream out(ctx->tune_file, std::ios::app);
-      out << "sigma_ab " << bp.n << " " << bp.nsig << " " << nm_stages << " 0 1 " << best << "\n";
+      out << "sigma_ab " << bp.n << " " << -bp.nsig << " " << nm_stages << " 0 1 " << best << "\n";
     }
   } else if (tune_now) {
     // every plan that fits, timed on this call's data (H^a c rewritten
