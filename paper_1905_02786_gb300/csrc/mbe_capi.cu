@@ -202,13 +202,14 @@ void solve_jobs(mbe_ctx* ctx, const std::vector<std::vector<int>>& acts, double*
     const bool mixed_bin = ctx->opt.precision == MBE_MIXED_BF16X3 && N > 1 && closed &&
                            sigma_tc_supported(n, tab->nstr) && ozaki_supported(tab->npair);
     const int Mm = mixed_subspace_alloc(ctx->opt.max_subspace);
-    // and, where its two-spin kernel takes the shape, the row sums and the
-    // packed words of the operand
-    const int most = (int)std::min<int64_t>(ctx->opt.max_batch, (int64_t)kv.second.size());
+    // and, where the two-spin kernel over (N-1)-electron strings takes the
+    // shape, the row sums and the packed words of the operand
+    const int most = (int)std::min<int64_t>({(int64_t)std::max(1, ctx->opt.max_batch),
+                                             (int64_t)kv.second.size(), SIGMA_NM1_MAX_BATCH});
+    const bool nm1_bin = mixed_bin && sigma_nm1_used(ctx->device, n, nsig, tab->nstr, most);
     const double nm1 =
-        mixed_bin && sigma_nm1_used(ctx->device, n, nsig, tab->nstr, std::max(1, most))
-            ? 4.0 * ((double)sigma_nm1_slot_floats(n, nsig, tab->nstr) +
-                     (double)tab->nstr * sigma_nm1_ldw(tab->nstr)) : 0.0;
+        nm1_bin ? 4.0 * ((double)sigma_nm1_slot_floats(n, nsig, tab->nstr) +
+                         (double)tab->nstr * sigma_nm1_ldw(tab->nstr)) : 0.0;
     double per = (mixed_bin ? (double)(4 * Mm + 46) * N + nm1 + 128.0 * 128.0 * 4.0
                             : (double)(2 * M + 6) * N * 8.0 +
                                   8.0 * (direct_nnz(n, nsig) * (double)tab->nstr +
@@ -217,6 +218,7 @@ void solve_jobs(mbe_ctx* ctx, const std::vector<std::vector<int>>& acts, double*
                  (double)tab->npair * tab->npair * 8.0 * 2.0;
     int64_t bmem = std::max<int64_t>(1, (int64_t)(budget / per));
     int64_t bmax = std::min<int64_t>(std::max(1, ctx->opt.max_batch), bmem);
+    if (nm1_bin) bmax = std::min<int64_t>(bmax, SIGMA_NM1_MAX_BATCH);
     const std::vector<int64_t>& idx = kv.second;
     for (size_t c0 = 0; c0 < idx.size(); c0 += bmax) {
       const int B = (int)std::min<int64_t>(bmax, (int64_t)idx.size() - (int64_t)c0);

@@ -563,6 +563,7 @@ void sigma_tc(mbe_ctx* ctx, BinProblem& bp, SigmaWork& w, float* c, int64_t c_st
 int32_t sigma_tc_error(mbe_ctx* ctx, SigmaWork& w);
 // two-spin part over pairs of (N-1)-electron strings (mbe_sigma_nm1.cu): the
 // shapes it takes, the floats of row sums per tuple, its TMEM operand stages
+constexpr int SIGMA_NM1_MAX_BATCH = 4096;   // its list of tuples in shared memory
 bool sigma_nm1_supported(int n, int nsig, int nstr, int B);
 int sigma_nm1_tiles(int n, int nsig, int nstr, int B);   // of one tuple (0: not supported)
 // the kernel of the two-spin part for B tuples of a shape (mbe_sigma_tc.cu):

@@ -73,7 +73,6 @@ constexpr int NM_EH = NM_EPI / 128;                 // its warps per TMEM quadra
 constexpr uint32_t NM_HINT_NS = 1000, NM_SLEEP = 64;
 constexpr uint32_t NM_SMEM_MAX = 222 * 1024;
 constexpr uint32_t NM_SMEM_MIN = 116 * 1024;   // one CTA per SM (512 TMEM columns)
-constexpr int NM_B_MAX = 4096;
 
 template <int N>
 struct Shape {
@@ -891,7 +890,7 @@ bool nm_plan_n(int nsig, int nstr, int B, NmPlan& L) {
 }
 
 bool nm_plan(int n, int nsig, int nstr, int B, NmPlan& L) {
-  if (nsig < 1 || nsig > n || B > NM_B_MAX) return false;
+  if (nsig < 1 || nsig > n || B > SIGMA_NM1_MAX_BATCH) return false;
   switch (n) {
 #define NM_CASE(N) case N: return nm_plan_n<N>(nsig, nstr, B, L);
     NM_CASE(5) NM_CASE(6) NM_CASE(7) NM_CASE(8) NM_CASE(9) NM_CASE(10) NM_CASE(11) NM_CASE(12)

@@ -45,3 +45,23 @@ def test_energies_vs_fp64(lib, norb, n, nsig, count):
         eps.append(np.array(e))
         m.close()
     assert np.abs(eps[1] - eps[0]).max() < 1e-8
+
+
+def test_bin_beyond_one_batch(lib):
+    """4,845 tuples of 4e/6o with max_batch above that: the (N-1)-electron kernel
+    takes 4,096 at a time, so the bin is solved as the two parts are, bit for bit."""
+    norb, nsig, n = 22, 2, 6
+    h, eri, _ = ms.gen_integrals(norb, nsig, 47)
+    tk = np.array(list(itertools.combinations(range(2, norb), n - nsig)), dtype=np.int32)
+    assert len(tk) == 4845
+
+    def solve(part):
+        m = lib.MBE(0, precision=lib.MBE_MIXED_BF16X3, max_batch=8192)
+        m.load(h, eri, 2 * nsig)
+        lib.mbe_set_reference(m.ctx, [0, 1], list(range(2, norb)))
+        e, st = lib.mbe_solve_tuples(m.ctx, part, n - nsig)
+        m.close()
+        assert np.all(st == 0)
+        return e
+
+    assert np.array_equal(solve(tk), np.concatenate([solve(tk[:4096]), solve(tk[4096:])]))
