@@ -92,7 +92,13 @@ typedef struct mbe_options {
                            of every converged CASCI for the energy backward
                            (formed from the vector right after its batch
                            converges; the vector itself is not kept)       */
-  int deterministic;    /* 1: fixed-order reductions only (no float atomics) */
+  int deterministic;    /* 1: fixed-order reductions only (no float atomics): a
+                           call repeated on the same GPU model gives the same
+                           bits.  The order, and in the mixed mode the kernel,
+                           follow from the tuples solved together and those
+                           still iterating: in another batch (max_batch, tuple
+                           list, GPU count) a tuple's energy agrees to its
+                           convergence target, not bit for bit               */
   int64_t mem_cap_bytes;/* cap on device memory the context may allocate; 0 =
                            no cap (exceeding it returns MBE_ENOMEM)          */
   int timing;           /* 1: time the sigma contraction launches with CUDA

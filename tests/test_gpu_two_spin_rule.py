@@ -65,3 +65,27 @@ def test_bin_beyond_one_batch(lib):
         return e
 
     assert np.array_equal(solve(tk), np.concatenate([solve(tk[:4096]), solve(tk[4096:])]))
+
+
+@pytest.mark.parametrize("n,nsig", [(10, 4), (9, 6)])
+def test_batch_and_alone(lib, n, nsig):
+    """A tuple in a batch and alone: repeated calls give the same bits, other
+    batches the same energy to the convergence target (1e-8 Eh)."""
+    norb = n + 2
+    h, eri, _ = ms.gen_integrals(norb, nsig, 67)
+    ref = list(range(nsig))
+    tk = np.array(list(itertools.islice(itertools.combinations(range(nsig, norb), n - nsig), 24)),
+                  dtype=np.int32)
+
+    def solve(max_batch):
+        m = lib.MBE(0, precision=lib.MBE_MIXED_BF16X3, max_batch=max_batch)
+        m.load(h, eri, 2 * nsig)
+        lib.mbe_set_reference(m.ctx, ref, list(range(nsig, norb)))
+        e, st = lib.mbe_solve_tuples(m.ctx, tk, n - nsig)
+        m.close()
+        assert np.all(st == 0)
+        return e
+
+    for b in (1, 5, 24):
+        assert np.array_equal(solve(b), solve(b))
+        assert np.abs(solve(b) - solve(24)).max() < 1e-8
