@@ -475,23 +475,26 @@ def main():
         peak_tf = fp_peaks["fp64_tflops"]
         peak_src = "FP64 FMA, measured by mbe_measure_peaks on this GPU"
         bound = "alu"
-        ksrc = "paper_1905_02786_gb300/csrc/mbe_sigma64.cu"
     else:
         # the sigma contraction: k_gemm_haa (one-spin part) + k_sigma_nm1
-        # (two-spin part; k_sigma_ab outside 5 to 12 orbitals), timed together with CUDA events on the library's
-        # stream; algorithmic flops 2 N_det npair^2 per sigma vector
+        # (two-spin part; k_sigma_ab where that is the faster one), timed
+        # together with CUDA events on the library's stream; flops of the dense
+        # pair form, 2 N_det npair^2 per sigma vector, several times what the
+        # kernels multiply
         kname = "k_gemm_haa+k_sigma_nm1"
         peak_tf = pk.get("bf16_tflops_sustained", 1700.0)
         peak_src = f"bf16 dense sustained, {pk_kind}"
         bound = "tensor"
-        ksrc = "paper_1905_02786_gb300/csrc/mbe_sigma_tc.cu"
+    ksources = {"k_gemm_haa": "paper_1905_02786_gb300/csrc/mbe_sigma_tc.cu",
+                "k_sigma_nm1": "paper_1905_02786_gb300/csrc/mbe_sigma_nm1.cu",
+                "k_sigma_direct": "paper_1905_02786_gb300/csrc/mbe_sigma64.cu"}
     # DRAM bytes per algorithmic flop from one ncu capture of the kernels
     # (8e/12o batch of 64 tuples, bench --profile-batch 64), scaled to this
     # run's average launch; null once a kernel source has changed
     traffic = 0.0
     for kn in kname.split("+"):
         tr = TRAFFIC.get(kn)
-        if not tr or tr["sha"] != src_sha(ksrc, kn):
+        if not tr or tr["sha"] != src_sha(ksources[kn], kn):
             traffic = None
             break
         traffic += tr["bytes_per_flop"] * dom_flops_per
@@ -589,7 +592,7 @@ def main():
                     "tensor_core_ms": st["dom_ms"], "fp64_ms": st["fp64_ms"],
                     "tensor_core_vectors_per_casci": st["dom_flops"] / max(st["sigma_flops"], 1)
                     * st["sigma_vectors"] / max(st["casci"], 1),
-                    "fp64_vectors_per_casci": st["fp64_flops"] / max(st["sigma_flops"], 1)
+                    "fp64_vectors_per_casci": (1.0 - st["dom_flops"] / max(st["sigma_flops"], 1))
                     * st["sigma_vectors"] / max(st["casci"], 1)},
                 "davidson_iters_mean": st["iters_total"] / max(st["casci"], 1),
                 "seconds_per_order": list(order_s),

@@ -187,9 +187,11 @@ typedef struct mbe_stats {
                              context stream); 0 unless opt.timing = 1         */
   double dom_flops;       /* their algorithmic flops, 2 N_det npair^2 per
                              sigma vector                                     */
-  int64_t fp64_launches;  /* launches of the FP64 (kl|ij) contraction kernel  */
+  int64_t fp64_launches;  /* launches of the FP64(-grade) sigma kernels       */
   double fp64_ms;         /* their summed device time (opt.timing = 1)        */
-  double fp64_flops;      /* their algorithmic flops                          */
+  double fp64_flops;      /* their flops: what the FP64 kernel multiplies over
+                             the string links (times two), 2 N_det npair^2 per
+                             vector for the sliced tensor-core contractions   */
   int64_t host_launches;  /* launch calls the host made: kernel launches
                              outside graphs plus graph launches               */
   int64_t graph_launches; /* CUDA graph launches (opt.graphs)                 */

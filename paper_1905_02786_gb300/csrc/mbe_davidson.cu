@@ -349,5 +349,8 @@ void davidson_batch(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int32_t* s
   ctx->stats.casci += B;
   ctx->stats.sigma_vectors += vecs;
   ctx->stats.sigma_flops += (double)vecs * per;
-  ctx->stats.fp64_flops += (double)vecs * per;   // exact sigma vectors
+  // exact sigma vectors, by what their route multiplies
+  ctx->stats.fp64_flops +=
+      (double)vecs *
+      (emulated ? per : direct_flops(bp.n, bp.nsig, bp.nsigb, bp.nstr, bp.nstrb, closed));
 }

@@ -565,8 +565,9 @@ void davidson_batch_mixed(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int3
   // E, which stays where a row of c is too long for the FP64 kernel)
   const bool exact_fused = sigma_exact_supported(bp.npair, bp.nstr);
   const bool exact_direct = !exact_fused && sigma_direct_supported(bp.n, bp.nsig, bp.nstr);
-  // exact point of the tuples in `mask`: V0 = x/|x|, exact A V0, theta_x,
-  // r_x and its norm; G = [[V0.AV0]]
+  // exact point of the tuples in `mask` (n_exact of them): V0 = x/|x|, exact A
+  // V0, theta_x, r_x and its norm; G = [[V0.AV0]]
+  int n_exact = B;
   auto exact_point = [&]() {
     k32_copy_i<<<1, 256, 0, st>>>(mask.ptr, active.ptr, B);
     CU_LAUNCH_CHECK();
@@ -583,7 +584,7 @@ void davidson_batch_mixed(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int3
     } else {
       sigma_emulated(ctx, bp, sw, C64.ptr, Lf, S64.ptr, Lf, active.ptr, shift, true);
     }
-    vecs_ex += B;
+    vecs_ex += n_exact;
     k_dot64<<<gcf, RT, 0, st>>>(C64.ptr, S64.ptr, Lf, ch, nchunks_f, active.ptr, rpart.ptr,
                                 cnt.ptr, xax.ptr);
     CU_LAUNCH_CHECK();
@@ -616,7 +617,7 @@ void davidson_batch_mixed(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int3
       gr.run(16, point);
     else
       point();
-    const int na = count_active();
+    const int na = n_exact = count_active();
     if (ctx->opt.verbose) {
       double t0 = 0.0, r0 = 0.0;
       CU_CHECK(cudaMemcpy(&t0, thx.ptr, sizeof(double), cudaMemcpyDeviceToHost));
@@ -676,5 +677,7 @@ void davidson_batch_mixed(mbe_ctx* ctx, BinProblem& bp, double* e_out_host, int3
   ctx->stats.sigma_vectors += vecs_tc + vecs_ex;
   ctx->stats.sigma_flops += (double)(vecs_tc + vecs_ex) * per;
   ctx->stats.dom_flops += (double)vecs_tc * per;
-  ctx->stats.fp64_flops += (double)vecs_ex * per;
+  ctx->stats.fp64_flops +=
+      (double)vecs_ex *
+      (exact_direct ? direct_flops(bp.n, bp.nsig, bp.nsigb, bp.nstr, bp.nstrb, true) : per);
 }

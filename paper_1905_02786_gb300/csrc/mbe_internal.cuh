@@ -514,6 +514,7 @@ struct DirectSide {
   const double* hv;        // their one-spin elements, per tuple
 };
 int direct_nnz(int n, int nsig);   // replacements of one string, itself included
+double direct_flops(int n, int nsig, int nsigb, int64_t nstr, int64_t nstrb, bool symmetric);
 // (masks is written too: the ascending strings)
 void launch_direct_tables(mbe_ctx* ctx, int n, int nsig, int nstr, uint32_t* masks,
                           uint16_t* hidx, uint32_t* olnk);

@@ -417,6 +417,15 @@ int direct_nnz(int n, int nsig) {
   return 1 + nsig * nv + nsig * (nsig - 1) / 2 * (nv * (nv - 1) / 2);
 }
 
+// flops of one sigma vector: two per element that the kernel multiplies (link
+// pairs, one-spin elements, links with the other spin's diagonal), of the upper
+// triangle where c = c^T
+double direct_flops(int n, int nsig, int nsigb, int64_t nstr, int64_t nstrb, bool symmetric) {
+  const double na = (double)nsig * (n - nsig), nb = (double)nsigb * (n - nsigb);
+  const double rows = symmetric ? 0.5 * nstr * (nstr + 1) : (double)nstr * nstrb;
+  return 2.0 * rows * (na * nb + na + nb + direct_nnz(n, nsig) + direct_nnz(n, nsigb) + 1);
+}
+
 void launch_direct_tables(mbe_ctx* ctx, int n, int nsig, int nstr, uint32_t* masks,
                           uint16_t* hidx, uint32_t* olnk) {
   Binom bn;   // C(15, 7) = 6435 at most
