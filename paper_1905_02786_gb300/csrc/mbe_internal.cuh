@@ -523,8 +523,8 @@ void launch_direct_values(mbe_ctx* ctx, int n, int nsig, int nstr, const uint32_
                           const double* gp, double* hv, double* wt);
 void sigma_direct_raw(mbe_ctx* ctx, int n, const DirectSide& al, const DirectSide& be,
                       const double* wt, const double* gp, const double* c, int64_t c_stride,
-                      double* out, int64_t out_stride, const int32_t* active,
-                      const int32_t* bmap, int nb, double spin_shift, int symmetric);   // 2: full
+                      double* out, int64_t out_stride, const int32_t* active, int nb,
+                      double spin_shift, int symmetric);   // 2: full
 StringTables* get_tables(mbe_ctx* ctx, int n, int nsig);
 // active electrons of each spin: alpha (orbitals below nocc_a), beta (below nocc)
 int count_sig(const mbe_ctx* ctx, const std::vector<int>& act);

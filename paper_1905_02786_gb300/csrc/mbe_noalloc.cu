@@ -135,7 +135,7 @@ int noalloc_sigma_run(mbe_ctx* ctx, const int* act, int nact, const double* c_de
     c_dev = (const double*)(base + L.c);
   }
   const DirectSide side = {nsig, (int)nstr, masks, olnk, hidx, hv};
-  sigma_direct_raw(ctx, nact, side, side, wt, gp, c_dev, ndet, sigma_dev, ndet, nullptr, nullptr, 1,
+  sigma_direct_raw(ctx, nact, side, side, wt, gp, c_dev, ndet, sigma_dev, ndet, nullptr, 1,
                    ctx->opt.spin_shift, false);
   if (e_core) {
     CU_CHECK(cudaMemcpyAsync(e_core, ecore, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));

@@ -260,14 +260,13 @@ struct DirArgs {
   int64_t c_stride;
   double* out;
   int64_t out_stride;
-  const int32_t *active, *bmap;
+  const int32_t* active;
   double shift, msms;
 };
 
 __global__ void __launch_bounds__(512)
 k_sigma_direct(const DirArgs A, const DirPlan L) {
-  const int bl = blockIdx.y;
-  const int b = A.bmap ? A.bmap[bl] : bl;
+  const int b = blockIdx.y;
   if (A.active && !A.active[b]) return;
   extern __shared__ __align__(16) unsigned char smem[];
   double* sG = reinterpret_cast<double*>(smem + L.g);
@@ -462,7 +461,7 @@ static void sigma_direct_attributes(int device) {
 void sigma_direct_raw(mbe_ctx* ctx, int n, const DirectSide& al, const DirectSide& be,
                       const double* wt, const double* gp, const double* c, int64_t c_stride,
                       double* out, int64_t out_stride, const int32_t* active,
-                      const int32_t* bmap, int nb, double spin_shift, int symmetric) {
+                      int nb, double spin_shift, int symmetric) {
   DirArgs A;
   A.n = n;
   A.npair = n * (n + 1) / 2;
@@ -488,7 +487,6 @@ void sigma_direct_raw(mbe_ctx* ctx, int n, const DirectSide& al, const DirectSid
   A.out = out;
   A.out_stride = out_stride;
   A.active = active;
-  A.bmap = bmap;
   A.shift = spin_shift;
   A.msms = 0.25 * (al.nsig - be.nsig) * (al.nsig - be.nsig + 2);   // Ms(Ms+1)
   const DirPlan L = direct_plan(A.npair, al.nsig * (n - al.nsig), A.nnz, be.nstr);
@@ -547,5 +545,5 @@ void sigma_direct(mbe_ctx* ctx, BinProblem& bp, const double* c, int64_t c_strid
   const DirectSide be = {bp.nsigb, bp.nstrb, bp.tabb->masks.ptr, bp.tabb->olnk.ptr,
                          bp.tabb->hidx.ptr, bp.closed() ? bp.hv.ptr : bp.hvb.ptr};
   sigma_direct_raw(ctx, bp.n, al, be, bp.wt.ptr, bp.gp.ptr, c, c_stride, out, out_stride, active,
-                   nullptr, bp.B, spin_shift, !symmetric || !bp.closed() ? 0 : packed ? 1 : 2);
+                   bp.B, spin_shift, !symmetric || !bp.closed() ? 0 : packed ? 1 : 2);
 }

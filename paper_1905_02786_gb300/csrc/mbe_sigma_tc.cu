@@ -954,12 +954,15 @@ constexpr uint32_t AB_SMEM_MAX = 224 * 1024;
 
 // operand plan of k_sigma_ab, the first that fits of: the pull lists in
 // shared memory with 4, then 3 A stages (two epilogue groups before one),
-// the lists in global memory likewise, then 2 stages.  Measured on the
-// order-6 bins of the 8e/23o workload (autotuner, 64 tuples): for 8e/12o the
-// lists in shared memory matter most (one group, 4 stages, lists in shared
-// memory 1.24 ms; two groups only fit with the lists in global memory,
-// 1.28 ms at best); for 6e/12o, where both fit, two groups win (0.25 against
-// 0.32 ms)
+// the lists in global memory likewise, then 2 stages.  Measured (autotuner) on
+// shapes that this kernel takes: 35 of 16e/12o lists in shared memory and 4
+// stages 0.679 ms, 3 stages 0.713, lists in global memory with two groups 0.740 at
+// best; 12 of 6e/13o 0.114, 0.120 and 0.131; where two groups fit beside the
+// lists, 35 of 12e/10o 0.133 against 0.161 with one; where the lists with 3 stages
+// do not fit, 2 of 10e/13o two groups and 3 stages 0.471, one group 0.524 at best, 8
+// of 8e/13o 0.453 and, lists in shared memory with 2 stages, 0.471.  The order picks
+// the fastest of all plans on these, within 2 % on 35 of 14e/11o (0.342 against
+// 0.336) and 14e/12o (0.094 against 0.092)
 inline bool ab_plan(int n, int nsig, int nstr, AbPlan& p) {
   const int npair = n * (n + 1) / 2;
   p.kp = round_up(npair, 16);
