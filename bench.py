@@ -40,9 +40,13 @@ DEFAULT_WORKLOAD = "h2o_dz_8e23o"
 # DRAM traffic per launch of the dominant kernels from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum), per algorithmic flop
 # (2 N_det npair^2 per sigma vector), keyed by kernel; valid only while the
-# kernel definition is unchanged (sha256 prefix of its source text).  No capture
-# of the present kernels over a full batch has been taken: null.
-TRAFFIC = {}
+# kernel definition is unchanged (sha256 prefix of its source text).  From the
+# captures of one launch over 64 active 8e/12o tuples (1.9081e+11 flop),
+# profiles/mixed_sigma_kernels_8e12o_batch16.md.
+TRAFFIC = {"k_gemm_haa": {"bytes_per_flop": (126372352 + 27657984) / 1.9081e11,
+                          "sha": "b2ed8e2372308b82"},
+           "k_sigma_nm1": {"bytes_per_flop": (107952640 + 108917760) / 1.9081e11,
+                           "sha": "af43244c8e7d8111"}}
 
 
 def peaks():
