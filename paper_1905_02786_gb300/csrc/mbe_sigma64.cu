@@ -264,7 +264,10 @@ struct DirArgs {
   double shift, msms;
 };
 
-__global__ void __launch_bounds__(512)
+// (two CTAs of 512 threads per SM, 62 registers: with the 40 registers that the
+// compiler takes for three, 3 x 8e/11o is 449 us against 437 and 14e/14o 109 ms
+// against 96; 45 of 6e/9o and 8e/9o are 129 us against 135)
+__global__ void __launch_bounds__(512, 2)
 k_sigma_direct(const DirArgs A, const DirPlan L) {
   const int b = blockIdx.y;
   if (A.active && !A.active[b]) return;
