@@ -588,7 +588,7 @@ int mbe_solve_tuples(mbe_ctx* ctx, int order, const int32_t* tuples, int64_t ntu
                             ctx->rdm_blocks.end());
     }
     solve_jobs(ctx, acts, eps.data(), st.data(), ctx->opt.keep_ci ? &rdm : nullptr, order);
-    ctx->cur_order = order;
+    ctx->cur_order = 0;   // no solved order until its arrays are on the device
     ctx->cur_tuples.assign(tuples, tuples + ntup * order);
     ctx->cur_eps = eps;
     ctx->cur_tuples_dev.reset(&ctx->pool, (size_t)ntup * order);
@@ -600,6 +600,7 @@ int mbe_solve_tuples(mbe_ctx* ctx, int order, const int32_t* tuples, int64_t ntu
                                cudaMemcpyHostToDevice, ctx->stream));
       CU_CHECK(cudaStreamSynchronize(ctx->stream));
     }
+    ctx->cur_order = order;
     if (ctx->opt.keep_ci) {
       for (int64_t t = 0; t < ntup; t++) {
         KeptRdm k;
@@ -722,11 +723,12 @@ int mbe_set_pruning_pairs(mbe_ctx* ctx, const int32_t* pairs, int npairs) {
       part[b] = a;
     }
     ctx->partner = part;
-    ctx->pruned = npairs > 0;
+    ctx->pruned = false;   // until the pairs are on the device
     ctx->partner_dev.reset(&ctx->pool, std::max(1, ctx->norb));
     CU_CHECK(cudaMemcpyAsync(ctx->partner_dev.ptr, part.data(), sizeof(int32_t) * ctx->norb,
                              cudaMemcpyHostToDevice, ctx->stream));
     CU_CHECK(cudaStreamSynchronize(ctx->stream));
+    ctx->pruned = npairs > 0;
     return MBE_OK;
   });
 }
@@ -836,7 +838,7 @@ int mbe_set_order_energies(mbe_ctx* ctx, int order, const int32_t* tuples, int64
         if (i && row[i] <= row[i - 1]) return fail(ctx, MBE_EINVAL, "tuple rows must be strictly ascending");
       }
     }
-    ctx->cur_order = order;
+    ctx->cur_order = 0;   // no solved order until its arrays are on the device
     ctx->cur_tuples.assign(tuples, tuples + ntup * order);
     ctx->cur_eps.assign(eps, eps + ntup);
     ctx->cur_tuples_dev.reset(&ctx->pool, (size_t)ntup * order);
@@ -848,6 +850,7 @@ int mbe_set_order_energies(mbe_ctx* ctx, int order, const int32_t* tuples, int64
                                cudaMemcpyHostToDevice, ctx->stream));
       CU_CHECK(cudaStreamSynchronize(ctx->stream));
     }
+    ctx->cur_order = order;
     return MBE_OK;
   });
 }

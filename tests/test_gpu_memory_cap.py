@@ -116,3 +116,37 @@ def test_increments_after_failed_growth(lib):
                 seen.add("full")
         m.close()
     assert seen == {"right", "full"}
+
+
+def test_no_order_after_failed_upload(lib):
+    """The 2,016 tuples and energies of order 2 (16 KB each) that do not fit are
+    not taken for a solved order."""
+    norb = 65
+    rng = np.random.default_rng(4)
+    h, eri, _ = ms.gen_integrals(norb, 1, 7)
+    exp = list(range(1, norb))
+    t1 = np.array([[o] for o in exp], dtype=np.int32)
+    t2 = np.array([[a, b] for a in exp for b in exp if a < b], dtype=np.int32)
+    e1, e2 = rng.standard_normal(len(t1)), rng.standard_normal(len(t2))
+    failed = 0
+    for cap in range(eri.nbytes + (64 << 10), eri.nbytes + (512 << 10), 8 << 10):
+        m = lib.MBE(0, mem_cap_bytes=cap)
+        try:
+            m.load(h, eri, 2)
+            lib.mbe_set_reference(m.ctx, [0], exp)
+            lib.mbe_set_order_energies(m.ctx, t1, e1, 1)
+            lib.mbe_increments(m.ctx, 1, 0.0, len(t1))
+        except lib.MBEError as err:
+            assert err.code == lib.MBE_ENOMEM
+            m.close()
+            continue
+        try:
+            lib.mbe_set_order_energies(m.ctx, t2, e2, 2)
+        except lib.MBEError as err:
+            assert err.code == lib.MBE_ENOMEM
+            failed += 1
+            with pytest.raises(lib.MBEError) as ei:
+                lib.mbe_increments(m.ctx, 2, 0.0, len(t2))
+            assert ei.value.code == lib.MBE_ESTATE
+        m.close()
+    assert failed
